@@ -13,6 +13,7 @@
 // m = 0..4, tabulated (complex) per axis at the unknown nodes by the host.
 #include <algorithm>
 #include <cmath>
+#include <cstring>
 
 #include "helm6_internal.h"
 
@@ -37,110 +38,211 @@ using Z = cpx<double>;
 
 __device__ __forceinline__ Z zc(c64d a) { return Z{a.re, a.im}; }
 
-// Complex table entry: term k, axis a, derivative order m, unknown node p.
-__device__ __forceinline__ Z tv(const double* tab, int mmax, int k, int a, int m, int p) {
-  const int64_t o = (((int64_t)k * 3 + a) * 5 + m) * mmax + p;
-  return Z{tab[2 * o], tab[2 * o + 1]};
-}
+// Table values of a separable term: real (Gaussian factors) or complex.
+struct Re {
+  double v;
+};
+__device__ __forceinline__ Re operator*(Re a, Re b) { return Re{a.v * b.v}; }
+__device__ __forceinline__ Re operator+(Re a, Re b) { return Re{a.v + b.v}; }
+__device__ __forceinline__ Z operator*(Z a, Re b) { return Z{a.re * b.v, a.im * b.v}; }
+// a + w x
+__device__ __forceinline__ Z mad(Z w, Re x, Z a) { return Z{fma(w.re, x.v, a.re), fma(w.im, x.v, a.im)}; }
+__device__ __forceinline__ Z mad(Z w, Z x, Z a) { return cfma(w, x, a); }
+template <bool REAL>
+struct TabT {
+  using t = Z;
+  static __device__ __forceinline__ Z ld(const double* p, int64_t o) { return Z{p[2 * o], p[2 * o + 1]}; }
+};
+template <>
+struct TabT<true> {
+  using t = Re;
+  static __device__ __forceinline__ Re ld(const double* p, int64_t o) { return Re{p[o]}; }
+};
 
-// Term-summed derivative f^(ox, oy, oz) at node (i, j, l).
-__device__ __forceinline__ Z deriv(const double* tab, const double* coef, int nterm, int mmax, int i, int j,
-                                   int l, int ox, int oy, int oz) {
-  Z s = Z{0.0, 0.0};
-  for (int k = 0; k < nterm; ++k) {
-    const Z v = tv(tab, mmax, k, 0, ox, i) * tv(tab, mmax, k, 1, oy, j) * tv(tab, mmax, k, 2, oz, l);
-    s = s + Z{coef[2 * k], coef[2 * k + 1]} * v;
+// Nodes [lo, hi) of each axis outside which every derivative of a term's factor is exactly 0
+// (a Gaussian's tails underflow); a term is skipped where its product is an exact zero.
+struct TermRange {
+  int lo[3], hi[3];
+};
+
+constexpr int RHS_WARPS = 4, RHS_ROWS = 16, RHS_TERMS = 32;  // warps and x rows of a block, terms per pass
+
+// A Neumann or Sommerfeld-like face's data term is, per separable term with normal factor
+// derivatives N0..N3 (N in the inward normal: odd ones change sign at the upper face) and
+// tangential factors S, T,   F -= c0 S0 T0 + c2 (S2 T0 + S0 T2)
+// with   Neumann      c0 = dn1 N1 + dn3 N3,  c2 = dnm N1
+//        Sommerfeld   c0 = -e1mu3 2h [a1 b1 + a2 b2 + a3 b3],  c2 = -e1mu3 (mu1h5 - 2h a3) b1,
+//        b1 = ik N0 + N1, b2 = (ik)^2 N0 + 2 ik N1 + N2, b3 = (ik)^3 N0 + 3 (ik)^2 N1 + 3 ik N2 + N3.
+template <bool REAL>
+__device__ __forceinline__ void face_pair(const RhsCoef& c, int kind, int side, const double* tab, int64_t o, int mmax,
+                                          Z& c0, Z& c2) {
+  using TT = TabT<REAL>;
+  const Z one{1.0, 0.0};
+  const Z n0 = one * TT::ld(tab, o), n2 = one * TT::ld(tab, o + 2 * (int64_t)mmax);
+  Z n1 = one * TT::ld(tab, o + mmax), n3 = one * TT::ld(tab, o + 3 * (int64_t)mmax);
+  if (side) {
+    n1 = -1.0 * n1;
+    n3 = -1.0 * n3;
   }
-  return s;
+  if (kind == HELM6_NEUMANN) {
+    c0 = zc(c.dn1) * n1 + c.dn3 * n3;
+    c2 = c.dnm * n1;
+  } else {
+    const Z ik = zc(c.ik), ik2 = ik * ik, ik3 = ik2 * ik;
+    const Z b1 = ik * n0 + n1;
+    const Z b2 = ik2 * n0 + 2.0 * (ik * n1) + n2;
+    const Z b3 = ik3 * n0 + 3.0 * (ik2 * n1) + 3.0 * (ik * n2) + n3;
+    const Z e = -1.0 * zc(c.e1mu3);
+    c0 = e * ((2.0 * c.h) * (zc(c.a1) * b1 + zc(c.a2) * b2 + c.a3 * b3));
+    c2 = e * ((zc(c.mu1h5) - Z{2.0 * c.h * c.a3, 0.0}) * b1);
+  }
 }
 
-__global__ void rhs_kernel(Geom g, RhsCoef c, int nsrc, int mmax, const double* __restrict__ tab,
-                           const double* __restrict__ amps, const double* __restrict__ noise,
-                           double* __restrict__ F) {
-  const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= g.N) return;
-  const int i = (int)(idx % g.mx);
-  const int j = (int)((idx / g.mx) % g.my);
-  const int l = (int)(idx / ((int64_t)g.mx * g.my));
-  Z S0{0, 0}, S1{0, 0}, S2{0, 0}, S3{0, 0};
-  for (int k = 0; k < nsrc; ++k) {
-    Z gx[5], gy[5], gz[5];
-#pragma unroll
-    for (int m = 0; m < 5; ++m) {
-      gx[m] = tv(tab, mmax, k, 0, m, i);
-      gy[m] = tv(tab, mmax, k, 1, m, j);
-      gz[m] = tv(tab, mmax, k, 2, m, l);
+// A block takes RHS_ROWS x rows (j, l).  The compact right side of a separable term is, along a
+// row, a combination of the three even derivatives of its x factor alone,
+//     F(i) = sum_t A_t X_t(i) + B_t X_t^(2)(i) + C_t X_t^(4)(i)  (+ the x faces' terms at the ends),
+// whose coefficients hold the y and z factors, the amplitude and the y and z faces' terms.  The
+// block forms them first, one thread per (row, term) and 32 terms at a time, then a warp walks
+// a row at 3 FMAs per term and component (real factors) instead of the products of every
+// derivative pair.  FP64 arithmetic bounds the kernel, and an FP64 instruction costs the same
+// with one lane as with 32: hence the coefficients of several rows at once.  At 256 x 258 x 258
+// with eight sources and noise the call takes 0.66 ms, a third of it the host's tables; every
+// derivative product at every point took 27.3 ms (the warp forming its own row's coefficients: 0.81).
+template <bool REAL>
+__global__ void __launch_bounds__(32 * RHS_WARPS) rhs_kernel(Geom g, RhsCoef c, int nterm, int mmax,
+                                                             const double* __restrict__ tab,
+                                                             const double* __restrict__ amps,
+                                                             const TermRange* __restrict__ rng,
+                                                             const double* __restrict__ noise, double2* __restrict__ F) {
+  using TT = TabT<REAL>;
+  __shared__ Z sA[RHS_ROWS][RHS_TERMS], sB[RHS_ROWS][RHS_TERMS], sC[RHS_ROWS][RHS_TERMS], sE[RHS_ROWS][2][RHS_TERMS];
+  __shared__ short2 sR[RHS_ROWS][RHS_TERMS];  // the term's nonzero x nodes (empty: skipped on this row)
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int64_t rows = (int64_t)g.my * g.mz, row0 = (int64_t)blockIdx.x * RHS_ROWS;
+  const int nrow = (int)min((int64_t)RHS_ROWS, rows - row0);
+  const double h2 = c.h * c.h, h4 = h2 * h2;
+  const Z h2cf = h2 * zc(c.cf);
+  for (int t0 = 0; t0 == 0 || t0 < nterm; t0 += RHS_TERMS) {
+    const int nt = min(RHS_TERMS, nterm - t0);
+    for (int e = threadIdx.x; e < nrow * nt; e += 32 * RHS_WARPS) {
+      const int r = e / nt, s = e - r * nt, t = t0 + s;
+      const int j = (int)((row0 + r) % g.my), l = (int)((row0 + r) / g.my);
+      const TermRange q = rng[t];
+      const bool on = j >= q.lo[1] && j < q.hi[1] && l >= q.lo[2] && l < q.hi[2];
+      sR[r][s] = on ? make_short2((short)q.lo[0], (short)q.hi[0]) : make_short2(0, 0);
+      if (!on) continue;
+      const Z h2q1 = h2 * zc(c.q1);
+      const double p4 = h2 * (h4 / 360.0), m4 = h2 * (h4 / 90.0);
+      const int64_t ox = (int64_t)t * 15 * mmax, oy = ox + 5 * (int64_t)mmax + j, oz = ox + 10 * (int64_t)mmax + l;
+      const auto y0 = TT::ld(tab, oy), y2 = TT::ld(tab, oy + 2 * (int64_t)mmax), y4 = TT::ld(tab, oy + 4 * (int64_t)mmax);
+      const auto z0 = TT::ld(tab, oz), z2 = TT::ld(tab, oz + 2 * (int64_t)mmax), z4 = TT::ld(tab, oz + 4 * (int64_t)mmax);
+      const Z am{amps[2 * t], amps[2 * t + 1]};
+      const auto yz = y0 * z0, l2 = y2 * z0 + y0 * z2;
+      Z A = (h2cf * yz) + (h2q1 * l2) + (Z{p4, 0.0} * (y4 * z0 + y0 * z4)) + (Z{m4, 0.0} * (y2 * z2));
+      Z B = (h2q1 * yz) + (Z{m4, 0.0} * l2);
+      const Z C = Z{p4, 0.0} * yz;
+      Z c0, c2;
+      for (int side = 0; side < 2; ++side) {
+        if (g.face[2 + side] != HELM6_DIRICHLET && j == (side ? g.my - 1 : 0)) {
+          face_pair<REAL>(c, g.face[2 + side], side, tab, oy, mmax, c0, c2);
+          A = A - (c0 * z0 + c2 * z2);
+          B = B - c2 * z0;
+        }
+        if (g.face[4 + side] != HELM6_DIRICHLET && l == (side ? g.mz - 1 : 0)) {
+          face_pair<REAL>(c, g.face[4 + side], side, tab, oz, mmax, c0, c2);
+          A = A - (c0 * y0 + c2 * y2);
+          B = B - c2 * y0;
+        }
+      }
+      for (int side = 0; side < 2; ++side) {
+        Z x{0.0, 0.0};
+        if (g.face[side] != HELM6_DIRICHLET) {
+          face_pair<REAL>(c, g.face[side], side, tab, ox + (side ? g.mx - 1 : 0), mmax, c0, c2);
+          x = am * (c0 * yz + c2 * l2);
+        }
+        sE[r][side][s] = x;
+      }
+      sA[r][s] = am * A;
+      sB[r][s] = am * B;
+      sC[r][s] = am * C;
     }
-    const Z f0 = gx[0] * gy[0] * gz[0];
-    const Z lap = gx[2] * gy[0] * gz[0] + gx[0] * gy[2] * gz[0] + gx[0] * gy[0] * gz[2];
-    const Z p4 = gx[4] * gy[0] * gz[0] + gx[0] * gy[4] * gz[0] + gx[0] * gy[0] * gz[4];
-    const Z m4 = gx[2] * gy[2] * gz[0] + gx[2] * gy[0] * gz[2] + gx[0] * gy[2] * gz[2];
-    const Z a = Z{amps[2 * k], amps[2 * k + 1]};
-    S0 = S0 + a * f0;
-    S1 = S1 + a * lap;
-    S2 = S2 + a * p4;
-    S3 = S3 + a * m4;
-  }
-  const double h = c.h, h2 = h * h, h4 = h2 * h2;
-  Z Fv = zc(c.cf) * S0 + zc(c.q1) * S1 + (h4 / 360.0) * S2 + (h4 / 90.0) * S3;
-  Fv = h2 * Fv;
-  if (noise) Fv = Fv + h2 * (zc(c.cf) * Z{noise[2 * idx], noise[2 * idx + 1]});
-
-  // face data terms
-  const int pos[3] = {i, j, l};
-  const int dimv[3] = {g.mx, g.my, g.mz};
-  for (int ax = 0; ax < 3; ++ax) {
-    for (int side = 0; side < 2; ++side) {
-      const int kind = g.face[2 * ax + side];
-      if (kind == HELM6_DIRICHLET) continue;
-      if (pos[ax] != (side == 0 ? 0 : dimv[ax] - 1)) continue;
-      const double sg = side == 0 ? 1.0 : -1.0;
-      const int t1 = (ax == 0) ? 1 : 0, t2 = (ax == 2) ? 1 : 2;
-      auto d = [&](int on, int o1, int o2) {
-        int o[3] = {0, 0, 0};
-        o[ax] = on;
-        o[t1] = o1;
-        o[t2] = o2;
-        Z v = deriv(tab, amps, nsrc, mmax, i, j, l, o[0], o[1], o[2]);
-        const double sgn = (on & 1) ? sg : 1.0;
-        return sgn * v;
-      };
-      if (kind == HELM6_NEUMANN) {
-        const Z DN = zc(c.dn1) * d(1, 0, 0) + c.dn3 * d(3, 0, 0) + c.dnm * (d(1, 2, 0) + d(1, 0, 2));
-        Fv = Fv - DN;
-      } else {
-        const Z ik = zc(c.ik), ik2 = ik * ik, ik3 = ik2 * ik;
-        const Z f0 = d(0, 0, 0), fn = d(1, 0, 0), fnn = d(2, 0, 0), fnnn = d(3, 0, 0);
-        const Z ftt = d(0, 2, 0), fss = d(0, 0, 2), fntt = d(1, 2, 0), fnss = d(1, 0, 2);
-        const Z fb_n = ik * f0 + fn;
-        const Z fb_nn = ik2 * f0 + 2.0 * (ik * fn) + fnn;
-        const Z fb_nnn = ik3 * f0 + 3.0 * (ik2 * fn) + 3.0 * (ik * fnn) + fnnn;
-        const Z fb_ntt = ik * ftt + fntt;
-        const Z fb_nss = ik * fss + fnss;
-        const Z Fbar = zc(c.a1) * fb_n + zc(c.a2) * fb_nn + c.a3 * (fb_nnn - fb_ntt - fb_nss);
-        const Z DS = Z{0.0, 0.0} - zc(c.e1mu3) * ((2.0 * h) * Fbar + zc(c.mu1h5) * (fb_ntt + fb_nss));
-        Fv = Fv - DS;
+    __syncthreads();
+    for (int r = w; r < nrow; r += RHS_WARPS) {
+      for (int i = lane; i < g.mx; i += 32) {
+        const int64_t idx = (row0 + r) * g.mx + i;
+        Z v{0.0, 0.0};
+        if (t0 > 0) {
+          const double2 f = F[idx];
+          v = Z{f.x, f.y};
+        } else if (noise) {
+          const double2 q = ((const double2*)noise)[idx];
+          v = h2cf * Z{q.x, q.y};
+        }
+        for (int s = 0; s < nt; ++s) {
+          const short2 q = sR[r][s];
+          if (i < q.x || i >= q.y) continue;
+          const int64_t o = (int64_t)(t0 + s) * 15 * mmax + i;
+          v = mad(sA[r][s], TT::ld(tab, o), v);
+          v = mad(sB[r][s], TT::ld(tab, o + 2 * (int64_t)mmax), v);
+          v = mad(sC[r][s], TT::ld(tab, o + 4 * (int64_t)mmax), v);
+          if (i == 0) v = v - sE[r][0][s];
+          if (i == g.mx - 1) v = v - sE[r][1][s];
+        }
+        F[idx] = make_double2(v.re, v.im);
       }
     }
+    __syncthreads();
   }
-  F[2 * idx] = Fv.re;
-  F[2 * idx + 1] = Fv.im;
 }
 
 }  // namespace
 
-// Upload the complex tables [nterm][3][5][mmax] and coefficients, launch, free.
-int launch_rhs(const Geom& g, double h, cd k, int nterm, int mmax, const std::vector<double>& tab,
-               const double* coef, const double* noise, double* F, cudaStream_t s) {
-  double *dtab = nullptr, *dcoef = nullptr;
-  if (cudaMallocAsync((void**)&dtab, tab.size() * sizeof(double), s) != cudaSuccess) return HELM6_ERR_NOMEM;
-  if (cudaMallocAsync((void**)&dcoef, (size_t)std::max(nterm, 1) * 2 * sizeof(double), s) != cudaSuccess) {
-    cudaFreeAsync(dtab, s);
+// Upload the tables (real [nterm][3][5][mmax] doubles or complex pairs of that shape), the
+// coefficients and the terms' nonzero ranges in one buffer, launch, free.
+int launch_rhs(const Geom& g, double h, cd k, int nterm, int mmax, const double* tab, bool real, const double* coef,
+               const double* noise, double* F, cudaStream_t s) {
+  const size_t per = (size_t)15 * mmax * (real ? 1 : 2), ntab = per * nterm;
+  const size_t nrng = ((size_t)nterm * sizeof(TermRange) + 7) / 8;
+  std::vector<double> buf(std::max<size_t>(ntab + 2 * (size_t)nterm + nrng, 1));
+  if (nterm > 0) {
+    std::copy(tab, tab + ntab, buf.begin());
+    std::copy(coef, coef + 2 * (size_t)nterm, buf.begin() + ntab);
+  }
+  const int mdim[3] = {g.mx, g.my, g.mz};
+  // a non-finite amplitude or table value reaches every point (0 * Inf): nothing is skipped then
+  std::vector<TermRange> rg((size_t)nterm);
+  for (int t = 0; t < nterm; ++t) {
+    bool finite = std::isfinite(coef[2 * t]) && std::isfinite(coef[2 * t + 1]);
+    const double* tt = tab + (size_t)t * per;
+    const int e = real ? 1 : 2;
+    for (int a = 0; a < 3; ++a) {
+      int lo = mdim[a], hi = 0;
+      for (int m = 0; m < 5; ++m) {
+        const double* p = tt + (size_t)(a * 5 + m) * mmax * e;
+        for (int i = 0; i < mdim[a] * e; ++i) {
+          if (!std::isfinite(p[i])) finite = false;
+          if (p[i] != 0.0) {
+            lo = std::min(lo, i / e);
+            hi = std::max(hi, i / e + 1);
+          }
+        }
+      }
+      rg[t].lo[a] = lo;
+      rg[t].hi[a] = hi;
+    }
+    if (!finite)
+      for (int a = 0; a < 3; ++a) {
+        rg[t].lo[a] = 0;
+        rg[t].hi[a] = mdim[a];
+      }
+  }
+  if (nterm > 0) std::memcpy(buf.data() + ntab + 2 * (size_t)nterm, rg.data(), (size_t)nterm * sizeof(TermRange));
+  double* dbuf = nullptr;
+  if (cudaMallocAsync((void**)&dbuf, buf.size() * sizeof(double), s) != cudaSuccess) {
+    cudaGetLastError();
     return HELM6_ERR_NOMEM;
   }
-  cudaMemcpyAsync(dtab, tab.data(), tab.size() * sizeof(double), cudaMemcpyHostToDevice, s);
-  if (nterm > 0)
-    cudaMemcpyAsync(dcoef, coef, (size_t)nterm * 2 * sizeof(double), cudaMemcpyHostToDevice, s);
+  cudaMemcpyAsync(dbuf, buf.data(), buf.size() * sizeof(double), cudaMemcpyHostToDevice, s);
 
   RhsCoef c;
   const cd I(0.0, 1.0);
@@ -162,22 +264,27 @@ int launch_rhs(const Geom& g, double h, cd k, int nterm, int mmax, const std::ve
   c.e1mu3 = to_pod(std::exp(ik * h) * mu3);
   c.mu1h5 = to_pod(mu1 * h5 / 3.0);
 
-  const int bs = 256;
+  const int64_t rows = (int64_t)g.my * g.mz;
+  const unsigned grid = (unsigned)((rows + RHS_ROWS - 1) / RHS_ROWS);
+  const double* damp = dbuf + ntab;
+  const TermRange* drng = (const TermRange*)(damp + 2 * (size_t)nterm);
   note_launch();
-  rhs_kernel<<<(unsigned)((g.N + bs - 1) / bs), bs, 0, s>>>(g, c, nterm, mmax, dtab, dcoef, noise, F);
-  cudaFreeAsync(dtab, s);
-  cudaFreeAsync(dcoef, s);
+  if (real)
+    rhs_kernel<true><<<grid, 32 * RHS_WARPS, 0, s>>>(g, c, nterm, mmax, dbuf, damp, drng, noise, (double2*)F);
+  else
+    rhs_kernel<false><<<grid, 32 * RHS_WARPS, 0, s>>>(g, c, nterm, mmax, dbuf, damp, drng, noise, (double2*)F);
+  cudaFreeAsync(dbuf, s);
   return cudaGetLastError() == cudaSuccess ? HELM6_OK : HELM6_ERR_CUDA;
 }
 
 // Gaussian sources: 1D derivative tables G^(m)(x) = (-1/sigma)^m He_m(t) exp(-t^2/2),
 // t = (x-c)/sigma, with He the probabilists' Hermite polynomials, at the unknown nodes of
-// each axis (real, stored as complex with zero imaginary part).
+// each axis (real).
 int rhs_gaussians(const Geom& g, double h, cd k, int nsrc, const double* centers, const double* amps,
                   double sigma, const double* noise, double* F, cudaStream_t s) {
   const int mmax = std::max(g.mx, std::max(g.my, g.mz));
   const int mdim[3] = {g.mx, g.my, g.mz};
-  std::vector<double> tab((size_t)std::max(nsrc, 1) * 15 * mmax * 2, 0.0);
+  std::vector<double> tab((size_t)nsrc * 15 * mmax, 0.0);
   for (int src = 0; src < nsrc; ++src) {
     for (int ax = 0; ax < 3; ++ax) {
       const int start = (g.face[2 * ax] == HELM6_DIRICHLET) ? 1 : 0;
@@ -191,13 +298,13 @@ int rhs_gaussians(const Geom& g, double h, cd k, int nsrc, const double* centers
         for (int m = 1; m < 4; ++m) he[m + 1] = t * he[m] - m * he[m - 1];
         double sc = 1.0;
         for (int m = 0; m < 5; ++m) {
-          tab[2 * (((size_t)src * 3 + ax) * 5 + m) * mmax + 2 * (size_t)p] = sc * he[m] * e;
+          tab[(((size_t)src * 3 + ax) * 5 + m) * mmax + (size_t)p] = sc * he[m] * e;
           sc *= -1.0 / sigma;
         }
       }
     }
   }
-  return launch_rhs(g, h, k, nsrc, mmax, tab, amps, noise, F, s);
+  return launch_rhs(g, h, k, nsrc, mmax, tab.data(), true, amps, noise, F, s);
 }
 
 // Separable source given by the caller's complex tables [nterm][3][5][mmax] (mmax the
@@ -205,9 +312,7 @@ int rhs_gaussians(const Geom& g, double h, cd k, int nsrc, const double* centers
 int rhs_separable(const Geom& g, double h, cd k, int nterm, const double* coef, const double* tables, double* F,
                   cudaStream_t s) {
   const int mmax = std::max(g.mx, std::max(g.my, g.mz));
-  std::vector<double> tab((size_t)std::max(nterm, 1) * 15 * mmax * 2, 0.0);
-  if (nterm > 0) std::copy(tables, tables + (size_t)nterm * 15 * mmax * 2, tab.begin());
-  return launch_rhs(g, h, k, nterm, mmax, tab, coef, nullptr, F, s);
+  return launch_rhs(g, h, k, nterm, mmax, tables, false, coef, nullptr, F, s);
 }
 
 namespace {
