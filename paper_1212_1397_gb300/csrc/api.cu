@@ -53,6 +53,9 @@ struct helm6_ctx {
   uint8_t *Wx_tc = nullptr, *Wy_tc = nullptr, *Vx_tc = nullptr, *Vy_tc = nullptr;
   int* tcerr = nullptr;
   ZLines zl;  // z-line pivot tables (tensor-core path)
+  // FP64: the transforms in integer slices on the tensor cores (x64), basis digits per matrix
+  bool x64 = false;
+  X64Basis Wx6, Vx6, Wy6, Vy6;
   // x/y transforms: HELM6_XFORM_DENSE, _FFT or _TENSOR per internal axis, and the FFT plans
   int xform[2] = {HELM6_XFORM_DENSE, HELM6_XFORM_DENSE};
   FftDev fft[2] = {};
@@ -121,10 +124,11 @@ struct helm6_ctx {
 
 namespace {
 
-constexpr int kDiverge = 1000;
-
 // Axis length rounded up to a multiple of 4 (row pitch of the tensor-core intermediates).
-inline int pad4(int m) { return (m + 3) & ~3; }  // SKS: relative residual growth that counts as divergence
+inline int pad4(int m) { return (m + 3) & ~3; }
+inline int pad2(int m) { return (m + 1) & ~1; }  // the same in FP64 (16-byte rows)
+
+constexpr int kDiverge = 1000;  // SKS: relative residual growth that counts as divergence
 
 #define CK(call)                                      \
   do {                                                \
@@ -336,7 +340,34 @@ void precond(helm6_ctx* c, const T* in, T* out, T* tA, T* tB, T* cw, const T* Vx
   prof_stop(c, HELM6_PH_XINV, e);
 }
 
+// FP64 transforms on the tensor cores: the layouts of precond_tc with FP64 pitches.
+void precond_x64(helm6_ctx* c, const double* in, double* out) {
+  const Geom& g = c->g;
+  cudaStream_t s = c->stream;
+  const int rows_x = 2 * g.mz * g.my, rows_y = 2 * g.mz * g.mx;
+  const int Xp = pad2(g.mx), Yp = pad2(g.my);
+  cudaEvent_t e = prof_start(c);
+  launch_xform64(c->Wx6, in, c->tA64, rows_x, 1, g.my, c->tcerr, s, g.mx, Yp);
+  prof_stop(c, HELM6_PH_XFWD, e);
+  e = prof_start(c);
+  launch_xform64(c->Wy6, c->tA64, c->tB64, rows_y, 0, 1, c->tcerr, s, Yp, Yp);
+  prof_stop(c, HELM6_PH_YFWD, e);
+  e = prof_start(c);
+  launch_ztri<double>(g, c->lamx, c->lamy, c->diag0, c->alpha, c->tB64, c->tA64, c->cw64, c->status, s, Yp);
+  prof_stop(c, HELM6_PH_ZTRI, e);
+  e = prof_start(c);
+  launch_xform64(c->Vy6, c->tA64, c->tB64, rows_y, 1, g.mx, c->tcerr, s, Yp, Xp);
+  prof_stop(c, HELM6_PH_YINV, e);
+  e = prof_start(c);
+  launch_xform64(c->Vx6, c->tB64, out, rows_x, 0, 1, c->tcerr, s, Xp, g.mx);
+  prof_stop(c, HELM6_PH_XINV, e);
+}
+
 void precond64(helm6_ctx* c, const double* in, double* out) {
+  if (c->x64) {
+    precond_x64(c, in, out);
+    return;
+  }
   precond<double>(c, in, out, c->tA64, c->tB64, c->cw64, c->Vx64, c->Wx64, c->Vy64, c->Wy64);
 }
 // Tensor-core path: x forward writes planes x-mode-major ([z][p][y], y pitch Yp); y forward
@@ -1340,9 +1371,35 @@ int helm6_create(helm6_ctx** out, int n, double h, helm6_c64 k, const int faces[
   // form where the axis length has one (unless dense is asked for), else dense
   const bool use_tc = o.precision == HELM6_MIXED && o.transform != HELM6_XFORM_FFT && c->g.mx <= tc_max_axis() &&
                       c->g.my <= tc_max_axis();
+  // FP64 with the form left to the library: both axes in integer slices on the tensor cores where
+  // they fit (helm6_transform still names the axis' form: FFT-type or dense).  Below 8,192 unknowns
+  // every form is a few microseconds of latency and the FFT form is the shorter one (n = 15: 15
+  // against 17 us per transform; n = 20, dense: 40 against 16).
+  if (o.precision == HELM6_FP64 && o.transform == HELM6_XFORM_AUTO && c->g.N >= 8192) {
+    std::vector<double> B[4];
+    std::vector<uint8_t> D[4];
+    X64Basis* X[4] = {&c->Wx6, &c->Vx6, &c->Wy6, &c->Vy6};
+    bool ok = true;
+    for (int a = 0; a < 4 && ok; ++a) {
+      const int lo = c->g.face[2 * (a / 2)], hi = c->g.face[2 * (a / 2) + 1];
+      x64_basis(n, lo, hi, a % 2 == 1, B[a]);
+      ok = x64_prepare(B[a], a < 2 ? c->g.mx : c->g.my, (lo == HELM6_DIRICHLET) == (hi == HELM6_DIRICHLET), *X[a], D[a]);
+    }
+    if (ok && x64_configure() != HELM6_OK) return fail(HELM6_ERR_CUDA);
+    for (int a = 0; a < 4 && ok; ++a) {
+      if ((rc = dalloc(c, &X[a]->dev, D[a].size()))) return fail(rc);
+      if (cudaMemcpy(X[a]->dev, D[a].data(), D[a].size(), cudaMemcpyHostToDevice) != cudaSuccess)
+        return fail(HELM6_ERR_CUDA);
+    }
+    c->x64 = ok;
+  }
   for (int a = 0; a < 2; ++a) {
     c->xform[a] = use_tc ? HELM6_XFORM_TENSOR : HELM6_XFORM_DENSE;
     FftHostPlan fp;
+    if (c->x64) {
+      if (fft_make_plan(n, c->g.face[2 * a], c->g.face[2 * a + 1], true, fp, false)) c->xform[a] = HELM6_XFORM_FFT;
+      continue;
+    }
     // FP64: the half-length sine/cosine form (the FP64 pipe bounds the kernel); FP32: the
     // extension form, whose rounding costs the mixed solve fewer iterations
     if (use_tc || o.transform == HELM6_XFORM_DENSE ||
@@ -1381,8 +1438,11 @@ int helm6_create(helm6_ctx** out, int n, double h, helm6_c64 k, const int faces[
     if (krylov && (rc = dalloc(c, &c->V64, v * (m + 1)))) return fail(rc);
     if (needZ && (rc = dalloc(c, &c->Z64, v * m))) return fail(rc);
     if (krylov && (rc = dalloc(c, &c->u64, v))) return fail(rc);
-    if ((rc = dalloc(c, &c->w64, v)) || (rc = dalloc(c, &c->zt64, v)) || (rc = dalloc(c, &c->tA64, v)) ||
-        (rc = dalloc(c, &c->tB64, v)) || (rc = dalloc(c, &c->cw64, v)))
+    // the tensor-core transforms' intermediates have rows padded to an even length
+    const size_t vpad = std::max(v, (size_t)2 * c->g.mz *
+                                        std::max((size_t)c->g.mx * pad2(c->g.my), (size_t)c->g.my * pad2(c->g.mx)));
+    if ((rc = dalloc(c, &c->w64, v)) || (rc = dalloc(c, &c->zt64, v)) || (rc = dalloc(c, &c->tA64, vpad)) ||
+        (rc = dalloc(c, &c->tB64, vpad)) || (rc = dalloc(c, &c->cw64, vpad)))
       return fail(rc);
   } else {
     const bool krylov = o.method == HELM6_GMRES || o.method == HELM6_FGMRES;

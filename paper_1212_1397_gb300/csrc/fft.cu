@@ -472,7 +472,7 @@ constexpr size_t kFftSmemMax = 227 * 1024;
 
 }  // namespace
 
-bool fft_make_plan(int n, int lo, int hi, bool half, FftHostPlan& h) {
+bool fft_make_plan(int n, int lo, int hi, bool half, FftHostPlan& h, bool tables) {
   const bool nlo = lo != HELM6_DIRICHLET, nhi = hi != HELM6_DIRICHLET;
   FftDev& f = h.d;
   f = FftDev{};
@@ -492,6 +492,7 @@ bool fft_make_plan(int n, int lo, int hi, bool half, FftHostPlan& h) {
   f.logP = ilog2(f.P);
   f.logM = f.M ? ilog2(f.M) : 0;
   if (smem_of(f, 1, 8) > kFftSmemMax) return false;
+  if (!tables) return true;
 
   // complex tables, interleaved: [w_P^k: P/2][w_M^k: M/2][bhat: M][w_L^t: L when Q > 1]
   // [(cos, sin)(pi j / N), j = 0..N: sine and cosine axes]

@@ -123,12 +123,27 @@ void tc_prepare_basis(const std::vector<double>& B, int P, int K, std::vector<ui
 void launch_xform_tc(const float* in, float* out, const uint8_t* W, int M_total, int K, int P, int terms,
                      int transposed, int R, int* err, cudaStream_t s, int ldin = 0, int ldo = 0);
 
+// FP64 x/y transform in exact integer slices on the tensor cores (xform64.cu): one basis matrix
+// (m x m) as digit planes, and the same for symmetric (fold) bases over half the points.
+struct X64Basis {
+  uint8_t* dev = nullptr;  // digit planes (device)
+  int m = 0, fold = 0, nk = 0, nch = 0, gcols = 0, ngroups = 0, eb = 0;
+};
+void x64_basis(int n, int lo, int hi, bool inverse, std::vector<double>& B);
+bool x64_prepare(const std::vector<double>& B, int m, bool fold, X64Basis& h, std::vector<uint8_t>& out);
+int x64_configure();
+// out(row, p) = sum_k in(row, k) B(p, k): rows of pitch ldin; transposed and row-major outputs
+// as launch_xform_tc; *err is set if a bounded wait timed out.
+void launch_xform64(const X64Basis& b, const double* in, double* out, int M_total, int transposed, int R, int* err,
+                    cudaStream_t s, int ldin, int ldo);
+
 // Tridiagonal solve along z for every (x, y) mode pair, Thomas algorithm started at the
 // Sommerfeld-like end (if any).  x: input, y: output (may alias x), cw: scratch of 2N T.
-// xmajor: planes stored x-mode-major (p*my + q) rather than y-major (q*mx + p).
+// ldq > 0: planes stored x-mode-major with q pitch ldq (p*ldq + q), x, y and cw so padded, rather
+// than y-major (q*mx + p).
 template <typename T>
 void launch_ztri(const Geom& g, const double* lamx, const double* lamy, c64d diag0, c64d alpha,
-                 const T* x, T* y, T* cw, int* status, cudaStream_t s, int xmajor = 0);
+                 const T* x, T* y, T* cw, int* status, cudaStream_t s, int ldq = 0);
 
 // The same z-line solve with the elimination's pivots precomputed in FP64 (once per
 // context) and stored in FP32 (tensor-core path): rinv holds the pivot reciprocal of every
@@ -166,8 +181,9 @@ struct FftHostPlan {
 };
 // Plan for n interior nodes and the axis' faces lo, hi (helm6_bc), in the half-length form
 // where `half` asks for it and the faces allow it; false when L has no
-// factorisation of the form above or a line does not fit in shared memory.
-bool fft_make_plan(int n, int lo, int hi, bool half, FftHostPlan& plan);
+// factorisation of the form above or a line does not fit in shared memory.  tables = false:
+// the sizes only.
+bool fft_make_plan(int n, int lo, int hi, bool half, FftHostPlan& plan, bool tables = true);
 void fft_configure();  // once per process: the kernels' dynamic shared memory limit
 // out = W in (inv = 0, forward) or V in (inv = 1) along axis 0 (x) or 1 (y) of the planar
 // field (same layout in and out; out may not alias in).
