@@ -53,6 +53,7 @@ struct helm6_ctx {
   uint8_t *Wx_tc = nullptr, *Wy_tc = nullptr, *Vx_tc = nullptr, *Vy_tc = nullptr;
   int* tcerr = nullptr;
   ZLines zl;  // z-line pivot tables (tensor-core path)
+  ZLinesT<double> zl64;  // ... and of an FP64 context
   // FP64: the transforms in integer slices on the tensor cores (x64), basis digits per matrix
   bool x64 = false;
   X64Basis Wx6, Vx6, Wy6, Vy6;
@@ -64,7 +65,7 @@ struct helm6_ctx {
   double* D64 = nullptr;           // Chebyshev direction
   double cheb_lo = 0, cheb_hi = 0;  // spectral interval of A A_p^{-1} (HELM6_CHEB)
   double *V64 = nullptr, *Z64 = nullptr, *w64 = nullptr, *zt64 = nullptr, *tA64 = nullptr,
-         *tB64 = nullptr, *cw64 = nullptr;
+         *tB64 = nullptr;
   // FP32 vectors (MIXED)
   float *V32 = nullptr, *Z32 = nullptr, *w32 = nullptr, *zt32 = nullptr, *tA32 = nullptr,
         *tB32 = nullptr, *cw32 = nullptr;
@@ -203,12 +204,16 @@ void prof_stop(helm6_ctx* c, int ph, cudaEvent_t a, double bytes = 0.0) {
 //      with end weights w = 1/2 at 0 and n+1
 // D-N: nodes 1..n+1, th_j = (2j-1) t/2, V[l][j] = sin(l th_j), V^{-1}[j][l] = (2/(n+1)) w_l sin(l th_j),
 //      w_{n+1} = 1/2, lam = -4 sin^2(th_j/2);  N-D: nodes 0..n, cos(l th_j), w_0 = 1/2.
-void basis(int n, int lo, int hi, std::vector<double>& V, std::vector<double>& W, std::vector<double>& lam) {
+// Without `matrices` the eigenvalues alone.
+void basis(int n, int lo, int hi, std::vector<double>& V, std::vector<double>& W, std::vector<double>& lam,
+           bool matrices) {
   const double t = M_PI / (n + 1);
   const bool nlo = lo != HELM6_DIRICHLET, nhi = hi != HELM6_DIRICHLET;
   const int m = n + (nlo ? 1 : 0) + (nhi ? 1 : 0);
-  V.assign((size_t)m * m, 0.0);
-  W.assign((size_t)m * m, 0.0);
+  if (matrices) {
+    V.assign((size_t)m * m, 0.0);
+    W.assign((size_t)m * m, 0.0);
+  }
   lam.assign(m, 0.0);
   const double sc = 2.0 / (n + 1);
   for (int jj = 0; jj < m; ++jj) {
@@ -238,6 +243,7 @@ void basis(int n, int lo, int hi, std::vector<double>& V, std::vector<double>& W
         wv = sc * wl * v;
         lam[jj] = -4.0 * std::pow(std::sin(th / 2), 2);
       }
+      if (!matrices) break;
       V[(size_t)p * m + jj] = v;   // row = node p, column = mode jj
       W[(size_t)jj * m + p] = wv;  // row = mode jj, column = node p
     }
@@ -324,7 +330,10 @@ void precond(helm6_ctx* c, const T* in, T* out, T* tA, T* tB, T* cw, const T* Vx
     launch_axis_gemm<T>(Wy, tA, tB, g.my, g.mx, g.mx, plane, 2 * g.mz, false, s);
   prof_stop(c, HELM6_PH_YFWD, e);
   e = prof_start(c);
-  launch_ztri<T>(g, c->lamx, c->lamy, c->diag0, c->alpha, tB, tA, cw, c->status, s);
+  if constexpr (std::is_same<T, double>::value)
+    launch_ztri_apply<double>(g, c->zl64, tB, tA, s);
+  else
+    launch_ztri<T>(g, c->lamx, c->lamy, c->diag0, c->alpha, tB, tA, cw, c->status, s);
   prof_stop(c, HELM6_PH_ZTRI, e);
   e = prof_start(c);
   if (fy)
@@ -353,7 +362,7 @@ void precond_x64(helm6_ctx* c, const double* in, double* out) {
   launch_xform64(c->Wy6, c->tA64, c->tB64, rows_y, 0, 1, c->tcerr, s, Yp, Yp);
   prof_stop(c, HELM6_PH_YFWD, e);
   e = prof_start(c);
-  launch_ztri<double>(g, c->lamx, c->lamy, c->diag0, c->alpha, c->tB64, c->tA64, c->cw64, c->status, s, Yp);
+  launch_ztri_apply<double>(g, c->zl64, c->tB64, c->tA64, s);
   prof_stop(c, HELM6_PH_ZTRI, e);
   e = prof_start(c);
   launch_xform64(c->Vy6, c->tA64, c->tB64, rows_y, 1, g.mx, c->tcerr, s, Yp, Xp);
@@ -368,7 +377,7 @@ void precond64(helm6_ctx* c, const double* in, double* out) {
     precond_x64(c, in, out);
     return;
   }
-  precond<double>(c, in, out, c->tA64, c->tB64, c->cw64, c->Vx64, c->Wx64, c->Vy64, c->Wy64);
+  precond<double>(c, in, out, c->tA64, c->tB64, nullptr, c->Vx64, c->Wx64, c->Vy64, c->Wy64);
 }
 // Tensor-core path: x forward writes planes x-mode-major ([z][p][y], y pitch Yp); y forward
 // contracts the now contiguous y ([z][p][q], pitch Yp); the z lines walk that order; y inverse
@@ -388,7 +397,7 @@ void precond_tc(helm6_ctx* c, const float* in, float* out) {
   launch_xform_tc(c->tA32, c->tB32, c->Wy_tc, rows_y, g.my, g.my, terms, 0, 1, c->tcerr, s, Yp, Yp);
   prof_stop(c, HELM6_PH_YFWD, e);
   e = prof_start(c);
-  launch_ztri_apply(g, c->zl, c->tB32, c->tA32, s);
+  launch_ztri_apply<float>(g, c->zl, c->tB32, c->tA32, s);
   prof_stop(c, HELM6_PH_ZTRI, e);
   e = prof_start(c);
   launch_xform_tc(c->tA32, c->tB32, c->Vy_tc, rows_y, g.my, g.my, terms, 1, g.mx, c->tcerr, s, Yp, Xp);
@@ -1349,26 +1358,6 @@ int helm6_create(helm6_ctx** out, int n, double h, helm6_c64 k, const int faces[
   }
   // bases
   std::vector<double> Vx, Wx, lx, Vy, Wy, ly;
-  basis(n, c->g.face[0], c->g.face[1], Vx, Wx, lx);  // the internal x and y faces
-  basis(n, c->g.face[2], c->g.face[3], Vy, Wy, ly);
-  const size_t mx2 = (size_t)c->g.mx * c->g.mx, my2 = (size_t)c->g.my * c->g.my;
-  if ((rc = dalloc(c, &c->Vx64, mx2)) || (rc = dalloc(c, &c->Wx64, mx2)) || (rc = dalloc(c, &c->Vy64, my2)) ||
-      (rc = dalloc(c, &c->Wy64, my2)) || (rc = dalloc(c, &c->Vx32, mx2)) || (rc = dalloc(c, &c->Wx32, mx2)) ||
-      (rc = dalloc(c, &c->Vy32, my2)) || (rc = dalloc(c, &c->Wy32, my2)) ||
-      (rc = dalloc(c, &c->lamx, (size_t)c->g.mx)) || (rc = dalloc(c, &c->lamy, (size_t)c->g.my)))
-    return fail(rc);
-  auto up64 = [&](double* d, const std::vector<double>& h_) {
-    return cudaMemcpy(d, h_.data(), h_.size() * sizeof(double), cudaMemcpyHostToDevice);
-  };
-  auto up32 = [&](float* d, const std::vector<double>& h_) {
-    std::vector<float> f(h_.begin(), h_.end());
-    return cudaMemcpy(d, f.data(), f.size() * sizeof(float), cudaMemcpyHostToDevice);
-  };
-  if (up64(c->Vx64, Vx) || up64(c->Wx64, Wx) || up64(c->Vy64, Vy) || up64(c->Wy64, Wy) || up64(c->lamx, lx) ||
-      up64(c->lamy, ly) || up32(c->Vx32, Vx) || up32(c->Wx32, Wx) || up32(c->Vy32, Vy) || up32(c->Wy32, Wy))
-    return fail(HELM6_ERR_CUDA);
-  // transforms: dense on tensor cores (MIXED, both axes fit, not FFT-forced), else the FFT
-  // form where the axis length has one (unless dense is asked for), else dense
   const bool use_tc = o.precision == HELM6_MIXED && o.transform != HELM6_XFORM_FFT && c->g.mx <= tc_max_axis() &&
                       c->g.my <= tc_max_axis();
   // FP64 with the form left to the library: both axes in integer slices on the tensor cores where
@@ -1376,14 +1365,14 @@ int helm6_create(helm6_ctx** out, int n, double h, helm6_c64 k, const int faces[
   // every form is a few microseconds of latency and the FFT form is the shorter one (n = 15: 15
   // against 17 us per transform; n = 20, dense: 40 against 16).
   if (o.precision == HELM6_FP64 && o.transform == HELM6_XFORM_AUTO && c->g.N >= 8192) {
-    std::vector<double> B[4];
+    std::vector<double> B;
     std::vector<uint8_t> D[4];
     X64Basis* X[4] = {&c->Wx6, &c->Vx6, &c->Wy6, &c->Vy6};
     bool ok = true;
     for (int a = 0; a < 4 && ok; ++a) {
       const int lo = c->g.face[2 * (a / 2)], hi = c->g.face[2 * (a / 2) + 1];
-      x64_basis(n, lo, hi, a % 2 == 1, B[a]);
-      ok = x64_prepare(B[a], a < 2 ? c->g.mx : c->g.my, (lo == HELM6_DIRICHLET) == (hi == HELM6_DIRICHLET), *X[a], D[a]);
+      x64_basis(n, lo, hi, a % 2 == 1, B);
+      ok = x64_prepare(B, a < 2 ? c->g.mx : c->g.my, (lo == HELM6_DIRICHLET) == (hi == HELM6_DIRICHLET), *X[a], D[a]);
     }
     if (ok && x64_configure() != HELM6_OK) return fail(HELM6_ERR_CUDA);
     for (int a = 0; a < 4 && ok; ++a) {
@@ -1393,6 +1382,35 @@ int helm6_create(helm6_ctx** out, int n, double h, helm6_c64 k, const int faces[
     }
     c->x64 = ok;
   }
+  // the dense matrices: what the tensor-core tiles of a MIXED context are made from, and device
+  // copies in the working precision where a SIMT dense form may read them
+  basis(n, c->g.face[0], c->g.face[1], Vx, Wx, lx, !c->x64);  // the internal x and y faces
+  basis(n, c->g.face[2], c->g.face[3], Vy, Wy, ly, !c->x64);
+  if ((rc = dalloc(c, &c->lamx, (size_t)c->g.mx)) || (rc = dalloc(c, &c->lamy, (size_t)c->g.my))) return fail(rc);
+  auto up64 = [&](double** d, const std::vector<double>& h_) -> int {
+    const int r2 = *d ? (int)HELM6_OK : dalloc(c, d, h_.size());
+    if (r2) return r2;
+    return cudaMemcpy(*d, h_.data(), h_.size() * sizeof(double), cudaMemcpyHostToDevice) == cudaSuccess
+               ? (int)HELM6_OK
+               : (int)HELM6_ERR_CUDA;
+  };
+  auto up32 = [&](float** d, const std::vector<double>& h_) -> int {
+    std::vector<float> f(h_.begin(), h_.end());
+    const int r2 = dalloc(c, d, f.size());
+    if (r2) return r2;
+    return cudaMemcpy(*d, f.data(), f.size() * sizeof(float), cudaMemcpyHostToDevice) == cudaSuccess
+               ? (int)HELM6_OK
+               : (int)HELM6_ERR_CUDA;
+  };
+  if ((rc = up64(&c->lamx, lx)) || (rc = up64(&c->lamy, ly))) return fail(rc);
+  if (o.precision == HELM6_FP64 && !c->x64 &&
+      ((rc = up64(&c->Vx64, Vx)) || (rc = up64(&c->Wx64, Wx)) || (rc = up64(&c->Vy64, Vy)) || (rc = up64(&c->Wy64, Wy))))
+    return fail(rc);
+  if (o.precision == HELM6_MIXED && !use_tc &&
+      ((rc = up32(&c->Vx32, Vx)) || (rc = up32(&c->Wx32, Wx)) || (rc = up32(&c->Vy32, Vy)) || (rc = up32(&c->Wy32, Wy))))
+    return fail(rc);
+  // transforms: dense on tensor cores (MIXED, both axes fit, not FFT-forced), else the FFT
+  // form where the axis length has one (unless dense is asked for), else dense
   for (int a = 0; a < 2; ++a) {
     c->xform[a] = use_tc ? HELM6_XFORM_TENSOR : HELM6_XFORM_DENSE;
     FftHostPlan fp;
@@ -1442,8 +1460,9 @@ int helm6_create(helm6_ctx** out, int n, double h, helm6_c64 k, const int faces[
     const size_t vpad = std::max(v, (size_t)2 * c->g.mz *
                                         std::max((size_t)c->g.mx * pad2(c->g.my), (size_t)c->g.my * pad2(c->g.mx)));
     if ((rc = dalloc(c, &c->w64, v)) || (rc = dalloc(c, &c->zt64, v)) || (rc = dalloc(c, &c->tA64, vpad)) ||
-        (rc = dalloc(c, &c->tB64, vpad)) || (rc = dalloc(c, &c->cw64, vpad)))
+        (rc = dalloc(c, &c->tB64, vpad)) || (rc = dalloc(c, &c->zl64.rinv, vpad)))
       return fail(rc);
+    c->zl64.ldq = c->x64 ? pad2(c->g.my) : 0;
   } else {
     const bool krylov = o.method == HELM6_GMRES || o.method == HELM6_FGMRES;
     // AUTO: FP16 from 2^23 unknowns, where the Gram-Schmidt passes are the bulk of a step;
@@ -1511,9 +1530,13 @@ int helm6_create(helm6_ctx** out, int n, double h, helm6_c64 k, const int faces[
       return fail(rc);
     c->zl.ldq = pad4(c->g.my);
     if ((rc = dalloc(c, &c->zl.rinv, (size_t)2 * c->g.mz * c->g.mx * c->zl.ldq))) return fail(rc);
-    if (cudaMemset(c->status, 0, sizeof(int)) != cudaSuccess) return fail(HELM6_ERR_CUDA);
-    launch_ztri_table(c->g, c->lamx, c->lamy, c->diag0, c->alpha, c->zl, c->status, 0);
-    if (cudaDeviceSynchronize() != cudaSuccess) return fail(HELM6_ERR_CUDA);
+  }
+  if (cudaMemset(c->status, 0, sizeof(int)) != cudaSuccess) return fail(HELM6_ERR_CUDA);
+  if (use_tc || o.precision == HELM6_FP64) {
+    if (use_tc)
+      launch_ztri_table<float>(c->g, c->lamx, c->lamy, c->diag0, c->alpha, c->zl, c->status, 0);
+    else
+      launch_ztri_table<double>(c->g, c->lamx, c->lamy, c->diag0, c->alpha, c->zl64, c->status, 0);
     int zst = 0;
     if (cudaMemcpy(&zst, c->status, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess) return fail(HELM6_ERR_CUDA);
     c->zline_breakdown = zst != 0;

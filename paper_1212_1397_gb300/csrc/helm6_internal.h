@@ -138,25 +138,29 @@ void launch_xform64(const X64Basis& b, const double* in, double* out, int M_tota
                     cudaStream_t s, int ldin, int ldo);
 
 // Tridiagonal solve along z for every (x, y) mode pair, Thomas algorithm started at the
-// Sommerfeld-like end (if any).  x: input, y: output (may alias x), cw: scratch of 2N T.
-// ldq > 0: planes stored x-mode-major with q pitch ldq (p*ldq + q), x, y and cw so padded, rather
-// than y-major (q*mx + p).
+// Sommerfeld-like end (if any), planes y-major (q*mx + p), the pivots formed on the way (the FP32
+// path without tensor cores).  x: input, y: output (may alias x), cw: scratch of 2N T.
 template <typename T>
 void launch_ztri(const Geom& g, const double* lamx, const double* lamy, c64d diag0, c64d alpha,
-                 const T* x, T* y, T* cw, int* status, cudaStream_t s, int ldq = 0);
+                 const T* x, T* y, T* cw, int* status, cudaStream_t s);
 
 // The same z-line solve with the elimination's pivots precomputed in FP64 (once per
-// context) and stored in FP32 (tensor-core path): rinv holds the pivot reciprocal of every
-// step of every line, planar (re then im), indexed like the field; the planes are
-// x-mode-major with q pitch ldq >= my (the padded layout of the transforms' intermediates).
-struct ZLines {
-  float* rinv = nullptr;
+// context) and stored in T (FP64, and FP32 on the tensor-core path): rinv holds the pivot
+// reciprocal of every step of every line, planar (re then im), indexed like the field; the
+// planes are x-mode-major with q pitch ldq >= my (the padded layout of the tensor-core
+// transforms' intermediates), or y-major (q*mx + p) where ldq is 0.
+template <typename T>
+struct ZLinesT {
+  T* rinv = nullptr;
   int ldq = 0;
 };
-void launch_ztri_table(const Geom& g, const double* lamx, const double* lamy, c64d diag0, c64d alpha, ZLines z,
+using ZLines = ZLinesT<float>;
+template <typename T>
+void launch_ztri_table(const Geom& g, const double* lamx, const double* lamy, c64d diag0, c64d alpha, ZLinesT<T> z,
                        int* status, cudaStream_t s);
-// y = the z-line solve of x (planar FP32 in that layout; y may not alias x).
-void launch_ztri_apply(const Geom& g, const ZLines& z, const float* x, float* y, cudaStream_t s);
+// y = the z-line solve of x (planar in that layout; y may not alias x).
+template <typename T>
+void launch_ztri_apply(const Geom& g, const ZLinesT<T>& z, const T* x, T* y, cudaStream_t s);
 
 // FFT-type x/y transforms (fft.cu): the closed-form 1D eigenbasis of one axis applied through
 // one complex DFT of length L = P * Q per line: of the line's odd or even extension, L = 2(n+1)

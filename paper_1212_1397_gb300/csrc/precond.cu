@@ -90,18 +90,14 @@ __global__ void __launch_bounds__(256)
 //   Neumann / Sommerfeld-like end (beta = 1), d_l = -2 + k^2h^2 + sigma (+ 2ikh at a
 //   Sommerfeld-like end).  Elimination starts at the Sommerfeld-like end when only the top
 //   face is one (there the pivots keep a positive imaginary part).
-//   ldq > 0: the plane is stored x-mode-major (index p*ldq + q, the layout the tensor-core
-//   transforms produce) instead of y-major (q*mx + p).
 template <typename T>
 __global__ void ztri_kernel(Geom g, const double* __restrict__ lamx, const double* __restrict__ lamy,
                             c64d diag0, c64d alpha, const T* __restrict__ x, T* __restrict__ y,
-                            T* __restrict__ cw, int* status, int ldq) {
-  const int64_t plane = (int64_t)g.mx * (ldq ? ldq : g.my);
+                            T* __restrict__ cw, int* status) {
+  const int64_t plane = (int64_t)g.mx * g.my;
   const int64_t pq = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (pq >= plane) return;
-  const int p = ldq ? (int)(pq / ldq) : (int)(pq % g.mx);
-  const int q = ldq ? (int)(pq % ldq) : (int)(pq / g.mx);
-  if (q >= g.my) return;
+  const int p = (int)(pq % g.mx), q = (int)(pq / g.mx);
   const double sig = lamx[p] + lamy[q];
   const int m = g.mz;
   const bool lo_s = g.face[4] == HELM6_SOMMERFELD, hi_s = g.face[5] == HELM6_SOMMERFELD;
@@ -202,15 +198,16 @@ __device__ __forceinline__ void line_coef(const Geom& g, int l, bool rev, double
   sup = rev ? a_l : c_l;
 }
 
-// Pivot table of the z lines, FP64 arithmetic stored in FP32 (once per context): for each
-// (p, q) line (planes x-mode-major with q pitch z.ldq) and step r of the elimination order,
-// rinv_r = 1 / (d_r - sub_r c'_{r-1}) with c'_r = sup_r rinv_r.
+// Pivot table of the z lines, FP64 arithmetic stored in TS (once per context): for each (p, q)
+// line and step r of the elimination order, rinv_r = 1 / (d_r - sub_r c'_{r-1}) with
+// c'_r = sup_r rinv_r.  Planes x-mode-major with q pitch z.ldq, or y-major where z.ldq is 0.
+template <typename TS>
 __global__ void ztri_table_kernel(Geom g, const double* __restrict__ lamx, const double* __restrict__ lamy,
-                                  c64d diag0, c64d alpha, ZLines z, int* status) {
-  const int64_t plane = (int64_t)g.mx * z.ldq;
+                                  c64d diag0, c64d alpha, ZLinesT<TS> z, int* status) {
+  const int64_t plane = (int64_t)g.mx * (z.ldq ? z.ldq : g.my);
   const int64_t pq = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (pq >= plane) return;
-  const int p = (int)(pq / z.ldq), q = (int)(pq % z.ldq);
+  const int p = (int)(z.ldq ? pq / z.ldq : pq % g.mx), q = (int)(z.ldq ? pq % z.ldq : pq / g.mx);
   if (q >= g.my) return;
   const double sig = lamx[p] + lamy[q];
   const int m = g.mz;
@@ -235,23 +232,25 @@ __global__ void ztri_table_kernel(Geom g, const double* __restrict__ lamx, const
     const double er = dr - sub * cr, ei = di - sub * ci;
     const double n2 = er * er + ei * ei;
     if (!(n2 > 0.0)) bad = true;
-    const double ir = er / n2, ii = -ei / n2;
+    const double inv = 1.0 / n2;
+    const double ir = sizeof(TS) == 8 ? er * inv : er / n2, ii = sizeof(TS) == 8 ? -ei * inv : -ei / n2;
     cr = sup * ir;
     ci = sup * ii;
     const int64_t idx = (int64_t)l * plane + pq;
-    z.rinv[idx] = (float)ir;
-    z.rinv[Np + idx] = (float)ii;
+    z.rinv[idx] = (TS)ir;
+    z.rinv[Np + idx] = (TS)ii;
   }
   if (bad) atomicExch(status, (int)HELM6_BREAKDOWN);
 }
 
-// line_coef in FP32 (the coefficients are 0, 1 or 2) for the per-apply sweeps.
-__device__ __forceinline__ void line_coef_f(const Geom& g, int l, bool rev, float& sub, float& sup) {
+// line_coef in the working precision (the coefficients are 0, 1 or 2) for the per-apply sweeps.
+template <typename T>
+__device__ __forceinline__ void line_coef_f(const Geom& g, int l, bool rev, T& sub, T& sup) {
   const int m = g.mz;
-  float a_l = (l == m - 1) ? ((g.face[5] != HELM6_DIRICHLET) ? 2.f : 1.f) : 1.f;
-  float c_l = (l == 0) ? ((g.face[4] != HELM6_DIRICHLET) ? 2.f : 1.f) : 1.f;
-  if (l == 0) a_l = 0.f;
-  if (l == m - 1) c_l = 0.f;
+  T a_l = (l == m - 1) ? ((g.face[5] != HELM6_DIRICHLET) ? T(2) : T(1)) : T(1);
+  T c_l = (l == 0) ? ((g.face[4] != HELM6_DIRICHLET) ? T(2) : T(1)) : T(1);
+  if (l == 0) a_l = T(0);
+  if (l == m - 1) c_l = T(0);
   sub = rev ? c_l : a_l;
   sup = rev ? a_l : c_l;
 }
@@ -263,19 +262,19 @@ __device__ __forceinline__ void line_coef_f(const Geom& g, int l, bool rev, floa
 // table only where the pivots have not converged (per line or per warp), or that bound the
 // lines in flight so that the forward results stay in L2, were 1.3 to 4 times slower: the
 // sweep is bound by the loads in flight, which conditional loads and fewer lines reduce.
-template <int U>
-__global__ void __launch_bounds__(128) ztri_lines_kernel(Geom g, ZLines z, const float* __restrict__ x,
-                                                         float* __restrict__ y) {
-  const int64_t plane = (int64_t)g.mx * z.ldq;
+template <typename T, int U>
+__global__ void __launch_bounds__(128) ztri_lines_kernel(Geom g, ZLinesT<T> z, const T* __restrict__ x,
+                                                         T* __restrict__ y) {
+  const int64_t plane = (int64_t)g.mx * (z.ldq ? z.ldq : g.my);
   const int64_t pq = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (pq >= plane || (int)(pq % z.ldq) >= g.my) return;
+  if (pq >= plane || (z.ldq && (int)(pq % z.ldq) >= g.my)) return;
   const int m = g.mz;
   const bool lo_s = g.face[4] == HELM6_SOMMERFELD, hi_s = g.face[5] == HELM6_SOMMERFELD;
   const bool rev = (!lo_s && hi_s);
   const int64_t N = (int64_t)m * plane;
-  cpx<float> yprev = mk(0.f, 0.f);
+  cpx<T> yprev = mk(T(0), T(0));
   for (int r0 = 0; r0 < m; r0 += U) {
-    cpx<float> xv[U], iv[U];
+    cpx<T> xv[U], iv[U];
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       const int r = r0 + u;
@@ -290,18 +289,18 @@ __global__ void __launch_bounds__(128) ztri_lines_kernel(Geom g, ZLines z, const
       const int r = r0 + u;
       if (r >= m) break;
       const int l = rev ? m - 1 - r : r;
-      float sub, sup;
+      T sub, sup;
       line_coef_f(g, l, rev, sub, sup);
-      const cpx<float> yp = (xv[u] - sub * yprev) * iv[u];
+      const cpx<T> yp = (sizeof(T) == 8 && sub == T(1) ? xv[u] - yprev : xv[u] - sub * yprev) * iv[u];
       const int64_t idx = (int64_t)l * plane + pq;
       y[idx] = yp.re;
       y[N + idx] = yp.im;
       yprev = yp;
     }
   }
-  cpx<float> next = mk(0.f, 0.f);
+  cpx<T> next = mk(T(0), T(0));
   for (int r0 = m - 1; r0 >= 0; r0 -= U) {
-    cpx<float> cv[U], yv[U];
+    cpx<T> cv[U], yv[U];
     // loads only here (the multiply by sup stays with the recursion below: measured 1.6x
     // faster than forming c' next to its load)
 #pragma unroll
@@ -319,10 +318,10 @@ __global__ void __launch_bounds__(128) ztri_lines_kernel(Geom g, ZLines z, const
       const int r = r0 - u;
       if (r < 0) break;
       const int l = rev ? m - 1 - r : r;
-      float sub, sup;
+      T sub, sup;
       line_coef_f(g, l, rev, sub, sup);
       const int64_t idx = (int64_t)l * plane + pq;
-      const cpx<float> v = yv[u] - (sup * cv[u]) * next;
+      const cpx<T> v = yv[u] - (sizeof(T) == 8 && sup == T(1) ? cv[u] : sup * cv[u]) * next;
       y[idx] = v.re;
       y[N + idx] = v.im;
       next = v;
@@ -345,35 +344,42 @@ void launch_axis_gemm(const T* A, const T* B, T* C, int m, int ncols, int ld, in
 
 template <typename T>
 void launch_ztri(const Geom& g, const double* lamx, const double* lamy, c64d diag0, c64d alpha,
-                 const T* x, T* y, T* cw, int* status, cudaStream_t s, int ldq) {
-  const int64_t lines = (int64_t)g.mx * (ldq ? ldq : g.my);
+                 const T* x, T* y, T* cw, int* status, cudaStream_t s) {
+  const int64_t lines = (int64_t)g.mx * g.my;
   const int bs = 128;
   note_launch();
   ztri_kernel<T><<<(unsigned)((lines + bs - 1) / bs), bs, 0, s>>>(g, lamx, lamy, diag0, alpha, x, y,
-                                                                  cw, status, ldq);
+                                                                  cw, status);
 }
 
 
-void launch_ztri_table(const Geom& g, const double* lamx, const double* lamy, c64d diag0, c64d alpha, ZLines z,
+template <typename T>
+void launch_ztri_table(const Geom& g, const double* lamx, const double* lamy, c64d diag0, c64d alpha, ZLinesT<T> z,
                        int* status, cudaStream_t s) {
-  const int64_t lines = (int64_t)g.mx * z.ldq;
+  const int64_t lines = (int64_t)g.mx * (z.ldq ? z.ldq : g.my);
   note_launch();
-  ztri_table_kernel<<<(unsigned)((lines + 127) / 128), 128, 0, s>>>(g, lamx, lamy, diag0, alpha, z, status);
+  ztri_table_kernel<T><<<(unsigned)((lines + 127) / 128), 128, 0, s>>>(g, lamx, lamy, diag0, alpha, z, status);
 }
 
-void launch_ztri_apply(const Geom& g, const ZLines& z, const float* x, float* y, cudaStream_t s) {
-  const int64_t lines = (int64_t)g.mx * z.ldq;
+template <typename T>
+void launch_ztri_apply(const Geom& g, const ZLinesT<T>& z, const T* x, T* y, cudaStream_t s) {
+  const int64_t lines = (int64_t)g.mx * (z.ldq ? z.ldq : g.my);
   note_launch();
-  ztri_lines_kernel<8><<<(unsigned)((lines + 127) / 128), 128, 0, s>>>(g, z, x, y);
+  ztri_lines_kernel<T, 8><<<(unsigned)((lines + 127) / 128), 128, 0, s>>>(g, z, x, y);
 }
+
+#define INST_Z(T)                                                                                              \
+  template void launch_ztri_table<T>(const Geom&, const double*, const double*, c64d, c64d, ZLinesT<T>, int*, \
+                                     cudaStream_t);                                                           \
+  template void launch_ztri_apply<T>(const Geom&, const ZLinesT<T>&, const T*, T*, cudaStream_t);
+INST_Z(float)
+INST_Z(double)
 
 template void launch_axis_gemm<float>(const float*, const float*, float*, int, int, int, int64_t, int,
                                       bool, cudaStream_t);
 template void launch_axis_gemm<double>(const double*, const double*, double*, int, int, int, int64_t,
                                        int, bool, cudaStream_t);
 template void launch_ztri<float>(const Geom&, const double*, const double*, c64d, c64d, const float*,
-                                 float*, float*, int*, cudaStream_t, int);
-template void launch_ztri<double>(const Geom&, const double*, const double*, c64d, c64d,
-                                  const double*, double*, double*, int*, cudaStream_t, int);
+                                 float*, float*, int*, cudaStream_t);
 
 }  // namespace helm6

@@ -663,15 +663,18 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(X_THREADS, 1) xform6
 
 int round32(int n) { return ((n + 31) / 32) * 32; }
 
-// FP16 bits of an integer of magnitude <= 128.
-uint16_t half_bits(int v) {
-  if (v == 0) return 0;
-  const uint16_t sign = v < 0 ? 0x8000 : 0;
-  const int a = std::abs(v);
-  int e = 0;
-  while ((a >> (e + 1)) != 0) ++e;
-  return (uint16_t)(sign | ((e + 15) << 10) | ((a << (10 - e)) & 0x3ff));
-}
+// FP16 bits of the integers -128 .. 128.
+struct HalfInts {
+  uint16_t bits[257];
+  HalfInts() {
+    for (int v = -128; v <= 128; ++v) {
+      const int a = std::abs(v);
+      int e = 0;
+      while ((a >> (e + 1)) != 0) ++e;
+      bits[v + 128] = a == 0 ? 0 : (uint16_t)((v < 0 ? 0x8000 : 0) | ((e + 15) << 10) | ((a << (10 - e)) & 0x3ff));
+    }
+  }
+};
 
 }  // namespace
 
@@ -734,6 +737,8 @@ bool x64_prepare(const std::vector<double>& B, int m, bool fold, X64Basis& h, st
   const size_t plane = (size_t)h.gcols * X_KT, stage = DG * plane;
   const int half = h.gcols / 2;
   out.assign((size_t)h.ngroups * h.nk * 2 * stage, 0);
+  static const HalfInts hi16;
+  const double scale = std::ldexp(1.0, 55 - h.eb);
   for (int g = 0; g < h.ngroups; ++g) {
     const int odd = fold && g >= h.nch ? 1 : 0, ch = g - odd * h.nch;
     for (int c = 0; c < h.gcols; ++c) {
@@ -743,17 +748,17 @@ bool x64_prepare(const std::vector<double>& B, int m, bool fold, X64Basis& h, st
       for (int k = 0; k < Kf; ++k) {
         double b = B[(size_t)p * K + k];
         if (odd && 2 * k == K - 1) b = 0.0;  // the middle point of an antisymmetric mode
-        int64_t x = std::llrint(std::ldexp(b, 55 - h.eb));
+        int64_t x = std::llrint(b * scale);
         for (int d = DG - 1; d >= 0; --d) {
           int v;
           if (d > 0) {
             v = (int)((x + 128) & 255) - 128;
-            x = (x - v) / 256;
+            x = (x - v) >> 8;
           } else {
             v = (int)x;
           }
           sum[d] += std::abs(v);
-          const uint16_t hb = half_bits(v);
+          const uint16_t hb = hi16.bits[v + 128];
           const size_t o = (((size_t)g * h.nk + k / X_KT) * 2 + c / half) * stage + (size_t)d * plane +
                            (size_t)((k % X_KT) / 8) * half * 16 + (size_t)(c % half) * 16 + (size_t)(k % 8) * 2;
           std::memcpy(out.data() + o, &hb, 2);
