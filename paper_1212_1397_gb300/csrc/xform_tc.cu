@@ -342,8 +342,10 @@ __global__ void __launch_bounds__(TC_THREADS, 1) xform_tc_kernel(TcArgs p) {
           const int row = it.m0 + rr, k = k0 + (bb >> 2);
           const bool valid = row < p.M_total && k < p.K;
           const float* src = valid ? p.in + (int64_t)row * p.ldin + k : p.in;
+          // (the row's padding behind point K - 1 is not read: it can hold anything, and its zero basis
+          // entries would not cancel a NaN)
           cp_async<VEC>(slot + (uint32_t)(rr * 128 + (((bb >> 4) ^ (rr & 7)) << 4) + (bb & 15)), src,
-                        valid ? VEC : 0);
+                        valid ? min(VEC, 4 * (p.K - k)) : 0);
         }
       }
       asm volatile("cp.async.commit_group;" ::: "memory");
