@@ -14,6 +14,9 @@ namespace helm6 {
 namespace {
 
 constexpr int BM = 64, BN = 64, BK = 16;
+// z-line sweeps: steps in registers and threads of a block (every line is in flight at once; blocks
+// of 64 spread 66,564 lines evenly over 152 SMs, blocks of 128 left some SMs 4 and some 3 of them)
+constexpr int ZT_U = 12, ZT_BLOCK = 64;
 
 // C(p, n) = sum_k A[p*m + k] B(k, n), one 64 x 64 tile of C per block, 4 x 4 per thread.
 template <typename T, bool ALONG_X>
@@ -263,7 +266,7 @@ __device__ __forceinline__ void line_coef_f(const Geom& g, int l, bool rev, T& s
 // lines in flight so that the forward results stay in L2, were 1.3 to 4 times slower: the
 // sweep is bound by the loads in flight, which conditional loads and fewer lines reduce.
 template <typename T, int U>
-__global__ void __launch_bounds__(128) ztri_lines_kernel(Geom g, ZLinesT<T> z, const T* __restrict__ x,
+__global__ void __launch_bounds__(ZT_BLOCK) ztri_lines_kernel(Geom g, ZLinesT<T> z, const T* __restrict__ x,
                                                          T* __restrict__ y) {
   const int64_t plane = (int64_t)g.mx * (z.ldq ? z.ldq : g.my);
   const int64_t pq = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -321,7 +324,9 @@ __global__ void __launch_bounds__(128) ztri_lines_kernel(Geom g, ZLinesT<T> z, c
       T sub, sup;
       line_coef_f(g, l, rev, sub, sup);
       const int64_t idx = (int64_t)l * plane + pq;
-      const cpx<T> v = yv[u] - (sizeof(T) == 8 && sup == T(1) ? cv[u] : sup * cv[u]) * next;
+      const cpx<T> cc = sizeof(T) == 8 && sup == T(1) ? cv[u] : sup * cv[u];
+      const cpx<T> v = mk(fmx(cc.im, next.im, fmx(-cc.re, next.re, yv[u].re)),
+                          fmx(-cc.im, next.re, fmx(-cc.re, next.im, yv[u].im)));
       y[idx] = v.re;
       y[N + idx] = v.im;
       next = v;
@@ -365,7 +370,7 @@ template <typename T>
 void launch_ztri_apply(const Geom& g, const ZLinesT<T>& z, const T* x, T* y, cudaStream_t s) {
   const int64_t lines = (int64_t)g.mx * (z.ldq ? z.ldq : g.my);
   note_launch();
-  ztri_lines_kernel<T, 8><<<(unsigned)((lines + 127) / 128), 128, 0, s>>>(g, z, x, y);
+  ztri_lines_kernel<T, ZT_U><<<(unsigned)((lines + ZT_BLOCK - 1) / ZT_BLOCK), ZT_BLOCK, 0, s>>>(g, z, x, y);
 }
 
 #define INST_Z(T)                                                                                              \
