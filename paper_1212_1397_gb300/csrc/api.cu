@@ -860,7 +860,7 @@ void enqueue_residual_dev(helm6_ctx* c, cudaStream_t s) {
 // residual, then a WHILE node whose body is the cycle (pre-cycle segment, m + 1 IF nodes
 // holding the Arnoldi steps, post-cycle segment).
 template <typename TV>
-int append_solve_graph(helm6_ctx* c, TV* V, cudaGraph_t G, int m) {
+int append_solve_graph(helm6_ctx* c, TV* V, cudaGraph_t G, int m, int share) {
   const int64_t N = c->g.N, vs = 2 * N;
   const int ldh = c->mrest + 1;
   const double vsc = std::is_same<TV, float>::value ? 1.0 : c->vscale;
@@ -896,7 +896,7 @@ int append_solve_graph(helm6_ctx* c, TV* V, cudaGraph_t G, int m) {
       if (full) {
         float* zj = c->Z32 + (int64_t)j * vs;
         precond32(c, c->u32, zj);
-        launch_stencil<float>(c->g, c->coef, zj, c->w32, nullptr, nullptr, 0, nullptr, nullptr, s);
+        launch_stencil<float>(c->g, c->coef, zj, c->w32, nullptr, nullptr, 0, nullptr, nullptr, s, share);
       }
       launch_dcgs_dot<float, TV>(V, vs, j, c->u32, full ? c->w32 : nullptr, N, c->partial, c->ndot, vsc, s);
       launch_reduce_cols(c->partial, c->ndot, 4 * j + 3, c->red, 0, s);
@@ -919,8 +919,9 @@ int append_solve_graph(helm6_ctx* c, TV* V, cudaGraph_t G, int m) {
   });
 }
 
-int append_solve(helm6_ctx* c, cudaGraph_t G, int m) {
-  return c->V16 ? append_solve_graph<__half>(c, c->V16, G, m) : append_solve_graph<float>(c, c->V32, G, m);
+int append_solve(helm6_ctx* c, cudaGraph_t G, int m, int share = 1) {
+  return c->V16 ? append_solve_graph<__half>(c, c->V16, G, m, share)
+                : append_solve_graph<float>(c, c->V32, G, m, share);
 }
 
 // Parameters of one solve into the control block (stream-ordered upload from pinned memory).
@@ -1014,7 +1015,7 @@ int batch_exec(const std::vector<helm6_ctx*>& act, int m, cudaGraphExec_t* out) 
   const long long l0 = launch_total();
   int rc = HELM6_OK;
   for (helm6_ctx* c : act)
-    if ((rc = append_solve(c, G, m))) break;
+    if ((rc = append_solve(c, G, m, (int)act.size()))) break;
   note_launch(-(int)(launch_total() - l0));
   cudaGraphExec_t ex = nullptr;
   if (rc == HELM6_OK && cudaGraphInstantiate(&ex, G, 0) != cudaSuccess) rc = HELM6_ERR_CUDA;

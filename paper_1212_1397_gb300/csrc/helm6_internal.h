@@ -91,11 +91,12 @@ void stencil_coefficients(cd k, double h, StencilCoef& c);
 
 // y = A x (mode 0);  y = f - A x (mode 1);  y = f + A x (mode 2, no norm), A given by its row
 // weights.
+// share: how many problems run side by side on the GPU (FP32, without a norm: sets the block size).
 // sumsq (nullable): per-block partial sums of |y|^2, nblk entries written, reduced by
 // reduce_sum.
 template <typename T>
 void launch_stencil(const Geom& g, const StencilCoef& c, const T* x, T* y, const T* f, T* r,
-                    int mode, double* sumsq, int* nblk, cudaStream_t s);
+                    int mode, double* sumsq, int* nblk, cudaStream_t s, int share = 1);
 
 // Number of blocks (and fused-norm partials) of launch_stencil for this geometry.
 int stencil_blocks(const Geom& g);

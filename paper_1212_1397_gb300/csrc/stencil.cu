@@ -9,18 +9,38 @@
 // across x/y faces and across Neumann z faces are even reflections (U_{-1} = U_1);
 // across Dirichlet faces they are zero.
 //
-// Thread block: a 32 x 8 (x, y) tile marching over a chunk of 32 z planes.  Each plane
+// Thread block: a 32 x 8 (x, y) tile marching over a chunk of up to 32 z planes.  Each plane
 // tile plus a one-point halo is staged in shared memory by asynchronous copies issued
 // three planes ahead into a ring of five buffers (one barrier per plane); each thread
 // keeps the three plane sums (C, Nb, Dg) of planes l-1, l, l+1 in registers, so every
 // input value is read from global memory once per chunk.
+#include <algorithm>
+
 #include "helm6_internal.h"
 
 namespace helm6 {
 
 namespace {
 
-constexpr int TX = 32, TY = 8, ZCH = 32;
+constexpr int TX = 32, TY = 8;
+constexpr int ZCH = 32;  // most z planes per block
+
+// Planes per block for `tiles` (x, y) tiles of mz planes: 32 where that leaves `per_sm` blocks per
+// SM, else half as many, down to 2 (a block reads two planes more than it computes).  A block
+// marches plane by plane, so on small grids its length is the kernel's time; on large ones longer
+// blocks read less twice.  Measured, 32 planes a block against this rule: FP32 34 -> 9 us at 32^3,
+// 35 -> 19 at 128^3, unchanged at 256^3 (16 planes there: 85 against 82); FP64 87 -> 12 and
+// 164 -> 157 us.
+constexpr int ZB32 = 3, ZB64 = 6;  // blocks per SM asked for: FP32, FP64 (best of 2 to 32 planes at 64^3 to 256^3)
+// share: problems running side by side, which fill the SMs together (6 problems of 96 to 160
+// points a side in one batch: 26.5 ms with each block length chosen as if alone, 25.3 so).
+int z_chunk(int tiles, int mz, int per_sm, int share = 1) {
+  static int sms = 0;
+  if (!sms) sms = device_sm_count();
+  int z = ZCH;
+  while (z > 2 && (int64_t)tiles * ((mz + z - 1) / z) * share < (int64_t)per_sm * sms) z /= 2;
+  return z;
+}
 
 template <typename T>
 struct Sums {
@@ -49,7 +69,7 @@ __device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0
 template <typename T, int MODE, bool NORM, bool RW>
 __global__ void __launch_bounds__(TX* TY)
     stencil_kernel(Geom g, StencilCoef coef, const T* __restrict__ x, T* __restrict__ y,
-                   const T* __restrict__ f, double* __restrict__ sumsq) {
+                   const T* __restrict__ f, double* __restrict__ sumsq, int zch) {
   // ring of NBUF staged planes; plane p + DIST is requested while plane p is used
   constexpr int DIST = 3, NBUF = DIST + 2;
   __shared__ T sre[NBUF][TY + 2][TX + 2];
@@ -58,8 +78,8 @@ __global__ void __launch_bounds__(TX* TY)
 
   const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * TX + tx;
   const int i = blockIdx.x * TX + tx, j = blockIdx.y * TY + ty;
-  const int l0 = blockIdx.z * ZCH;
-  const int l1 = min(l0 + ZCH, g.mz);
+  const int l0 = blockIdx.z * zch;
+  const int l1 = min(l0 + zch, g.mz);
   const int64_t plane = (int64_t)g.mx * g.my;
   const bool active = (i < g.mx) && (j < g.my);
 
@@ -218,7 +238,6 @@ __global__ void __launch_bounds__(TX* TY)
 // 16-byte chunks when mx % 4 == 0; the two edge columns, and everything when a chunk would
 // cross the field's x extent, are copied element by element with the ghost rules.
 constexpr int T4X = 32, T4Y = 16, T4R = 4, T4ROWS = T4Y + 2, T4LD = 40;
-constexpr int Z4CH = 32;  // z planes per block of the FP32 kernel (16 measured slower at 256^3)
 constexpr int T4SLOTS = 2 * T4ROWS * 10;  // components x rows x (8 chunks + 2 edges)
 
 __device__ __forceinline__ int ghost_index(int gi, int m, int lo_neumann, int hi_neumann) {
@@ -242,7 +261,7 @@ struct StencilCoef32 {
 template <int MODE, bool NORM, bool RW>
 __global__ void __launch_bounds__(T4X* T4Y / T4R)
     stencil4_kernel(Geom g, StencilCoef32 coef, const float* __restrict__ x, float* __restrict__ y,
-                    const float* __restrict__ f, double* __restrict__ sumsq) {
+                    const float* __restrict__ f, double* __restrict__ sumsq, int zch) {
   constexpr int DIST = 3, NBUF = DIST + 2;
   constexpr int NT = T4X * T4Y / T4R;  // 128 threads
   __shared__ __align__(16) float sbuf[NBUF][2][T4ROWS][T4LD];
@@ -251,8 +270,8 @@ __global__ void __launch_bounds__(T4X* T4Y / T4R)
   const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * T4X + tx;
   const int x0 = blockIdx.x * T4X, y0 = blockIdx.y * T4Y;
   const int i = x0 + tx;
-  const int l0 = blockIdx.z * Z4CH;
-  const int l1 = min(l0 + Z4CH, g.mz);
+  const int l0 = blockIdx.z * zch;
+  const int l1 = min(l0 + zch, g.mz);
   const int64_t plane = (int64_t)g.mx * g.my;
   const bool xn0 = g.face[0] == HELM6_NEUMANN, xn1 = g.face[1] == HELM6_NEUMANN;
   const bool yn0 = g.face[2] == HELM6_NEUMANN, yn1 = g.face[3] == HELM6_NEUMANN;
@@ -450,16 +469,21 @@ __global__ void __launch_bounds__(T4X* T4Y / T4R)
 
 int stencil_blocks(const Geom& g) {
   // the larger of the two kernels' grids (FP64: 32 x 8 tiles, FP32: 32 x 16 tiles)
-  return ((g.mx + TX - 1) / TX) * ((g.my + TY - 1) / TY) * ((g.mz + ZCH - 1) / ZCH);
+  const int t8 = ((g.mx + TX - 1) / TX) * ((g.my + TY - 1) / TY), t16 = ((g.mx + T4X - 1) / T4X) * ((g.my + T4Y - 1) / T4Y);
+  const int z8 = z_chunk(t8, g.mz, ZB64), z16 = z_chunk(t16, g.mz, ZB32);
+  return std::max(t8 * ((g.mz + z8 - 1) / z8), t16 * ((g.mz + z16 - 1) / z16));
 }
 
 template <typename T>
 void launch_stencil(const Geom& g, const StencilCoef& c, const T* x, T* y, const T* f, T* r,
-                    int mode, double* sumsq, int* nblk, cudaStream_t s) {
+                    int mode, double* sumsq, int* nblk, cudaStream_t s, int share) {
   (void)r;
   if (sizeof(T) == 4) {
     dim3 block(T4X, T4Y / T4R);
-    dim3 grid((g.mx + T4X - 1) / T4X, (g.my + T4Y - 1) / T4Y, (g.mz + Z4CH - 1) / Z4CH);
+    dim3 grid((g.mx + T4X - 1) / T4X, (g.my + T4Y - 1) / T4Y);
+    // (a norm's partial sums follow the blocks: the same for every caller)
+    const int zch = z_chunk((int)(grid.x * grid.y), g.mz, ZB32, sumsq ? 1 : share);
+    grid.z = (g.mz + zch - 1) / zch;
     if (nblk) *nblk = (int)(grid.x * grid.y * grid.z);
     note_launch();
     const float* xf = (const float*)x;
@@ -479,9 +503,9 @@ void launch_stencil(const Geom& g, const StencilCoef& c, const T* x, T* y, const
 #define HELM6_S4(M, N)                                                                   \
   do {                                                                                   \
     if (rw)                                                                              \
-      stencil4_kernel<M, N, true><<<grid, block, 0, s>>>(g, c32, xf, yf, ff, N ? sumsq : nullptr);  \
+      stencil4_kernel<M, N, true><<<grid, block, 0, s>>>(g, c32, xf, yf, ff, N ? sumsq : nullptr, zch);  \
     else                                                                                 \
-      stencil4_kernel<M, N, false><<<grid, block, 0, s>>>(g, c32, xf, yf, ff, N ? sumsq : nullptr); \
+      stencil4_kernel<M, N, false><<<grid, block, 0, s>>>(g, c32, xf, yf, ff, N ? sumsq : nullptr, zch); \
   } while (0)
     if (mode == 0 && !nrm)
       HELM6_S4(0, false);
@@ -497,7 +521,9 @@ void launch_stencil(const Geom& g, const StencilCoef& c, const T* x, T* y, const
     return;
   }
   dim3 block(TX, TY);
-  dim3 grid((g.mx + TX - 1) / TX, (g.my + TY - 1) / TY, (g.mz + ZCH - 1) / ZCH);
+  dim3 grid((g.mx + TX - 1) / TX, (g.my + TY - 1) / TY);
+  const int zch = z_chunk((int)(grid.x * grid.y), g.mz, ZB64);
+  grid.z = (g.mz + zch - 1) / zch;
   if (nblk) *nblk = (int)(grid.x * grid.y * grid.z);
   note_launch();
   const bool nrm = sumsq != nullptr;
@@ -506,9 +532,9 @@ void launch_stencil(const Geom& g, const StencilCoef& c, const T* x, T* y, const
 #define HELM6_SG(M, N)                                                                        \
   do {                                                                                        \
     if (rw)                                                                                   \
-      stencil_kernel<T, M, N, true><<<grid, block, 0, s>>>(g, c, x, y, f, N ? sumsq : nullptr);  \
+      stencil_kernel<T, M, N, true><<<grid, block, 0, s>>>(g, c, x, y, f, N ? sumsq : nullptr, zch);  \
     else                                                                                      \
-      stencil_kernel<T, M, N, false><<<grid, block, 0, s>>>(g, c, x, y, f, N ? sumsq : nullptr); \
+      stencil_kernel<T, M, N, false><<<grid, block, 0, s>>>(g, c, x, y, f, N ? sumsq : nullptr, zch); \
   } while (0)
   if (mode == 0 && !nrm)
     HELM6_SG(0, false);
@@ -524,8 +550,8 @@ void launch_stencil(const Geom& g, const StencilCoef& c, const T* x, T* y, const
 }
 
 template void launch_stencil<float>(const Geom&, const StencilCoef&, const float*, float*,
-                                    const float*, float*, int, double*, int*, cudaStream_t);
+                                    const float*, float*, int, double*, int*, cudaStream_t, int);
 template void launch_stencil<double>(const Geom&, const StencilCoef&, const double*, double*,
-                                     const double*, double*, int, double*, int*, cudaStream_t);
+                                     const double*, double*, int, double*, int*, cudaStream_t, int);
 
 }  // namespace helm6
