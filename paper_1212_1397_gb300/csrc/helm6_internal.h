@@ -128,10 +128,12 @@ void launch_xform_tc(const float* in, float* out, const uint8_t* W, int M_total,
 // (m x m) as digit planes, and the same for symmetric (fold) bases over half the points.
 struct X64Basis {
   uint8_t* dev = nullptr;  // digit planes (device)
+  size_t bytes = 0;
   int m = 0, fold = 0, nk = 0, nch = 0, gcols = 0, ngroups = 0, eb = 0;
 };
-void x64_basis(int n, int lo, int hi, bool inverse, std::vector<double>& B);
-bool x64_prepare(const std::vector<double>& B, int m, bool fold, X64Basis& h, std::vector<uint8_t>& out);
+X64Basis x64_plan(int n, int lo, int hi);
+void x64_trig(int n, int lo, int hi, std::vector<double>& trig);
+void launch_x64_digits(int n, int lo, int hi, int inverse, X64Basis& h, const double* trig, int* over, cudaStream_t s);
 int x64_configure();
 // out(row, p) = sum_k in(row, k) B(p, k): rows of pitch ldin; transposed and row-major outputs
 // as launch_xform_tc; *err is set if a bounded wait timed out.

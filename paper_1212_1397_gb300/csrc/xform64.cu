@@ -663,113 +663,116 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(X_THREADS, 1) xform6
 
 int round32(int n) { return ((n + 31) / 32) * 32; }
 
-// FP16 bits of the integers -128 .. 128.
-struct HalfInts {
-  uint16_t bits[257];
-  HalfInts() {
-    for (int v = -128; v <= 128; ++v) {
-      const int a = std::abs(v);
-      int e = 0;
-      while ((a >> (e + 1)) != 0) ++e;
-      bits[v + 128] = a == 0 ? 0 : (uint16_t)((v < 0 ? 0x8000 : 0) | ((e + 15) << 10) | ((a << (10 - e)) & 0x3ff));
+// One axis' closed-form eigenbasis (the layouts and normalisation of the dense bases): entry
+// (node l, mode j) is trig[l j mod 2 D], every angle exactly reduced.
+struct X64Axis {
+  int N, m, D;           // intervals, unknowns, half period of the table
+  int nlo, nhi, inverse;
+  double sc;             // 2 / N
+};
+
+__device__ __forceinline__ double basis_entry(const X64Axis& a, const double* trig, int p, int k) {
+  // inverse: B(p, k) = V(node p, mode k); forward: B(p, k) = W(mode p, node k)
+  const int node = a.inverse ? p : k, mode = a.inverse ? k : p;
+  const bool quarter = a.nlo != a.nhi;
+  const int64_t l = a.nlo ? node : node + 1;
+  const int64_t j = quarter ? 2 * (mode + 1) - 1 : (a.nlo ? mode : mode + 1);
+  const double v = trig[(l * j) % (2 * a.D)];
+  if (a.inverse) return v;
+  double w = 1.0;
+  if (a.nlo && a.nhi && (j == 0 || j == a.N)) w *= 0.5;
+  if ((a.nlo && l == 0) || (a.nhi && l == a.N)) w *= 0.5;
+  return a.sc * w * v;
+}
+
+// Digit planes of one column (mode or node p) per block, in the transform kernel's layout.  *over is
+// set when an accumulator could leave the integers that FP32 holds exactly: level l sums the basis
+// digits 0..l times data digits of at most 128.
+__global__ void __launch_bounds__(128) x64_digits_kernel(X64Axis a, X64Basis h, const double* __restrict__ trig,
+                                                         double scale, int* over) {
+  __shared__ int ssum;
+  const int g = blockIdx.x / h.gcols, c = blockIdx.x % h.gcols, half = h.gcols / 2;
+  const int odd = h.fold && g >= h.nch ? 1 : 0, ch = g - odd * h.nch;
+  const int p = h.fold ? 2 * (ch * h.gcols + c) + odd : ch * h.gcols + c;
+  const int K = a.m, Kf = h.fold ? (K + 1) / 2 : K;
+  const size_t plane = (size_t)h.gcols * X_KT, stage = DG * plane;
+  if (threadIdx.x == 0) ssum = 0;
+  __syncthreads();
+  int sum = 0;
+  for (int k = threadIdx.x; k < h.nk * X_KT; k += blockDim.x) {
+    double b = 0.0;  // padding modes and points
+    if (p < a.m && k < Kf && !(odd && 2 * k == K - 1)) b = basis_entry(a, trig, p, k);
+    int64_t x = __double2ll_rn(b * scale);
+    uint8_t* o = h.dev + (((size_t)g * h.nk + k / X_KT) * 2 + c / half) * stage +
+                 (size_t)((k % X_KT) / 8) * half * 16 + (size_t)(c % half) * 16 + (size_t)(k % 8) * 2;
+    for (int d = DG - 1; d >= 0; --d) {
+      const int v = d > 0 ? (int)((x + 128) & 255) - 128 : (int)x;
+      x = (x - v) >> 8;
+      sum += abs(v);
+      *(__half*)(o + (size_t)d * plane) = __int2half_rn(v);
     }
   }
-};
+  atomicAdd(&ssum, sum);
+  __syncthreads();
+  if (threadIdx.x == 0 && 128ll * ssum > 1ll << 24) atomicExch(over, 1);
+}
 
 }  // namespace
 
-// Closed-form 1D eigenbasis of an axis (the layouts and normalisation of the dense bases), every
-// entry from an exactly reduced angle: V[p][j] = trig(pi a_p b_j / D) with integers a, b.
-void x64_basis(int n, int lo, int hi, bool inverse, std::vector<double>& B) {
+// Sizes of the basis planes of an axis with n interior nodes.
+X64Basis x64_plan(int n, int lo, int hi) {
   const bool nlo = lo != HELM6_DIRICHLET, nhi = hi != HELM6_DIRICHLET;
-  const int N = n + 1, m = n + (nlo ? 1 : 0) + (nhi ? 1 : 0);
-  const bool quarter = nlo != nhi;
-  const int D = quarter ? 2 * N : N;
-  std::vector<double> trig(2 * (size_t)D);
-  for (int t = 0; t < 2 * D; ++t) {
-    // sin or cos of pi t / D from the first octant
-    int q = t;
-    double sg = 1.0;
-    if (nlo) {
-      if (q > D) q = 2 * D - q;                       // cos(2 pi - x) = cos x
-      if (2 * q > D) { q = D - q; sg = -1.0; }        // cos(pi - x) = -cos x
-      trig[t] = 2 * q == D ? 0.0 : sg * (4 * q <= D ? std::cos(M_PI * q / D) : std::sin(M_PI * (D - 2 * q) / (2.0 * D)));
-    } else {
-      if (q >= D) { q -= D; sg = -1.0; }              // sin(x + pi) = -sin x
-      if (2 * q > D) q = D - q;                       // sin(pi - x) = sin x
-      trig[t] = sg * (4 * q <= D ? std::sin(M_PI * q / D) : std::cos(M_PI * (D - 2 * q) / (2.0 * D)));
-    }
-  }
-  B.assign((size_t)m * m, 0.0);
-  const double sc = 2.0 / N;
-  for (int p = 0; p < m; ++p)
-    for (int jj = 0; jj < m; ++jj) {
-      const int64_t l = nlo ? p : p + 1;                                    // node
-      const int64_t j = quarter ? 2 * (jj + 1) - 1 : (nlo ? jj : jj + 1);  // mode
-      const double v = trig[(size_t)((l * j) % (2 * D))];
-      if (inverse) {
-        B[(size_t)p * m + jj] = v;
-      } else {
-        double w = 1.0;
-        if (nlo && nhi && (j == 0 || j == N)) w *= 0.5;
-        if ((nlo && l == 0) || (nhi && l == N)) w *= 0.5;
-        B[(size_t)jj * m + p] = sc * w * v;
-      }
-    }
-}
-
-// Digit planes of the basis B (m x m, row-major) in the kernel's layout; false when the axis is
-// out of the kernel's range (an accumulator could leave the integers FP32 holds exactly).
-bool x64_prepare(const std::vector<double>& B, int m, bool fold, X64Basis& h, std::vector<uint8_t>& out) {
-  const int P = m, K = m, Kf = fold ? (K + 1) / 2 : K;
-  const int cnt = fold ? (P + 1) / 2 : P;  // modes of the larger parity
-  h.m = m;
-  h.fold = fold;
+  X64Basis h;
+  h.m = n + (nlo ? 1 : 0) + (nhi ? 1 : 0);
+  h.fold = nlo == nhi;
+  const int Kf = h.fold ? (h.m + 1) / 2 : h.m, cnt = Kf;  // points of a product; modes of the larger parity
   h.nk = (Kf + X_KT - 1) / X_KT;
   h.nch = (cnt + X_NMAX - 1) / X_NMAX;
   h.gcols = round32((cnt + h.nch - 1) / h.nch);
-  h.ngroups = (fold && P > 1 ? 2 : 1) * h.nch;
-  double mx = 0.0;
-  for (double b : B) mx = std::max(mx, std::fabs(b));
-  h.eb = (int)std::ceil(std::log2(mx));
-  if (std::ldexp(1.0, h.eb) < mx) ++h.eb;
-  // per CTA of a pair: half of the group's modes
-  const size_t plane = (size_t)h.gcols * X_KT, stage = DG * plane;
-  const int half = h.gcols / 2;
-  out.assign((size_t)h.ngroups * h.nk * 2 * stage, 0);
-  static const HalfInts hi16;
-  const double scale = std::ldexp(1.0, 55 - h.eb);
-  for (int g = 0; g < h.ngroups; ++g) {
-    const int odd = fold && g >= h.nch ? 1 : 0, ch = g - odd * h.nch;
-    for (int c = 0; c < h.gcols; ++c) {
-      const int p = fold ? 2 * (ch * h.gcols + c) + odd : ch * h.gcols + c;
-      if (p >= P) continue;
-      int64_t sum[DG] = {};
-      for (int k = 0; k < Kf; ++k) {
-        double b = B[(size_t)p * K + k];
-        if (odd && 2 * k == K - 1) b = 0.0;  // the middle point of an antisymmetric mode
-        int64_t x = std::llrint(b * scale);
-        for (int d = DG - 1; d >= 0; --d) {
-          int v;
-          if (d > 0) {
-            v = (int)((x + 128) & 255) - 128;
-            x = (x - v) >> 8;
-          } else {
-            v = (int)x;
-          }
-          sum[d] += std::abs(v);
-          const uint16_t hb = hi16.bits[v + 128];
-          const size_t o = (((size_t)g * h.nk + k / X_KT) * 2 + c / half) * stage + (size_t)d * plane +
-                           (size_t)((k % X_KT) / 8) * half * 16 + (size_t)(c % half) * 16 + (size_t)(k % 8) * 2;
-          std::memcpy(out.data() + o, &hb, 2);
-        }
-      }
-      int64_t lvl = 0;  // level l sums the basis digits 0..l, each times a data digit <= 128
-      for (int d = 0; d < DG; ++d) lvl += 128 * sum[d];
-      if (lvl > (int64_t)1 << 24) return false;
+  h.ngroups = (h.fold && h.m > 1 ? 2 : 1) * h.nch;
+  h.bytes = (size_t)h.ngroups * h.nk * 2 * DG * h.gcols * X_KT;
+  return h;
+}
+
+// The trigonometric table of an axis: sin or cos of pi t / D, t < 2 D, from the first octant.
+void x64_trig(int n, int lo, int hi, std::vector<double>& trig) {
+  const bool nlo = lo != HELM6_DIRICHLET, nhi = hi != HELM6_DIRICHLET;
+  const int N = n + 1, D = nlo != nhi ? 2 * N : N;
+  trig.resize(2 * (size_t)D);
+  for (int t = 0; t < 2 * D; ++t) {
+    int q = t;
+    double sg = 1.0;
+    if (nlo) {
+      if (q > D) q = 2 * D - q;                 // cos(2 pi - x) = cos x
+      if (2 * q > D) { q = D - q; sg = -1.0; }  // cos(pi - x) = -cos x
+      trig[t] = 2 * q == D ? 0.0 : sg * (4 * q <= D ? std::cos(M_PI * q / D) : std::sin(M_PI * (D - 2 * q) / (2.0 * D)));
+    } else {
+      if (q >= D) { q -= D; sg = -1.0; }        // sin(x + pi) = -sin x
+      if (2 * q > D) q = D - q;                 // sin(pi - x) = sin x
+      trig[t] = sg * (4 * q <= D ? std::sin(M_PI * q / D) : std::cos(M_PI * (D - 2 * q) / (2.0 * D)));
     }
   }
-  return true;
+}
+
+// Fill the planes at h.dev of the forward or inverse basis (stream-ordered); *over (device) is set when
+// the axis is out of the kernel's range.
+void launch_x64_digits(int n, int lo, int hi, int inverse, X64Basis& h, const double* trig, int* over, cudaStream_t s) {
+  const bool nlo = lo != HELM6_DIRICHLET, nhi = hi != HELM6_DIRICHLET;
+  X64Axis a;
+  a.N = n + 1;
+  a.m = h.m;
+  a.nlo = nlo;
+  a.nhi = nhi;
+  a.D = nlo != nhi ? 2 * a.N : a.N;
+  a.inverse = inverse;
+  a.sc = 2.0 / a.N;
+  // |B| <= 1 (inverse) or 2 / N
+  h.eb = 0;
+  if (!inverse)
+    while (std::ldexp(1.0, h.eb - 1) >= a.sc) --h.eb;
+  if (!inverse && a.sc > 1.0) h.eb = 1;
+  note_launch();
+  x64_digits_kernel<<<h.ngroups * h.gcols, 128, 0, s>>>(a, h, trig, std::ldexp(1.0, 55 - h.eb), over);
 }
 
 int x64_configure() {
