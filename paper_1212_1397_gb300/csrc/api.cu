@@ -41,6 +41,7 @@ struct helm6_ctx {
   int ndot = 0;        // blocks of the Gram-Schmidt reduction kernel
   double *Hr = nullptr, *Tm = nullptr, *red = nullptr, *coefv = nullptr, *qv = nullptr;
   int* brk = nullptr;
+  unsigned* step_count = nullptr;  // blocks of a step kernel that have reduced their column
   double* u64 = nullptr;
   float* u32 = nullptr;
   double last_beta = 0;  // ||F - A U|| after the last FP64 residual
@@ -72,8 +73,8 @@ struct helm6_ctx {
   __half* V16 = nullptr;  // FP16 basis (HELM6_BASIS_F16) in place of V32, holding vscale V_i
   double vscale = 1.0;
   // small device arrays
-  double *partial = nullptr, *spart = nullptr, *H = nullptr, *cs = nullptr, *sn = nullptr,
-         *gv = nullptr, *yv = nullptr, *h2 = nullptr, *scal = nullptr;
+  double *partial = nullptr, *spart = nullptr, *H = nullptr, *Qr = nullptr,
+         *gv = nullptr, *yv = nullptr, *scal = nullptr;
   int* status = nullptr;
   double* pinned = nullptr;  // host-pinned readback slots
   cudaEvent_t step_ev[2] = {nullptr, nullptr};  // Arnoldi step completion (alternating)
@@ -477,6 +478,12 @@ int residual64(helm6_ctx* c, double* beta) {
 
 void push_hist(helm6_stats* st, double v);
 
+// The step algebra's device arrays.
+StepMem step_mem(const helm6_ctx* c, bool flexible) {
+  return StepMem{c->Hr, c->H, c->mrest + 1, flexible ? c->Tm : nullptr, c->mrest, c->Qr, c->gv, c->coefv,
+                 c->scal + 2, c->brk, c->step_count};
+}
+
 // One Arnoldi cycle with delayed classical Gram-Schmidt.  On entry u holds the starting
 // residual (any scale; g_0 = ||u||).  Step j applies the preconditioner and the operator
 // to u_j, reduces V^H u_j, V^H w, ||u_j||^2 and u_j^H w in one pass, completes column j-1
@@ -540,9 +547,7 @@ int arnoldi(helm6_ctx* c, TV* V, T* Z, T* u, T* w, T* zt, int m, double abs_tol,
     launch_dcgs_dot<T, TV>(V, vs, j, u, full ? w : nullptr, N, c->partial, c->ndot, vsc, s);
     prof_stop(c, HELM6_PH_DOT, e, vbb * j + vb * (full ? 2 : 1));
     e = prof_start(c);
-    launch_reduce_cols(c->partial, c->ndot, 4 * j + 3, c->red, 0, s);
-    launch_dcgs_step(j, full ? 1 : 0, c->red, c->Hr, c->H, ldh, flexible ? c->Tm : nullptr, c->mrest, c->cs, c->sn,
-                     c->gv, c->coefv, c->scal + 2, c->brk, s);
+    launch_dcgs_step(j, full ? 1 : 0, c->partial, c->ndot, c->red, step_mem(c, flexible), nullptr, m, 0, s);
     prof_stop(c, HELM6_PH_SMALL, e, 8.0 * c->ndot * (4 * j + 3));
     CK(cudaMemcpyAsync(&c->pinned[8 + (j & 1)], c->scal + 2, sizeof(double), cudaMemcpyDeviceToHost, s));
     CK(cudaMemcpyAsync(&c->pinned[10 + (j & 1)], c->brk, sizeof(int), cudaMemcpyDeviceToHost, s));
@@ -613,7 +618,7 @@ int arnoldi(helm6_ctx* c, TV* V, T* Z, T* u, T* w, T* zt, int m, double abs_tol,
     }
   }
   *kout = k;
-  if (k > 0) launch_backsolve(c->H, ldh, k, c->gv, c->yv, s);
+  if (k > 0) launch_ls_solve(c->H, ldh, k, c->gv, c->yv, flexible ? c->Tm : nullptr, c->mrest, c->qv, s);
   CK(cudaGetLastError());
   return HELM6_OK;
 }
@@ -664,7 +669,6 @@ int solve_fp64(helm6_ctx* c, double normF, double tol, int m, int maxit, helm6_s
     iters += k;
     if (k > 0) {
       if (flex) {
-        launch_tri_mul(c->Tm, c->mrest, k, c->yv, c->qv, c->stream);
         launch_lincomb<double, double>(c->Z64, 2 * c->g.N, k, c->qv, 1.0, c->U64, c->g.N, 1, c->stream);
       } else {
         launch_lincomb<double, double>(c->V64, 2 * c->g.N, k, c->yv, 1.0, c->E64, c->g.N, 0, c->stream);
@@ -751,7 +755,6 @@ int solve_mixed(helm6_ctx* c, double normF, double tol, int m, int maxit, helm6_
     fix_hist(st, h0, beta / normF);
     iters += k;
     bool apply = k > 0;
-    if (k > 0) launch_tri_mul(c->Tm, c->mrest, k, c->yv, c->qv, c->stream);
     if (use_cnn) {
       // A network that returns NaN/Inf (corrupt weights, an input far outside its training
       // range) makes the cycle's estimate or coefficients non-finite.  Then U64 keeps the
@@ -899,20 +902,17 @@ int append_solve_graph(helm6_ctx* c, TV* V, cudaGraph_t G, int m, int share) {
         launch_stencil<float>(c->g, c->coef, zj, c->w32, nullptr, nullptr, 0, nullptr, nullptr, s, share);
       }
       launch_dcgs_dot<float, TV>(V, vs, j, c->u32, full ? c->w32 : nullptr, N, c->partial, c->ndot, vsc, s);
-      launch_reduce_cols(c->partial, c->ndot, 4 * j + 3, c->red, 0, s);
-      launch_dcgs_step(j, full ? 1 : 0, c->red, c->Hr, c->H, ldh, c->Tm, c->mrest, c->cs, c->sn, c->gv, c->coefv,
-                       c->scal + 2, c->brk, s);
+      launch_dcgs_step(j, full ? 1 : 0, c->partial, c->ndot, c->red, step_mem(c, true), gc, m,
+                       j < m ? ha.h[j + 1] : ha.h[j], s);
       if (full)
         launch_dcgs_update<float, TV>(V, vs, j, c->u32, c->w32, V + (int64_t)j * vs, N, c->coefv, c->ncgs, vsc, s);
-      launch_gctl_step(gc, j, m, c->scal + 2, c->brk, j < m ? ha.h[j + 1] : ha.h[j], s);
     });
     if (rc) return rc;
     prev = ifn;
   }
   cudaGraphNode_t post;
   return add_segment(c, body, &prev, 1, &post, [&](cudaStream_t s) {
-    launch_backsolve(c->H, ldh, 0, c->gv, c->yv, s, &gc->k);
-    launch_tri_mul(c->Tm, c->mrest, 0, c->yv, c->qv, s, &gc->k);
+    launch_ls_solve(c->H, ldh, 0, c->gv, c->yv, c->Tm, c->mrest, c->qv, s, &gc->k);
     launch_lincomb<float, double>(c->Z32, vs, 0, c->qv, 1.0, c->U64, N, 1, s, &gc->k, &gc->beta);
     enqueue_residual_dev(c, s);
     launch_gctl_residual(gc, c->scal, c->status, c->tcerr, 0, hw, s);
@@ -1516,13 +1516,14 @@ int helm6_create(helm6_ctx** out, int n, double h, helm6_c64 k, const int faces[
       (rc = dalloc(c, &c->coefv, ncol)) || (rc = dalloc(c, &c->Hr, (size_t)2 * (m + 1) * m)) ||
       (rc = dalloc(c, &c->Tm, (size_t)2 * m * m)) || (rc = dalloc(c, &c->qv, (size_t)2 * (m + 1))) ||
       (rc = dalloc(c, &c->brk, 1)) || (rc = dalloc(c, &c->spart, (size_t)c->nsten)) ||
-      (rc = dalloc(c, &c->H, (size_t)2 * (m + 1) * m)) || (rc = dalloc(c, &c->cs, (size_t)2 * (m + 1))) ||
-      (rc = dalloc(c, &c->sn, (size_t)2 * (m + 1))) || (rc = dalloc(c, &c->gv, (size_t)2 * (m + 1))) ||
-      (rc = dalloc(c, &c->yv, (size_t)2 * (m + 1))) || (rc = dalloc(c, &c->h2, (size_t)2 * (m + 1))) ||
+      (rc = dalloc(c, &c->H, (size_t)2 * (m + 1) * m)) || (rc = dalloc(c, &c->Qr, (size_t)2 * (m + 1) * (m + 1))) ||
+      (rc = dalloc(c, &c->gv, (size_t)2 * (m + 1))) || (rc = dalloc(c, &c->yv, (size_t)2 * (m + 1))) ||
+      (rc = dalloc(c, &c->step_count, 1)) ||
       (rc = dalloc(c, &c->scal, 8)) || (rc = dalloc(c, &c->status, 1)))
     return fail(rc);
   if ((rc = dalloc(c, &c->tcerr, 1))) return fail(rc);
-  if (cudaMemset(c->tcerr, 0, sizeof(int)) != cudaSuccess) return fail(HELM6_ERR_CUDA);
+  if (cudaMemset(c->tcerr, 0, sizeof(int)) != cudaSuccess || cudaMemset(c->step_count, 0, sizeof(unsigned)) != cudaSuccess)
+    return fail(HELM6_ERR_CUDA);
   if (use_tc) {
     if (tc_configure() != HELM6_OK) return fail(HELM6_ERR_CUDA);
     std::vector<uint8_t> t;

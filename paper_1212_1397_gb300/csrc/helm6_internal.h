@@ -198,8 +198,6 @@ template <typename T>
 void launch_fft_axis(const FftDev& f, int axis, int inv, const Geom& g, const T* in, T* out, cudaStream_t s);
 
 // BLAS-1 style kernels on planar complex vectors of N points.
-void launch_reduce_cols(const double* partial, int nblocks, int ncols, double* out, int accumulate,
-                        cudaStream_t s);  // out[i] (+)= sum_b partial[b][i], complex double
 template <typename T>
 void launch_sumsq(const T* x, int64_t N, double* partial, int nblocks, cudaStream_t s);
 template <typename T>
@@ -223,16 +221,10 @@ void launch_caller_to_planar(const Geom& g, int xaxis, const double* zin, double
 void launch_planar_to_caller(const Geom& g, int xaxis, const double* in, double* zout, cudaStream_t s);
 void launch_reduce_sum(const double* partial, int n, double* out, cudaStream_t s);  // one double
 
-// Givens update of Hessenberg column j on the device (single thread, FP64):
-// applies the j previous rotations to H[:, j], makes rotation j, updates g; writes
-// |g_{j+1}| to *res.  H column-major with leading dimension ldh, complex double.
-void launch_givens(double* H, int ldh, int j, double* cs, double* sn, double* g, double* res,
-                   cudaStream_t s);
-// H[j+1, j] = sqrt(*sumsq); inv = 1/that (0 if zero).
-void launch_set_subdiag(double* H, int ldh, int j, const double* sumsq, double* inv, cudaStream_t s);
-// Solve the j x j upper triangular system R y = g (complex double) on the device.
-void launch_backsolve(const double* H, int ldh, int j, const double* g, double* y, cudaStream_t s,
-                      const int* j_dev = nullptr);
+// y = R^-1 g for the j x j upper triangular R (complex double) on the device and, with T, q = T y
+// (T upper triangular, leading dimension ldt); j_dev (nullable): j is read on the device.
+void launch_ls_solve(const double* R, int ldh, int j, const double* g, double* y, const double* T, int ldt, double* q,
+                     cudaStream_t s, const int* j_dev = nullptr);
 
 // Compact right side for Gaussian sources (FP64, complex128 interleaved output F).
 // centers: host nsrc*3, amps: host nsrc*2 (re, im); noise: device complex128 or nullptr.
@@ -254,15 +246,12 @@ template <typename TI, typename TO>
 void launch_axpy(const TI* x, TO* y, int64_t N, double alpha, cudaStream_t s);
 // y = a y + b x (planar FP64, 2N reals).
 void launch_axpby(const double* x, double* y, int64_t N, double a, double b, cudaStream_t s);
-// p[0] = re, p[1] = im on the device (stream-ordered).
-void launch_set_complex(double* p, double re, double im, cudaStream_t s);
-
 // Arnoldi by delayed classical Gram-Schmidt (one reduction and one update pass per step):
 //   launch_dcgs_dot:    block partials of V_i^H u, V_i^H w (i < count), ||u||^2, u^H w
 //                       (w may be null: the last step of a cycle has no new vector)
-//   launch_dcgs_step:   FP64 small algebra of step j (see krylov.cu)
+//   launch_dcgs_step:   sums of the partials, FP64 small algebra of step j and, in device-driven
+//                       solves (gc), the decision whether step j + 1 runs (see krylov.cu)
 //   launch_dcgs_update: v_out = (u - V s)/alpha,  u = (w - V t - v_out c)/alpha
-//   launch_tri_mul:     q = T y for the flexible solution update
 template <typename T>
 int cgs_blocks(int64_t N);
 int dot_blocks();
@@ -274,10 +263,19 @@ void launch_dcgs_dot(const TV* V, int64_t vs, int count, const T* u, const T* w,
 template <typename T, typename TV>
 void launch_dcgs_update(const TV* V, int64_t vs, int count, T* u, const T* w, TV* v_out, int64_t N,
                         const double* coef, int nblocks, double vscale, cudaStream_t s);
-void launch_dcgs_step(int j, int has_w, const double* red, double* Hr, double* R, int ldh, double* T, int ldt,
-                      double* cs, double* sn, double* g, double* coef, double* est, int* brk, cudaStream_t s);
-void launch_tri_mul(const double* T, int ldt, int k, const double* y, double* q, cudaStream_t s,
-                    const int* k_dev = nullptr);
+struct StepMem {
+  double *Hr, *R;      // raw and rotated Hessenberg matrix, leading dimension ldh
+  int ldh;
+  double* T;           // z_l = sum_i T[i, l] z~_i (flexible), leading dimension ldt; or null
+  int ldt;
+  double* Q;           // the product of the rotations, column-major, leading dimension ldh
+  double *g, *coef, *est;
+  int* brk;
+  unsigned* count;     // zero between launches
+};
+struct GraphCtl;
+void launch_dcgs_step(int j, int has_w, const double* partial, int nblocks, double* red, const StepMem& a, GraphCtl* gc,
+                      int m, cudaGraphConditionalHandle next, cudaStream_t s);
 
 // Learned second preconditioner stage (cnn.cu).  theta: HELM6_CNN_NPARAMS master
 // parameters; wf / wb: BF16-rounded taps of every layer in the forward layout
@@ -322,9 +320,6 @@ struct StepHandles {
   cudaGraphConditionalHandle h[65];
 };
 void launch_gctl_cycle(GraphCtl* g, const StepHandles& ha, int m, cudaStream_t s);
-void launch_gctl_step(GraphCtl* g, int j, int m, const double* est, const int* brk, cudaGraphConditionalHandle next,
-                      cudaStream_t s);
-
 // Kernels launched by the library so far (process-wide counter, for measurement).
 void note_launch(int n = 1);
 long long launch_total();

@@ -33,20 +33,6 @@ __device__ __forceinline__ double block_sum(double v, double* sh) {
   return v;
 }
 
-// out[c] (+)= sum_b partial[b*ncols + c]; also adds into accum[c] when accum != nullptr.
-__global__ void reduce_cols_kernel(const double* __restrict__ partial, int nblocks, int ncols,
-                                   double* __restrict__ out, int accumulate, double* accum) {
-  __shared__ double sh[RB / 32];
-  const int c = blockIdx.x;
-  double v = 0.0;
-  for (int b = threadIdx.x; b < nblocks; b += blockDim.x) v += partial[(int64_t)b * ncols + c];
-  v = block_sum(v, sh);
-  if (threadIdx.x == 0) {
-    out[c] = accumulate ? out[c] + v : v;
-    if (accum) accum[c] += v;
-  }
-}
-
 template <typename T>
 __global__ void __launch_bounds__(RB) sumsq_kernel(const T* __restrict__ x, int64_t N,
                                                    double* __restrict__ partial) {
@@ -542,279 +528,299 @@ __global__ void __launch_bounds__(RB) dcgs_update_kernel(const TV* __restrict__ 
   }
 }
 
-// ---- GMRES least squares (FP64, one thread) ----
+// ---- FP64 small algebra ----
+// An FP64 instruction of one warp takes its scheduler 64 cycles on GB300 whether one lane works or
+// 32 do, so the kernels below spread every product over lanes and warps and keep the serial part
+// to a few dozen instructions.
 struct zc {
   double re, im;
 };
 __device__ __forceinline__ zc ld(const double* p) { return zc{p[0], p[1]}; }
 __device__ __forceinline__ void st(double* p, zc v) { p[0] = v.re; p[1] = v.im; }
 __device__ __forceinline__ zc zmul(zc a, zc b) { return zc{a.re * b.re - a.im * b.im, a.re * b.im + a.im * b.re}; }
-__device__ __forceinline__ zc zadd(zc a, zc b) { return zc{a.re + b.re, a.im + b.im}; }
-__device__ __forceinline__ double zabs(zc a) { return hypot(a.re, a.im); }
-
-// Rotation i acts on rows (i, i+1): [c s; -conj(s) c], c real (stored in cs[2i]), s complex.
-__global__ void givens_kernel(double* H, int ldh, int j, double* cs, double* sn, double* g, double* res) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  double* col = H + 2 * (int64_t)j * ldh;
-  for (int i = 0; i < j; ++i) {
-    const zc hi = ld(col + 2 * i), hn = ld(col + 2 * (i + 1));
-    const double c = cs[2 * i];
-    const zc s = ld(sn + 2 * i);
-    const zc t = zadd(zc{c * hi.re, c * hi.im}, zmul(s, hn));
-    const zc u = zadd(zmul(zc{-s.re, s.im}, hi), zc{c * hn.re, c * hn.im});  // -conj(s) hi + c hn
-    st(col + 2 * i, t);
-    st(col + 2 * (i + 1), u);
-  }
-  const zc a = ld(col + 2 * j), b = ld(col + 2 * (j + 1));
-  const double aa = zabs(a), bb = zabs(b);
-  const double den = hypot(aa, bb);
-  double c;
-  zc s;
-  if (den == 0.0) {
-    c = 1.0;
-    s = zc{0.0, 0.0};
-  } else if (aa == 0.0) {
-    c = 0.0;
-    s = zc{1.0, 0.0};
-  } else {
-    c = aa / den;
-    const zc ph = zc{a.re / aa, a.im / aa};
-    s = zmul(ph, zc{b.re / den, -b.im / den});
-  }
-  cs[2 * j] = c;
-  cs[2 * j + 1] = 0.0;
-  st(sn + 2 * j, s);
-  st(col + 2 * j, zadd(zc{c * a.re, c * a.im}, zmul(s, b)));
-  st(col + 2 * (j + 1), zc{0.0, 0.0});
-  const zc gj = ld(g + 2 * j);
-  st(g + 2 * (j + 1), zmul(zc{-s.re, s.im}, gj));
-  st(g + 2 * j, zc{c * gj.re, c * gj.im});
-  *res = zabs(ld(g + 2 * (j + 1)));
+__device__ __forceinline__ zc zfma(zc a, zc b, zc c) {
+  return zc{fma(a.re, b.re, fma(-a.im, b.im, c.re)), fma(a.re, b.im, fma(a.im, b.re, c.im))};
 }
 
+constexpr int STEP_MAXJ = 64;  // largest restart length (helm6_opts.max_restart <= 64)
+constexpr int STEP_W = RB / 32;
 
-// Small FP64 algebra of one delayed Gram-Schmidt Arnoldi step j (one thread).
-// red: reduced sums s_i = V_i^H u_j, t_i = V_i^H w (i < j), a = ||u_j||^2, b = u_j^H w.
+// One delayed Gram-Schmidt Arnoldi step j: column sums of the reduction's partials (block c sums
+// column c), then, in the block that finishes last, the step's algebra.
+// red: s_i = V_i^H u_j, t_i = V_i^H w (i < j), a = ||u_j||^2, b = u_j^H w.
 // u_j = V s + alpha v_j with alpha^2 = a - ||s||^2.
-//   * column j-1 of the raw Hessenberg Hr gets += s and subdiagonal alpha; it is copied to R
-//     and rotated (Givens), giving the residual estimate *est = |g_j| (j = 0: g_0 = alpha);
+//   * column j-1 of the raw Hessenberg Hr gets += s and subdiagonal alpha; its rotated form goes
+//     to R.  The rotations so far are kept as their product Q (row r reaches columns 0..r+1), so
+//     that the column is rotated by one matrix-vector product instead of j dependent rotations;
+//     the new rotation zeroes the subdiagonal and gives the residual estimate *est = |g_j|
+//     (j = 0: g_0 = alpha);
 //   * with w = A M^{-1} u_j (has_w): v_j^H w = (b - s^H t)/alpha = c_j, column j of Hr is
 //     ([t; c_j] - Hr[:, 0..j-1] s)/alpha, and T (z_l = sum_i T[i,l] z~_i) gets column
 //     (e_j - T s)/alpha;
 //   * coef = [s, t, c_j, 1/alpha] for the update pass v_j = (u - V s)/alpha,
-//     u_{j+1} = (w - V t - v_j c_j)/alpha.
+//     u_{j+1} = (w - V t - v_j c_j)/alpha;
+//   * gc (device-driven solves): iteration count, history, and whether step j + 1 runs.
 // *brk = 1 when alpha^2 <= 1e-28 a (u_j in the span of the basis: breakdown).
-constexpr int STEP_T = 128;   // threads of the step kernel
-constexpr int STEP_MAXJ = 64;  // largest restart length (helm6_opts.max_restart <= 64)
-
-// Sums of three doubles over the block; every thread receives them.
-__device__ __forceinline__ void block_sum3(double& a, double& b, double& c, double* sh) {
-  a = warp_sum(a);
-  b = warp_sum(b);
-  c = warp_sum(c);
-  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-  if (l == 0) {
-    sh[3 * w] = a;
-    sh[3 * w + 1] = b;
-    sh[3 * w + 2] = c;
-  }
-  __syncthreads();
-  a = b = c = 0.0;
-  for (int i = 0; i < STEP_T / 32; ++i) {
-    a += sh[3 * i];
-    b += sh[3 * i + 1];
-    c += sh[3 * i + 2];
-  }
-  __syncthreads();
-}
-
-// One block of STEP_T threads; the rotation sweep runs on thread 0 over shared-memory copies
-// of the column and of the previous rotations, the O(j^2) products warp per row.
-__global__ void __launch_bounds__(STEP_T) dcgs_step_kernel(int j, int has_w, const double* red, double* Hr, double* R,
-                                                           int ldh, double* T, int ldt, double* cs, double* sn,
-                                                           double* g, double* coef, double* est, int* brk) {
-  __shared__ double shr[3 * STEP_T / 32];
-  __shared__ double scol[2 * (STEP_MAXJ + 2)], scs[STEP_MAXJ + 1], ssn[2 * (STEP_MAXJ + 1)];
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const double* sv = red;
-  const double* tv = red + 2 * j;
-  const double a = red[4 * j];
-  const zc b = zc{red[4 * j + 1], red[4 * j + 2]};
-  double s2 = 0.0, pr = 0.0, pi = 0.0;
-  for (int i = tid; i < j; i += STEP_T) {
-    s2 += sv[2 * i] * sv[2 * i] + sv[2 * i + 1] * sv[2 * i + 1];
-    if (has_w) {
-      const zc q = zmul(zc{sv[2 * i], -sv[2 * i + 1]}, ld(tv + 2 * i));
-      pr += q.re;
-      pi += q.im;
-    }
-  }
-  block_sum3(s2, pr, pi, shr);
-  const double al2 = a - s2;
-  const bool bd = !(al2 > 1e-28 * fmax(a, 1e-300)) || !isfinite(al2);
-  const double al = bd ? 0.0 : sqrt(al2);
-  const double inv = bd ? 0.0 : 1.0 / al;
-  if (tid == 0) *brk = bd ? 1 : 0;
-  for (int i = tid; i < j; i += STEP_T) {
-    coef[2 * i] = sv[2 * i];
-    coef[2 * i + 1] = sv[2 * i + 1];
-    coef[2 * j + 2 * i] = tv[2 * i];
-    coef[2 * j + 2 * i + 1] = tv[2 * i + 1];
-  }
-  if (j >= 1) {
-    // lagged correction of column j - 1 and its subdiagonal
-    double* hc = Hr + 2 * (int64_t)(j - 1) * ldh;
-    for (int i = tid; i < j; i += STEP_T) {
-      hc[2 * i] += sv[2 * i];
-      hc[2 * i + 1] += sv[2 * i + 1];
-    }
+// One launch in place of three (column sums, algebra on one thread's rotations, control): 37 -> 14 us
+// per step at restart length 30, 22 -> 9 us on the small grids' first steps.
+__global__ void __launch_bounds__(RB) dcgs_step_kernel(int j, int has_w, const double* __restrict__ partial, int nblocks,
+                                                       double* red, StepMem a, GraphCtl* gc, int m,
+                                                       cudaGraphConditionalHandle next) {
+  __shared__ double sh[STEP_W];
+  __shared__ bool last;
+  const int ncols = 4 * j + 3, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  {
+    const int c = blockIdx.x;
+    double v = 0.0;
+    for (int b = tid; b < nblocks; b += RB) v += partial[(int64_t)b * ncols + c];
+    v = block_sum(v, sh);
     if (tid == 0) {
-      hc[2 * j] = al;
-      hc[2 * j + 1] = 0.0;
+      red[c] = v;
+      __threadfence();
+      last = atomicAdd(a.count, 1u) == (unsigned)ncols - 1u;
     }
     __syncthreads();
-    for (int r = tid; r <= 2 * j + 1; r += STEP_T) scol[r] = hc[r];
-    for (int i = tid; i < j - 1; i += STEP_T) {
-      scs[i] = cs[2 * i];
-      ssn[2 * i] = sn[2 * i];
-      ssn[2 * i + 1] = sn[2 * i + 1];
+    if (!last) return;
+    __threadfence();
+    if (tid == 0) *a.count = 0u;
+  }
+  // partial products of warp w: rows by lane, the columns w, w + 8, ...
+  __shared__ zc sp[3][STEP_W][STEP_MAXJ + 1];
+  __shared__ zc ss[STEP_MAXJ + 1], st_[STEP_MAXJ + 1], sh_[STEP_MAXJ + 1];  // s, t, corrected column j - 1
+  __shared__ zc srot[STEP_MAXJ + 1];
+  __shared__ double ssum[3], sal[3];  // ||s||^2, s^H t; alpha, 1 / alpha, breakdown
+  volatile double* vr = red;
+  const int ldh = a.ldh;
+  if (tid < j) {
+    const zc sv{vr[2 * tid], vr[2 * tid + 1]}, tv{vr[2 * j + 2 * tid], vr[2 * j + 2 * tid + 1]};
+    ss[tid] = sv;
+    st_[tid] = tv;
+    a.coef[2 * tid] = sv.re;
+    a.coef[2 * tid + 1] = sv.im;
+    a.coef[2 * j + 2 * tid] = tv.re;
+    a.coef[2 * j + 2 * tid + 1] = tv.im;
+    const zc h = ld(a.Hr + 2 * ((int64_t)(j - 1) * ldh + tid));
+    sh_[tid] = zc{h.re + sv.re, h.im + sv.im};
+  }
+  __syncthreads();
+  // ||s||^2 (warp 0), s^H t (warps 1 and 2)
+  if (warp < 3) {
+    double v = 0.0;
+    for (int i = lane; i < j; i += 32) {
+      const zc q = ss[i], t = st_[i];
+      v = warp == 0 ? fma(q.re, q.re, fma(q.im, q.im, v))
+                    : warp == 1 ? fma(q.re, t.re, fma(q.im, t.im, v)) : fma(q.re, t.im, fma(-q.im, t.re, v));
     }
-    __syncthreads();
-    if (tid == 0) {
-      // previous rotations on the column, then the rotation that zeroes its subdiagonal
-      const int jj = j - 1;
-      for (int i = 0; i < jj; ++i) {
-        const zc hi = ld(scol + 2 * i), hn = ld(scol + 2 * (i + 1));
-        const double c = scs[i];
-        const zc s = ld(ssn + 2 * i);
-        st(scol + 2 * i, zadd(zc{c * hi.re, c * hi.im}, zmul(s, hn)));
-        st(scol + 2 * (i + 1), zadd(zmul(zc{-s.re, s.im}, hi), zc{c * hn.re, c * hn.im}));
+    v = warp_sum(v);
+    if (lane == 0) ssum[warp] = v;
+  }
+  const zc z0{0.0, 0.0};
+  for (int r = lane; r < j; r += 32) {
+    zc q = z0, h = z0, t = z0;
+    for (int i = warp; i < j; i += STEP_W) {
+      // Q row r reaches column r + 1, Hr is Hessenberg (row r from column r - 1), T upper triangular
+      if (i <= r + 1) q = zfma(ld(a.Q + 2 * ((int64_t)i * ldh + r)), sh_[i], q);
+      if (has_w && i >= r - 1) h = zfma(i == j - 1 ? sh_[r] : ld(a.Hr + 2 * ((int64_t)i * ldh + r)), ss[i], h);
+      if (has_w && a.T && i >= r) t = zfma(ld(a.T + 2 * ((int64_t)i * a.ldt + r)), ss[i], t);
+    }
+    sp[0][warp][r] = q;
+    sp[1][warp][r] = h;
+    sp[2][warp][r] = t;
+  }
+  __syncthreads();
+  if (tid == RB - 1) {
+    const double av = vr[4 * j], al2 = av - (j > 0 ? ssum[0] : 0.0);
+    const bool bd = !(al2 > 1e-28 * fmax(av, 1e-300)) || !isfinite(al2);
+    const double inv = bd ? 0.0 : rsqrt(al2);
+    sal[0] = bd ? 0.0 : al2 * inv;
+    sal[1] = inv;
+    sal[2] = bd ? 1.0 : 0.0;
+    *a.brk = bd ? 1 : 0;
+  }
+  // the eight warps' products of row r: threads 0..63 Q, 64..127 Hr, 128..191 T
+  {
+    const int k = tid >> 6;
+    if (k < 3)
+      for (int r = tid & 63; r < j; r += 64) {
+        zc v = z0;
+        for (int w = 0; w < STEP_W; ++w) {
+          v.re += sp[k][w][r].re;
+          v.im += sp[k][w][r].im;
+        }
+        if (k == 0) srot[r] = v;
+        else sp[k][0][r] = v;
       }
-      const zc x = ld(scol + 2 * jj), y = ld(scol + 2 * (jj + 1));
-      const double ax = zabs(x), ay = zabs(y);
-      const double den = hypot(ax, ay);
-      double c;
-      zc s;
+  }
+  __syncthreads();
+  const double al = sal[0], inv = sal[1];
+  const bool bd = sal[2] != 0.0;
+  const bool run = has_w && !bd;
+  // ([t; c_j] - Hr s) / alpha and (e_j - T s) / alpha; rows 0..j - 1 (row j of Hr s is alpha s_{j-1})
+  if (run && tid >= 64) {
+    const int k = tid >> 6;
+    if (k == 1)
+      for (int r = tid & 63; r < j; r += 64) {
+        const zc t = st_[r], h = sp[1][0][r];
+        st(a.Hr + 2 * ((int64_t)j * ldh + r), zc{(t.re - h.re) * inv, (t.im - h.im) * inv});
+      }
+    else if (k == 2 && a.T)
+      for (int r = tid & 63; r < j; r += 64) {
+        const zc t = sp[2][0][r];
+        st(a.T + 2 * ((int64_t)j * a.ldt + r), zc{-t.re * inv, -t.im * inv});
+      }
+  }
+  if (tid == RB - 1) {
+    zc cj = z0;
+    if (run) {
+      cj = zc{(vr[4 * j + 1] - (j > 0 ? ssum[1] : 0.0)) * inv, (vr[4 * j + 2] - (j > 0 ? ssum[2] : 0.0)) * inv};
+      zc h = cj;
+      if (j > 0) {
+        h.re = fma(-al, ss[j - 1].re, h.re);
+        h.im = fma(-al, ss[j - 1].im, h.im);
+      }
+      st(a.Hr + 2 * ((int64_t)j * ldh + j), zc{h.re * inv, h.im * inv});
+      if (a.T) st(a.T + 2 * ((int64_t)j * a.ldt + j), zc{inv, 0.0});
+    }
+    a.coef[4 * j] = cj.re;
+    a.coef[4 * j + 1] = cj.im;
+    a.coef[4 * j + 2] = inv;
+  }
+  if (j == 0) {
+    if (tid == 0) {
+      st(a.g, zc{al, 0.0});
+      st(a.Q, zc{1.0, 0.0});
+      *a.est = al;
+    }
+  } else if (warp == 0) {
+    // the rotation [c s; -conj(s) c] that takes (x, alpha) to (., 0)
+    const int jj = j - 1;
+    const zc x = srot[jj];
+    const double nx = fma(x.re, x.re, x.im * x.im), n2 = fma(al, al, nx);
+    double c;
+    zc s;
+    if (nx > 1e-290 && n2 < 1e290) {
+      const double rx = rsqrt(nx), r2 = rsqrt(n2), f = al * rx * r2;
+      c = nx * rx * r2;
+      s = zc{x.re * f, x.im * f};
+    } else {
+      const double ax = hypot(x.re, x.im), den = hypot(ax, al);
       if (den == 0.0) {
         c = 1.0;
-        s = zc{0.0, 0.0};
+        s = z0;
       } else if (ax == 0.0) {
         c = 0.0;
         s = zc{1.0, 0.0};
       } else {
         c = ax / den;
-        s = zmul(zc{x.re / ax, x.im / ax}, zc{y.re / den, -y.im / den});
+        s = zc{x.re / ax * (al / den), x.im / ax * (al / den)};
       }
-      cs[2 * jj] = c;
-      cs[2 * jj + 1] = 0.0;
-      st(sn + 2 * jj, s);
-      st(scol + 2 * jj, zadd(zc{c * x.re, c * x.im}, zmul(s, y)));
-      st(scol + 2 * (jj + 1), zc{0.0, 0.0});
-      const zc gj = ld(g + 2 * jj);
-      const zc gn = zmul(zc{-s.re, s.im}, gj);
-      st(g + 2 * (jj + 1), gn);
-      st(g + 2 * jj, zc{c * gj.re, c * gj.im});
-      *est = zabs(gn);
     }
-    __syncthreads();
-    double* rc = R + 2 * (int64_t)(j - 1) * ldh;
-    for (int r = tid; r <= 2 * j + 1; r += STEP_T) rc[r] = scol[r];
-  } else if (tid == 0) {
-    g[0] = al;
-    g[1] = 0.0;
-    *est = al;
-  }
-  if (!has_w || bd) {
-    if (tid == 0) {
-      coef[4 * j] = 0.0;
-      coef[4 * j + 1] = 0.0;
-      coef[4 * j + 2] = inv;
-    }
-    return;
-  }
-  // c_j = (b - s^H t) / alpha
-  const zc cj = zc{(b.re - pr) * inv, (b.im - pi) * inv};
-  // column j of Hr: ([t; c_j] - Hr[:, 0..j-1] s) / alpha, rows 0..j (Hessenberg: i >= r - 1)
-  double* hj = Hr + 2 * (int64_t)j * ldh;
-  for (int r = warp; r <= j; r += STEP_T / 32) {
-    double qr = 0.0, qi = 0.0;
-    for (int i = (r > 0 ? r - 1 : 0) + lane; i < j; i += 32) {
-      const zc q = zmul(ld(Hr + 2 * ((int64_t)i * ldh + r)), ld(sv + 2 * i));
-      qr += q.re;
-      qi += q.im;
-    }
-    qr = warp_sum(qr);
-    qi = warp_sum(qi);
+    double* rc = a.R + 2 * (int64_t)jj * ldh;
     if (lane == 0) {
-      const zc base = (r < j) ? ld(tv + 2 * r) : cj;
-      hj[2 * r] = (base.re - qr) * inv;
-      hj[2 * r + 1] = (base.im - qi) * inv;
+      st(rc + 2 * jj, zc{fma(c, x.re, s.re * al), fma(c, x.im, s.im * al)});
+      st(rc + 2 * j, z0);
+      const zc gj = ld(a.g + 2 * jj), gn = zmul(zc{-s.re, s.im}, gj);
+      st(a.g + 2 * j, gn);
+      st(a.g + 2 * jj, zc{c * gj.re, c * gj.im});
+      *a.est = sqrt(fma(gn.re, gn.re, gn.im * gn.im));
     }
-  }
-  // T column j: (e_j - T s) / alpha (T upper triangular)
-  if (T) {
-    for (int r = warp; r < j; r += STEP_T / 32) {
-      double qr = 0.0, qi = 0.0;
-      for (int i = r + lane; i < j; i += 32) {
-        const zc q = zmul(ld(T + 2 * ((int64_t)i * ldt + r)), ld(sv + 2 * i));
-        qr += q.re;
-        qi += q.im;
+    for (int i = lane; i < jj; i += 32) st(rc + 2 * i, srot[i]);
+    // rows jj and j of Q: [c s; -conj(s) c] times (row jj, e_j)
+    for (int i = lane; i <= j; i += 32) {
+      double* q = a.Q + 2 * (int64_t)i * ldh;
+      if (i < j) {
+        const zc o = ld(q + 2 * jj);
+        st(q + 2 * jj, zc{c * o.re, c * o.im});
+        st(q + 2 * j, zmul(zc{-s.re, s.im}, o));
+      } else {
+        st(q + 2 * jj, s);
+        st(q + 2 * j, zc{c, 0.0});
       }
-      qr = warp_sum(qr);
-      qi = warp_sum(qi);
-      if (lane == 0) {
-        T[2 * ((int64_t)j * ldt + r)] = -qr * inv;
-        T[2 * ((int64_t)j * ldt + r) + 1] = -qi * inv;
-      }
     }
-    if (tid == 0) {
-      T[2 * ((int64_t)j * ldt + j)] = inv;
-      T[2 * ((int64_t)j * ldt + j) + 1] = 0.0;
+    // the corrected column of the raw matrix
+    double* hc = a.Hr + 2 * (int64_t)jj * ldh;
+    for (int i = lane; i <= j; i += 32) st(hc + 2 * i, i < j ? sh_[i] : zc{al, 0.0});
+    __syncwarp();
+  }
+  if (gc && tid == 0) {
+    const double e = *a.est;
+    bool stop;
+    if (j == 0) {
+      stop = bd || !isfinite(e);
+    } else {
+      gc->iters++;
+      if (gc->nhist < HELM6_MAX_HIST) gc->hist[gc->nhist++] = e * gc->beta / gc->normF;
+      stop = !(e > gc->itol) || !isfinite(e) || bd || j >= m || gc->iters >= gc->maxit;
     }
-  }
-  if (tid == 0) {
-    coef[4 * j] = cj.re;
-    coef[4 * j + 1] = cj.im;
-    coef[4 * j + 2] = inv;
+    if (stop) gc->k = j;
+    if (j < m) cudaGraphSetConditional(next, stop ? 0u : 1u);
   }
 }
 
-// q = T[0..k-1, 0..k-1] y (T upper triangular, column-major, leading dimension ldt).
-__global__ void tri_mul_kernel(const double* T, int ldt, int k, const double* y, double* q, const int* k_dev) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  if (k_dev) k = *k_dev;
-  for (int r = 0; r < k; ++r) {
-    zc acc = zc{0.0, 0.0};
-    for (int i = r; i < k; ++i) acc = zadd(acc, zmul(ld(T + 2 * ((int64_t)i * ldt + r)), ld(y + 2 * i)));
-    st(q + 2 * r, acc);
-  }
-}
-
-__global__ void set_subdiag_kernel(double* H, int ldh, int j, const double* sumsq, double* inv) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  const double nrm = sqrt(fmax(*sumsq, 0.0));
-  double* col = H + 2 * (int64_t)j * ldh;
-  col[2 * (j + 1)] = nrm;
-  col[2 * (j + 1) + 1] = 0.0;
-  *inv = (nrm > 0.0) ? 1.0 / nrm : 0.0;
-}
-
-__global__ void backsolve_kernel(const double* H, int ldh, int j, const double* g, double* y, const int* j_dev) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
+// y = R^-1 g (R upper triangular, column-major), one step per column: lane r keeps row r's
+// right side, the lane of the column divides and broadcasts; then q = T y, rows by lane and columns
+// by warp.  The next column is requested before the current one is used.
+__global__ void __launch_bounds__(RB) ls_solve_kernel(const double* __restrict__ R, int ldh, int j,
+                                                      const double* __restrict__ g, double* y,
+                                                      const double* __restrict__ T, int ldt, double* q,
+                                                      const int* j_dev) {
+  __shared__ zc sy[STEP_MAXJ], sp[STEP_W][STEP_MAXJ];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   if (j_dev) j = *j_dev;
-  for (int r = j - 1; r >= 0; --r) {
-    zc acc = ld(g + 2 * r);
-    for (int c = r + 1; c < j; ++c) {
-      const zc h = ld(H + 2 * ((int64_t)c * ldh + r));
-      const zc yc = ld(y + 2 * c);
-      const zc p = zmul(h, yc);
-      acc.re -= p.re;
-      acc.im -= p.im;
+  const zc z0{0.0, 0.0};
+  if (warp == 0) {
+    constexpr int RR = STEP_MAXJ / 32;  // rows of a lane
+    zc acc[RR], di[RR], cur[RR], nxt[RR];
+    auto column = [&](int c, zc(&o)[RR]) {
+#pragma unroll
+      for (int k = 0; k < RR; ++k) o[k] = c >= 0 && lane + 32 * k < c ? ld(R + 2 * ((int64_t)c * ldh + lane + 32 * k)) : z0;
+    };
+#pragma unroll
+    for (int k = 0; k < RR; ++k) {
+      const int r = lane + 32 * k;
+      acc[k] = di[k] = z0;
+      if (r < j) {
+        acc[k] = ld(g + 2 * r);
+        const zc d = ld(R + 2 * ((int64_t)r * ldh + r));
+        const double n2 = d.re * d.re + d.im * d.im;
+        if (n2 > 0.0) di[k] = zc{d.re / n2, -d.im / n2};
+      }
     }
-    const zc d = ld(H + 2 * ((int64_t)r * ldh + r));
-    const double n2 = d.re * d.re + d.im * d.im;
-    zc v = (n2 > 0.0) ? zmul(acc, zc{d.re / n2, -d.im / n2}) : zc{0.0, 0.0};
-    st(y + 2 * r, v);
+    column(j - 1, cur);
+    for (int c = j - 1; c >= 0; --c) {
+      column(c - 1, nxt);
+#pragma unroll
+      for (int k = 0; k < RR; ++k)
+        if (c >> 5 == k && lane == (c & 31)) {
+          const zc v = zmul(acc[k], di[k]);
+          sy[c] = v;
+          st(y + 2 * c, v);
+        }
+      __syncwarp();
+      const zc v{-sy[c].re, -sy[c].im};
+#pragma unroll
+      for (int k = 0; k < RR; ++k) {
+        if (32 * k < c) acc[k] = zfma(cur[k], v, acc[k]);
+        cur[k] = nxt[k];
+      }
+    }
+  }
+  __syncthreads();
+  if (!T) return;
+  for (int r = lane; r < j; r += 32) {
+    zc v = z0;
+    for (int i = warp; i < j; i += STEP_W)
+      if (i >= r) v = zfma(ld(T + 2 * ((int64_t)i * ldt + r)), sy[i], v);
+    sp[warp][r] = v;
+  }
+  __syncthreads();
+  for (int r = threadIdx.x; r < j; r += RB) {
+    zc v = z0;
+    for (int w = 0; w < STEP_W; ++w) {
+      v.re += sp[w][r].re;
+      v.im += sp[w][r].im;
+    }
+    st(q + 2 * r, v);
   }
 }
 
@@ -824,13 +830,6 @@ __global__ void axpy_kernel(const TI* __restrict__ x, TO* __restrict__ y, int64_
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < n2; idx += stride)
     y[idx] += (TO)(alpha * (double)x[idx]);
-}
-
-__global__ void set_complex_kernel(double* p, double re, double im) {
-  if (threadIdx.x == 0 && blockIdx.x == 0) {
-    p[0] = re;
-    p[1] = im;
-  }
 }
 
 int grid_for(int64_t n, int bs) {
@@ -854,12 +853,6 @@ int device_sm_count() {
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   return sms > 0 ? sms : 1;
-}
-
-void launch_reduce_cols(const double* partial, int nblocks, int ncols, double* out, int accumulate,
-                        cudaStream_t s) {
-  note_launch();
-  reduce_cols_kernel<<<ncols, RB, 0, s>>>(partial, nblocks, ncols, out, accumulate, nullptr);
 }
 
 template <typename T>
@@ -926,31 +919,16 @@ void launch_reduce_sum(const double* partial, int n, double* out, cudaStream_t s
   reduce_sum_kernel<<<1, RB, 0, s>>>(partial, n, out);
 }
 
-void launch_givens(double* H, int ldh, int j, double* cs, double* sn, double* g, double* res,
-                   cudaStream_t s) {
+void launch_dcgs_step(int j, int has_w, const double* partial, int nblocks, double* red, const StepMem& a, GraphCtl* gc,
+                      int m, cudaGraphConditionalHandle next, cudaStream_t s) {
   note_launch();
-  givens_kernel<<<1, 32, 0, s>>>(H, ldh, j, cs, sn, g, res);
+  dcgs_step_kernel<<<4 * j + 3, RB, 0, s>>>(j, has_w, partial, nblocks, red, a, gc, m, next);
 }
 
-void launch_dcgs_step(int j, int has_w, const double* red, double* Hr, double* R, int ldh, double* T, int ldt,
-                      double* cs, double* sn, double* g, double* coef, double* est, int* brk, cudaStream_t s) {
+void launch_ls_solve(const double* R, int ldh, int j, const double* g, double* y, const double* T, int ldt, double* q,
+                     cudaStream_t s, const int* j_dev) {
   note_launch();
-  dcgs_step_kernel<<<1, STEP_T, 0, s>>>(j, has_w, red, Hr, R, ldh, T, ldt, cs, sn, g, coef, est, brk);
-}
-
-void launch_tri_mul(const double* T, int ldt, int k, const double* y, double* q, cudaStream_t s, const int* k_dev) {
-  note_launch();
-  tri_mul_kernel<<<1, 32, 0, s>>>(T, ldt, k, y, q, k_dev);
-}
-
-void launch_set_subdiag(double* H, int ldh, int j, const double* sumsq, double* inv, cudaStream_t s) {
-  note_launch();
-  set_subdiag_kernel<<<1, 32, 0, s>>>(H, ldh, j, sumsq, inv);
-}
-
-void launch_backsolve(const double* H, int ldh, int j, const double* g, double* y, cudaStream_t s, const int* j_dev) {
-  note_launch();
-  backsolve_kernel<<<1, 32, 0, s>>>(H, ldh, j, g, y, j_dev);
+  ls_solve_kernel<<<1, RB, 0, s>>>(R, ldh, j, g, y, T, ldt, q, j_dev);
 }
 
 __global__ void axpby_kernel(const double* __restrict__ x, double* __restrict__ y, int64_t n, double a, double b) {
@@ -967,11 +945,6 @@ template <typename TI, typename TO>
 void launch_axpy(const TI* x, TO* y, int64_t N, double alpha, cudaStream_t s) {
   note_launch();
   axpy_kernel<TI, TO><<<grid_for(2 * N, RB), RB, 0, s>>>(x, y, 2 * N, alpha);
-}
-
-void launch_set_complex(double* p, double re, double im, cudaStream_t s) {
-  note_launch();
-  set_complex_kernel<<<1, 32, 0, s>>>(p, re, im);
 }
 
 template void launch_axpy<float, double>(const float*, double*, int64_t, double, cudaStream_t);
@@ -1130,24 +1103,6 @@ __global__ void gctl_cycle_kernel(GraphCtl* g, StepHandles ha, int m) {
   for (int j = 0; j <= m; ++j) cudaGraphSetConditional(ha.h[j], j == 0 ? 1u : 0u);
 }
 
-// After Arnoldi step j (its estimate is that of column j - 1): whether step j + 1 runs.
-__global__ void gctl_step_kernel(GraphCtl* g, int j, int m, const double* est, const int* brk,
-                                 cudaGraphConditionalHandle next) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  const double e = *est;
-  const int b = *brk;
-  bool stop;
-  if (j == 0) {
-    stop = b || !isfinite(e);
-  } else {
-    g->iters++;
-    if (g->nhist < HELM6_MAX_HIST) g->hist[g->nhist++] = e * g->beta / g->normF;
-    stop = !(e > g->itol) || !isfinite(e) || b || j >= m || g->iters >= g->maxit;
-  }
-  if (stop) g->k = j;
-  if (j < m) cudaGraphSetConditional(next, stop ? 0u : 1u);
-}
-
 }  // namespace
 
 void launch_gctl_residual(GraphCtl* g, const double* sumsq, const int* zst, const int* tcerr, int first,
@@ -1159,10 +1114,4 @@ void launch_gctl_cycle(GraphCtl* g, const StepHandles& ha, int m, cudaStream_t s
   note_launch();
   gctl_cycle_kernel<<<1, 32, 0, s>>>(g, ha, m);
 }
-void launch_gctl_step(GraphCtl* g, int j, int m, const double* est, const int* brk, cudaGraphConditionalHandle next,
-                      cudaStream_t s) {
-  note_launch();
-  gctl_step_kernel<<<1, 32, 0, s>>>(g, j, m, est, brk, next);
-}
-
 }  // namespace helm6
