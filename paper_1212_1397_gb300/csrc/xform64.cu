@@ -29,8 +29,8 @@
 //     (the mirrored ones too) into an FP64 ring with cp.async and turn them into the seven FP16
 //     digit planes of the A operand;
 //   * a producer thread streams its CTA's half of the basis' digit planes (cp.async.bulk);
-//   * the MMA warp of the first CTA issues the 28 products of a stage for both, once the second
-//     CTA's has told it that its operands are there;
+//   * the MMA warp of the first CTA issues the 28 products of a stage for both; the second one's passes
+//     its operands' barrier on to the first one's, so that each waits once per stage;
 //   * eight epilogue warps take the finished sums out of tensor memory as 64-bit integers,
 //     release it, then round and store them while the next group runs;
 //   * two scanner warps find the row exponents of the next unit's rows (which also brings those
@@ -77,7 +77,7 @@ constexpr int O_D = O_B + X_NS * B_BYTES;
 constexpr int O_S = O_D + X_ND * D_BYTES;
 constexpr int O_E = O_S + X_EPI * STG_BYTES;   // row exponents, two units
 constexpr int O_BAR = O_E + 2 * X_M * 4;
-constexpr int X_NBAR = 4 * X_NS + 7;
+constexpr int X_NBAR = 2 * X_NS + 7;
 constexpr int O_MISC = O_BAR + X_NBAR * 8;
 constexpr int X_SMEM = O_MISC + 16 + 1024;
 static_assert(X_SMEM <= 232448, "shared memory per CTA");
@@ -111,7 +111,7 @@ __device__ __forceinline__ uint64_t sdesc(uint32_t addr, uint32_t lbo, uint32_t 
 __device__ __forceinline__ bool try_wait(uint32_t bar, uint32_t parity) {
   uint32_t ok;
   asm volatile(
-      "{\n .reg .pred P1;\n mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 P1, [%1], %2;\n"
+      "{\n .reg .pred P1;\n mbarrier.try_wait.parity.shared::cta.b64 P1, [%1], %2;\n"
       " selp.b32 %0, 1, 0, P1;\n}\n"
       : "=r"(ok)
       : "r"(bar), "r"(parity)
@@ -133,12 +133,13 @@ __device__ __forceinline__ bool poll1(uint32_t bar, uint32_t parity, volatile in
   return false;
 }
 
-// Warp-uniform bounded wait: lane 0 polls, the warp takes its answer.
+// Warp-uniform bounded wait: every lane polls.  (Lane 0 alone and a shuffle of its answer: the warp
+// diverges and meets again on each wait; 372/799/742/404 us for the four transforms of a 256^3
+// preconditioner against 344/682/631/377.)
 template <int NAP>
-__device__ __forceinline__ bool pollw(uint32_t bar, uint32_t parity, volatile int* fail, int lane) {
-  int ok = 0;
-  if (lane == 0) ok = poll1<NAP>(bar, parity, fail) ? 1 : 0;
-  return __shfl_sync(0xffffffffu, ok, 0) != 0;
+__device__ __forceinline__ bool pollw(uint32_t bar, uint32_t parity, volatile int* fail) {
+  const bool ok = poll1<NAP>(bar, parity, fail);
+  return __all_sync(0xffffffffu, ok) != 0;
 }
 
 // D (FP32) += A B^T, FP16 operands from shared memory; executed by the whole warp, issued by one
@@ -163,7 +164,7 @@ __device__ __forceinline__ void commit(uint32_t bar) {
 __device__ __forceinline__ void arrive_lead(uint32_t bar) {
   uint32_t a;
   asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(a) : "r"(bar));
-  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(a) : "memory");
+  asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(a) : "memory");
 }
 
 __device__ __forceinline__ void cluster_sync() {
@@ -271,23 +272,19 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(X_THREADS, 1) xform6
   volatile int* fail = (volatile int*)(tslot + 1);
   int* rowexp = (int*)(smem + O_E);
   const uint32_t bar0 = s_addr(smem + O_BAR);
-  auto afull = [&](int s) { return bar0 + 8u * s; };               // digit planes of a stage written
-  auto bfull = [&](int s) { return bar0 + 8u * (X_NS + s); };      // basis planes of a stage arrived
-  auto sfree = [&](int s) { return bar0 + 8u * (2 * X_NS + s); };  // the stage's MMAs completed
-  auto peer = [&](int s) { return bar0 + 8u * (3 * X_NS + s); };   // first CTA: the second one's operands are there
-  const uint32_t tfull = bar0 + 8u * (4 * X_NS);                   // the group's accumulators complete
-  const uint32_t tempty = bar0 + 8u * (4 * X_NS + 1);              // first CTA: ... and drained in both
-  auto efull = [&](int b) { return bar0 + 8u * (4 * X_NS + 2 + b); };  // row exponents of a unit known
-  auto efree = [&](int b) { return bar0 + 8u * (4 * X_NS + 5 + b); };  // ... and read by everybody
-  const uint32_t drain = bar0 + 8u * (4 * X_NS + 4);               // every MMA issued completed
+  auto full = [&](int s) { return bar0 + 8u * s; };            // the stage's operands are there (first CTA: in both)
+  auto sfree = [&](int s) { return bar0 + 8u * (X_NS + s); };  // the stage's MMAs completed
+  const uint32_t tfull = bar0 + 8u * (2 * X_NS);                   // the group's accumulators complete
+  const uint32_t tempty = bar0 + 8u * (2 * X_NS + 1);              // first CTA: ... and drained in both
+  auto efull = [&](int b) { return bar0 + 8u * (2 * X_NS + 2 + b); };  // row exponents of a unit known
+  auto efree = [&](int b) { return bar0 + 8u * (2 * X_NS + 5 + b); };  // ... and read by everybody
+  const uint32_t drain = bar0 + 8u * (2 * X_NS + 4);               // every MMA issued completed
 
   if (tid == 0) {
     auto init = [](uint32_t b, int n) { asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(b), "r"(n)); };
     for (int s = 0; s < X_NS; ++s) {
-      init(afull(s), X_CONV / 2);
-      init(bfull(s), 1);
+      init(full(s), 4 + (rank ? 1 : 2));  // a converter group, the producer; first CTA: the relay
       init(sfree(s), 1);
-      init(peer(s), 1);
     }
     init(tfull, 1);
     init(tempty, 2 * X_EPI);
@@ -324,17 +321,18 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(X_THREADS, 1) xform6
           for (int kt = 0; kt < p.nk; ++kt, ++q) {
             const int s = q % X_NS, u = q / X_NS;
             if (u >= 1 && !poll1<100>(sfree(s), (u - 1) & 1, fail)) break;
-            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bfull(s)), "r"(bstage) : "memory");
+            const uint32_t bar = full(s);
+            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bstage) : "memory");
             asm volatile(
                 "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
                     s_addr(smem + O_B + s * B_BYTES)),
-                "l"(Wg + (size_t)kt * 2 * bstage), "r"(bstage), "r"(bfull(s))
+                "l"(Wg + (size_t)kt * 2 * bstage), "r"(bstage), "r"(bar)
                 : "memory");
             last = q;
           }
         }
       }
-      if (last >= 0) poll1<100>(bfull(last % X_NS), (last / X_NS) & 1, fail);  // the last copy has landed
+      if (last >= 0) poll1<100>(full(last % X_NS), (last / X_NS) & 1, fail);  // the last copy has landed
     }
     __syncwarp();
   } else if (warp == X_WMMA) {
@@ -357,11 +355,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(X_THREADS, 1) xform6
           asm volatile("tcgen05.fence::after_thread_sync;");
         }
         for (int kt = 0; kt < p.nk; ++kt) {
-          ok = poll1<20>(afull(s), ph, fail) && poll1<20>(bfull(s), ph, fail) && (rank || poll1<20>(peer(s), ph, fail));
+          ok = poll1<20>(full(s), ph, fail);
           ok = __all_sync(0xffffffffu, ok);
           if (!ok) break;
           if (rank) {
-            if (lane == 0) arrive_lead(peer(s));
+            if (lane == 0) arrive_lead(full(s));
           } else {
             asm volatile("tcgen05.fence::after_thread_sync;");
             const uint64_t a0 = adesc + (uint64_t)(s * (A_BYTES >> 4)), b0 = bdesc + (uint64_t)(s * (B_BYTES >> 4));
@@ -392,7 +390,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(X_THREADS, 1) xform6
     bool ok = true;
     for (int i = 0; i < nun && ok; ++i) {
       const int b = i & 1, m0 = unit_at(i).m0;
-      if (i >= 2 && !pollw<100>(efree(b), ((i >> 1) - 1) & 1, fail, lane)) break;
+      if (i >= 2 && !pollw<100>(efree(b), ((i >> 1) - 1) & 1, fail)) break;
       for (int rr = w0; rr < w0 + X_M / X_SCAN; rr += 4) {
         uint32_t mx[4] = {0u, 0u, 0u, 0u};
         const uint32_t* src = (const uint32_t*)(p.in + (int64_t)(m0 + rr) * p.ldin) + 1;
@@ -459,7 +457,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(X_THREADS, 1) xform6
     bool ok = true;
     for (int i = 0; i < nun && ok; ++i) {
       const Unit un = unit_at(i);
-      if (!pollw<20>(efull(i & 1), (i >> 1) & 1, fail, lane)) break;
+      if (!pollw<20>(efull(i & 1), (i >> 1) & 1, fail)) break;
       const int emax = row_emax(rowexp[(i & 1) * X_M + r]);
       __syncwarp();
       if (lane == 0) arrive(efree(i & 1));
@@ -512,7 +510,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(X_THREADS, 1) xform6
           }
           __syncwarp();
           issue();  // the ring slot just read is free again
-          if (u >= 1 && !pollw<20>(sfree(s), (u - 1) & 1, fail, lane)) {
+          if (u >= 1 && !pollw<20>(sfree(s), (u - 1) & 1, fail)) {
             ok = false;
             break;
           }
@@ -538,7 +536,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(X_THREADS, 1) xform6
           }
           asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
           __syncwarp();
-          if (lane == 0) arrive(afull(s));
+          if (lane == 0) arrive(full(s));
         }
       }
     }
@@ -553,7 +551,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(X_THREADS, 1) xform6
     bool ok = true;
     for (int i = 0; i < nun && ok; ++i) {
       const Unit un = unit_at(i);
-      if (!pollw<100>(efull(i & 1), (i >> 1) & 1, fail, lane)) break;
+      if (!pollw<100>(efull(i & 1), (i >> 1) & 1, fail)) break;
       const int lrow = 32 * (quarter & 1) + lane, row0 = un.m0 + 32 * (quarter & 1), row = row0 + lane;
       const bool live = row < p.M_total;
       const int nrows = min(32, p.M_total - row0);
@@ -570,7 +568,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(X_THREADS, 1) xform6
         obase = (int64_t)plane * p.ldo * p.P + rr;
       }
       for (int g = un.g0; g < un.g1; ++g, ++ng) {
-        if (!pollw<100>(tfull, ng & 1, fail, lane)) {
+        if (!pollw<100>(tfull, ng & 1, fail)) {
           ok = false;
           break;
         }
