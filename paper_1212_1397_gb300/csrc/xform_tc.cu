@@ -12,28 +12,35 @@
 // three rings in shared memory:
 //   * eight converter warps (warp w <-> rows 16 w .. 16 w + 15 of the tile) copy their rows'
 //     32 FP32 values of a stage into an FP32 ring with cp.async, three stages ahead (each
-//     instruction of a warp covers whole 128-byte row segments), then split them (half a
-//     row per thread) into the BF16 hi/lo operand ring (no-swizzle K-major core matrices:
-//     8 rows x 16 bytes, 8-row groups 128 B apart, K step one column of core matrices) and
-//     arrive on the stage's `afull` mbarrier.  Output columns beyond 256 (at most 8, the
-//     258-point Neumann axes) are accumulated in FP32 by the same threads from the values
+//     instruction of a warp covers whole 128-byte row segments), split them (half a
+//     row per thread), then wait for the operand slot, write the BF16 hi/lo operands (no-swizzle
+//     K-major core matrices: 8 rows x 16 bytes, 8-row groups 128 B apart, K step one column of
+//     core matrices) and arrive on the stage's `full` mbarrier.  Output columns beyond 256 (at most 8,
+//     the 258-point Neumann axes) are accumulated in FP32 by the same threads from the values
 //     they already hold, and written by them;
-//   * one producer thread streams the basis stage (hi and lo tiles, prepared on the host)
-//     into the basis ring with cp.async.bulk completing on `bfull`;
-//   * one MMA thread waits for both, issues the tcgen05.mma's of the stage into one of two
-//     256-column tensor-memory accumulators and commits them to `sfree` (which releases the
-//     stage's operand slots) and, after a tile's last stage, to `tfull`;
+//   * one producer thread streams the basis stage (hi and lo tiles, prepared on the host) into the
+//     basis ring with cp.async.bulk, completing on `full` too: the MMA warp waits once per stage;
+//   * one MMA warp issues the tcgen05.mma's (one elected lane, operands in uniform registers) into
+//     one of two 256-column tensor-memory accumulators and commits them to `sfree` (which
+//     releases the stage's operand slots) and, after a tile's last stage, to `tfull`;
 //   * eight epilogue warps drain the other accumulator (tcgen05.ld, 32 lanes = 32 rows per
 //     warp, two warps per lane quarter taking alternate 16-column chunks) while the next
 //     tile's MMAs run, store it either transposed within planes of R rows
 //     (out[(row/R)*R*P + p*R + row%R]: consecutive lanes on consecutive addresses) or
 //     row-major through a per-warp shared-memory transpose (out[row*P + p]: row segments
-//     written by consecutive lanes), and release it on `tempty`.  The global stores are
-//     the slowest part of a tile (measured), hence eight warps issuing them.
+//     written by consecutive lanes), and release it on `tempty`.
+// What bounds it is the converters' serial chain (copy landed, split, slot free, operands written,
+// fence, arrive: about 1,900 cycles a stage, 56 stages per CTA at 256^3), not the products (771
+// cycles a stage), so its hand-offs are what counts: the split before the wait for the slot, one
+// barrier per stage, waits polled by whole warps, copy addresses carried along instead of taken
+// from a running index by division.  At 256^3 with 258-point y the transforms x, y, y^-1, x^-1 of
+// a preconditioner take 72/89/87/60 us (75/101/101/66 before these), at 128^3 17/16/18/14
+// (20/19/21/16).  CTA pairs (cta_group::2, half the shared-memory traffic per product) measured
+// the same at 256^3 and 1.5 to 2 us slower per transform below 160^3.
 // Every mbarrier wait is bounded and warp-uniform; a timeout sets a shared flag that ends
-// every role's loop, and *err for the host.  Whatever the path, the MMA thread waits
-// (bounded) for all of its committed MMAs, the producer for its last bulk copy and the
-// converters for their cp.async groups before the tensor memory is freed.
+// every role's loop, and *err for the host.  Whatever the path, the CTA waits (bounded) for its committed
+// MMAs, the producer for its last bulk copy and the converters for their cp.async groups before
+// the tensor memory is freed.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -45,7 +52,7 @@ namespace helm6 {
 
 namespace {
 
-constexpr int TC_M = 128;
+constexpr int TC_M = 128;                // rows of a tile (MMA M)
 constexpr int TC_KT = 32;                // K per stage
 constexpr int TC_KC = TC_KT / 8;         // core-matrix columns per stage
 constexpr int TC_GMAX = 256;             // output columns of one work item (MMA N limit)
@@ -59,20 +66,20 @@ constexpr int TC_THREADS = 576;
 constexpr int A_TILE = TC_M * TC_KT * 2;            // bytes of one BF16 term of a data stage
 constexpr int A_STAGE = 2 * A_TILE;                 // hi + lo
 constexpr int A_LBO = (TC_M / 8) * 128;             // K step of the data stage
-constexpr int B_STAGE = 2 * TC_KC * TC_GMAX * 16;   // hi + lo basis, 256 rows
+constexpr int B_STAGE = 2 * TC_KC * TC_GMAX * 16;    // hi + lo basis
 constexpr int D_STAGE = TC_M * TC_KT * 4;           // FP32 data, 128 B per row
 constexpr int EPI_COLS = 16;                        // columns per epilogue chunk
 constexpr int STG_TLD = 36;                         // staged column stride of the transposed store
 constexpr int STG_FLOATS = EPI_COLS * STG_TLD;      // per-warp staging (>= 32 rows x 16 columns)
+constexpr int TAIL_LD = ((TC_GMAX + TC_TAILMAX + TC_KT - 1) / TC_KT) * TC_KT;  // tail row stride (288)
+constexpr int TAIL_FLOATS = TC_TAILMAX * TAIL_LD;
 constexpr int OFF_A = 0;
 constexpr int OFF_B = OFF_A + NS * A_STAGE;
 constexpr int OFF_D = OFF_B + NS * B_STAGE;
 constexpr int OFF_T = OFF_D + ND * D_STAGE;
-constexpr int TAIL_LD = ((TC_GMAX + TC_TAILMAX + TC_KT - 1) / TC_KT) * TC_KT;  // tail row stride (288)
-constexpr int TAIL_FLOATS = TC_TAILMAX * TAIL_LD;
 constexpr int OFF_S = OFF_T + TAIL_FLOATS * 4;
 constexpr int OFF_BAR = OFF_S + EPI_WARPS * STG_FLOATS * 4;
-constexpr int NBAR = 3 * NS + 5;  // afull, bfull, sfree per stage; tfull, tempty per buffer; drain
+constexpr int NBAR = 2 * NS + 5;  // full, sfree per stage; tfull, tempty per buffer; drain
 constexpr int OFF_MISC = OFF_BAR + NBAR * 8;
 constexpr int SMEM_BYTES = OFF_MISC + 16 + 1024;  // + alignment of the base to 1024
 static_assert(SMEM_BYTES <= 232448, "shared memory per CTA");
@@ -82,7 +89,7 @@ constexpr int kMaxPolls = 1 << 22;
 struct TcArgs {
   const float* in;
   float* out;
-  const uint8_t* W;   // per column group: [kt][term][kc][Npad_g / 8][8 rows][16 B]
+  const uint8_t* W;   // per column group: [kt][half][term][kc][npad_g / 2 columns][16 B]
   const float* Bt;    // tail basis rows (FP32, tail x K) or null
   int M_total, K, P, nk, terms, transposed, R;
   int ldin;  // input row pitch (floats, >= K)
@@ -129,22 +136,38 @@ __device__ __forceinline__ bool poll1(uint32_t bar, uint32_t parity, volatile in
   return false;
 }
 
-// Warp-uniform bounded wait: lane 0 polls, the warp takes its answer.
-__device__ __forceinline__ bool pollw(uint32_t bar, uint32_t parity, volatile int* fail, int lane) {
-  int ok = 0;
-  if (lane == 0) ok = poll1(bar, parity, fail) ? 1 : 0;
-  return __shfl_sync(0xffffffffu, ok, 0) != 0;
+// Warp-uniform bounded wait: every lane polls.  With lane 0 alone polling and a shuffle of its
+// answer the warp diverges and meets again on each wait, which the converters' serial chain feels:
+// at 256^3 the four transforms took 75/93/91/71 us so and 73/88/86/60 us this way.
+__device__ __forceinline__ bool pollw(uint32_t bar, uint32_t parity, volatile int* fail) {
+  const bool ok = poll1(bar, parity, fail);
+  return __all_sync(0xffffffffu, ok) != 0;
 }
 
+// Executed by the whole warp, issued by one elected lane (the operands stay in uniform registers).
 __device__ __forceinline__ void mma(uint32_t tmem, uint64_t a, uint64_t b, uint32_t id, uint32_t acc) {
   asm volatile(
-      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-      " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem),
+      "{\n .reg .pred p, e;\n setp.ne.b32 p, %4, 0;\n elect.sync _|e, 0xffffffff;\n"
+      " @e tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem),
       "l"(a), "l"(b), "r"(id), "r"(acc));
 }
 
+// Arrive on this barrier once the MMAs issued so far have completed.
 __device__ __forceinline__ void commit(uint32_t bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
+  asm volatile(
+      "{\n .reg .pred e;\n elect.sync _|e, 0xffffffff;\n"
+      " @e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}\n" ::"r"(bar)
+      : "memory");
+}
+
+__device__ __forceinline__ void arrive(uint32_t bar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+
+__device__ __forceinline__ void bulk(uint32_t dst, const void* src, int bytes, uint32_t bar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+               "l"(src), "r"(bytes), "r"(bar)
+               : "memory");
 }
 
 // 16 consecutive tensor-memory columns of the warp's 32 lanes (one row per thread).
@@ -210,17 +233,15 @@ __global__ void __launch_bounds__(TC_THREADS, 1) xform_tc_kernel(TcArgs p) {
   uint32_t* tslot = (uint32_t*)(smem + OFF_MISC);
   volatile int* fail = (volatile int*)(tslot + 1);
   const uint32_t bar0 = s_addr(bars);
-  auto afull = [&](int s) { return bar0 + 8u * s; };             // converters stored the data stage
-  auto bfull = [&](int s) { return bar0 + 8u * (NS + s); };      // basis stage arrived
-  auto sfree = [&](int s) { return bar0 + 8u * (2 * NS + s); };  // the stage's MMAs completed
-  auto tfull = [&](int b) { return bar0 + 8u * (3 * NS + b); };  // accumulator b complete
-  auto tempty = [&](int b) { return bar0 + 8u * (3 * NS + 2 + b); };  // accumulator b drained
-  const uint32_t drain = bar0 + 8u * (3 * NS + 4);                 // every MMA issued completed
+  auto full = [&](int s) { return bar0 + 8u * s; };          // the stage's operands are there
+  auto sfree = [&](int s) { return bar0 + 8u * (NS + s); };  // the stage's MMAs completed
+  auto tfull = [&](int b) { return bar0 + 8u * (2 * NS + b); };  // accumulator b complete
+  auto tempty = [&](int b) { return bar0 + 8u * (2 * NS + 2 + b); };  // accumulator b drained
+  const uint32_t drain = bar0 + 8u * (2 * NS + 4);                 // every MMA issued completed
 
   if (tid == 0) {
     for (int s = 0; s < NS; ++s) {
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(afull(s)), "r"(CONV_WARPS));
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bfull(s)), "r"(1));
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(full(s)), "r"(CONV_WARPS + 1));
       asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(sfree(s)), "r"(1));
     }
     for (int b = 0; b < 2; ++b) {
@@ -246,8 +267,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1) xform_tc_kernel(TcArgs p) {
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;");
   const uint32_t tmem = *tslot;
-  const int nitems = (int)blockIdx.x < p.nwork ? (p.nwork - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
-  const int nstages = nitems * p.nk;
+  const int nitems = blockIdx.x < p.nwork ? (p.nwork - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
+  auto item_at = [&](int i) { return item(p, (int)blockIdx.x + i * (int)gridDim.x); };
 
   if (warp == W_PROD) {
     // ---- basis producer ----
@@ -255,68 +276,63 @@ __global__ void __launch_bounds__(TC_THREADS, 1) xform_tc_kernel(TcArgs p) {
     if (lane == 0) {
       int g = 0;
       for (int i = 0; i < nitems && !*fail; ++i) {
-        const Item it = item(p, (int)blockIdx.x + i * (int)gridDim.x);
-        const int gpad = round16(p.gcols);
+        const Item it = item_at(i);
         const int bterm = TC_KC * it.npad * 16;
         const int btx = (p.terms == 3 ? 2 : 1) * bterm;
-        const uint8_t* Wg = p.W + (size_t)it.grp * p.nk * 2 * TC_KC * gpad * 16;
+        const uint8_t* Wg = p.W + (size_t)it.grp * p.nk * 2 * TC_KC * p.gcols * 16;
         for (int kt = 0; kt < p.nk; ++kt, ++g) {
           const int s = g % NS, u = g / NS;
           if (u >= 1 && !poll1(sfree(s), (u - 1) & 1, fail)) break;
-          const uint32_t dst = s_addr(smem + OFF_B + s * B_STAGE);
-          asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bfull(s)), "r"(btx) : "memory");
-          asm volatile(
-              "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
-              "l"(Wg + (size_t)kt * 2 * bterm), "r"(btx), "r"(bfull(s))
-              : "memory");
+          const uint32_t dst = s_addr(smem + OFF_B + s * B_STAGE), bar = full(s);
+          asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(btx) : "memory");
+          bulk(dst, Wg + (size_t)kt * 2 * bterm, btx, bar);
           last = g;
         }
         if (*fail) break;
       }
       // the last copy must have landed before the CTA ends
-      if (last >= 0) poll1(bfull(last % NS), (last / NS) & 1, fail);
+      if (last >= 0) poll1(full(last % NS), (last / NS) & 1, fail);
     }
     __syncwarp();
   } else if (warp == W_MMA) {
-    // ---- MMA issuer ----
-    if (lane == 0) {
-      int g = 0;
-      for (int i = 0; i < nitems && !*fail; ++i) {
-        const Item it = item(p, (int)blockIdx.x + i * (int)gridDim.x);
-        const int b = i & 1, v = i >> 1;
-        if (v >= 1 && !poll1(tempty(b), (v - 1) & 1, fail)) break;
-        asm volatile("tcgen05.fence::after_thread_sync;");
-        const uint32_t id = idesc(it.npad);
-        const uint32_t bterm = TC_KC * it.npad * 16, b_lbo = (uint32_t)it.npad * 16;
-        const uint32_t d = tmem + (uint32_t)(b * TC_GMAX);
-        bool ok = true;
-        for (int kt = 0; kt < p.nk; ++kt, ++g) {
-          const int s = g % NS, u = g / NS;
-          if (!poll1(afull(s), u & 1, fail) || !poll1(bfull(s), u & 1, fail)) {
-            ok = false;
-            break;
-          }
-          asm volatile("tcgen05.fence::after_thread_sync;");
-          const uint32_t aHi = s_addr(smem + OFF_A + s * A_STAGE), aLo = aHi + A_TILE;
-          const uint32_t bHi = s_addr(smem + OFF_B + s * B_STAGE), bLo = bHi + bterm;
-          const int nkk = min(TC_KT / 16, (p.K - kt * TC_KT + 15) / 16);
-          for (int kk = 0; kk < nkk; ++kk) {
-            const uint32_t acc = (kt > 0 || kk > 0) ? 1u : 0u;
-            const uint64_t ah = sdesc(aHi + kk * 2 * A_LBO, A_LBO, 128);
-            const uint64_t bh = sdesc(bHi + kk * 2 * b_lbo, b_lbo, 128);
-            mma(d, ah, bh, id, acc);
-            if (p.terms >= 2) mma(d, sdesc(aLo + kk * 2 * A_LBO, A_LBO, 128), bh, id, 1u);
-            if (p.terms >= 3) mma(d, ah, sdesc(bLo + kk * 2 * b_lbo, b_lbo, 128), id, 1u);
-          }
-          commit(sfree(s));
-        }
+    // ---- MMA issuer (the whole warp runs the loop, one elected lane issues) ----
+    int s = 0;
+    uint32_t ph = 0;
+    bool ok = true;
+    for (int i = 0; i < nitems && ok; ++i) {
+      const Item it = item_at(i);
+      const int b = i & 1, v = i >> 1;
+      if (v >= 1 && !pollw(tempty(b), (v - 1) & 1, fail)) break;
+      asm volatile("tcgen05.fence::after_thread_sync;");
+      const uint32_t id = idesc(it.npad);
+      const uint32_t bterm = TC_KC * it.npad * 16, b_lbo = (uint32_t)it.npad * 16;
+      const uint32_t d = tmem + (uint32_t)(b * TC_GMAX);
+      for (int kt = 0; kt < p.nk; ++kt) {
+        ok = pollw(full(s), ph, fail);
         if (!ok) break;
-        commit(tfull(b));
+        asm volatile("tcgen05.fence::after_thread_sync;");
+        const uint32_t aHi = s_addr(smem + OFF_A + s * A_STAGE), aLo = aHi + A_TILE;
+        const uint32_t bHi = s_addr(smem + OFF_B + s * B_STAGE), bLo = bHi + bterm;
+        const int nkk = min(TC_KT / 16, (p.K - kt * TC_KT + 15) / 16);
+        for (int kk = 0; kk < nkk; ++kk) {
+          const uint32_t acc = (kt > 0 || kk > 0) ? 1u : 0u;
+          const uint64_t ah = sdesc(aHi + kk * 2 * A_LBO, A_LBO, 128);
+          const uint64_t bh = sdesc(bHi + kk * 2 * b_lbo, b_lbo, 128);
+          mma(d, ah, bh, id, acc);
+          if (p.terms >= 2) mma(d, sdesc(aLo + kk * 2 * A_LBO, A_LBO, 128), bh, id, 1u);
+          if (p.terms >= 3) mma(d, ah, sdesc(bLo + kk * 2 * b_lbo, b_lbo, 128), id, 1u);
+        }
+        commit(sfree(s));
+        if (++s == NS) {
+          s = 0;
+          ph ^= 1u;
+        }
       }
-      // every MMA issued above has completed before the tensor memory is freed
-      commit(drain);
-      poll1(drain, 0, fail);
+      if (ok) commit(tfull(b));
     }
+    // every MMA issued above has completed before the tensor memory is freed
+    commit(drain);
+    poll1(drain, 0, fail);
     __syncwarp();
   } else if (warp >= EPI_WARPS) {
     // ---- converters: warp cw copies rows 16 cw .. 16 cw + 15 of each stage into the FP32
@@ -329,75 +345,107 @@ __global__ void __launch_bounds__(TC_THREADS, 1) xform_tc_kernel(TcArgs p) {
     float tacc[TC_TAILMAX];
 #pragma unroll
     for (int c = 0; c < TC_TAILMAX; ++c) tacc[c] = 0.f;
-    // issue the copies of stage q (work item q / nk, K stage q % nk) into ring slot q % ND
-    auto issue = [&](int q) {
-      if (q < nstages) {
-        const Item it = item(p, (int)blockIdx.x + (q / p.nk) * (int)gridDim.x);
-        const int k0 = (q % p.nk) * TC_KT;
-        const uint32_t slot = ring + (uint32_t)((q % ND) * D_STAGE);
+    // the next stage to copy: item ci, K stage ck, ring slot cs.  One copy instruction covers RPC rows
+    // and a lane keeps its place within a row, so that an item costs one address and a stage a few
+    // additions (stage and item taken from a running index by division cost 680 cycles a stage,
+    // as much as the conversion).
+    constexpr int LPR = 128 / VEC, RPC = 32 / LPR;
+    const int lr = lane / LPR, bb = (lane % LPR) * VEC;
+    const uint32_t rdst = ring + (uint32_t)((16 * cw + lr) * 128 + (bb & 15));
+    int ci = 0, ck = 0, cs = 0, crow = 0;
+    const float* csrc = p.in;
+    auto copy_item = [&]() {
+      if (ci < nitems) {
+        crow = item_at(ci).m0 + 16 * cw + lr;
+        csrc = p.in + (int64_t)crow * p.ldin + (bb >> 2);
+      }
+    };
+    copy_item();
+    auto issue = [&]() {
+      if (ci < nitems) {
+        const int k = ck * TC_KT + (bb >> 2);
+        // (the row's padding behind point K - 1 is not read: it can hold anything, and its zero basis
+        // entries would not cancel a NaN)
+        const int bytes = min(VEC, max(0, 4 * (p.K - k)));
 #pragma unroll
-        for (int c = 0; c < 64 / VEC; ++c) {
-          const int o = (c * 32 + lane) * VEC;             // byte within the warp's 16 x 128 B
-          const int rr = 16 * cw + (o >> 7), bb = o & 127;  // tile row, byte within its segment
-          const int row = it.m0 + rr, k = k0 + (bb >> 2);
-          const bool valid = row < p.M_total && k < p.K;
-          const float* src = valid ? p.in + (int64_t)row * p.ldin + k : p.in;
-          // (the row's padding behind point K - 1 is not read: it can hold anything, and its zero basis
-          // entries would not cancel a NaN)
-          cp_async<VEC>(slot + (uint32_t)(rr * 128 + (((bb >> 4) ^ (rr & 7)) << 4) + (bb & 15)), src,
-                        valid ? min(VEC, 4 * (p.K - k)) : 0);
+        for (int c = 0; c < 16 / RPC; ++c) {
+          const bool in = bytes > 0 && crow + c * RPC < p.M_total;
+          cp_async<VEC>(rdst + (uint32_t)(cs * D_STAGE + c * RPC * 128 + (((bb >> 4) ^ ((lr + c * RPC) & 7)) << 4)),
+                        in ? csrc + (int64_t)(c * RPC) * p.ldin + ck * TC_KT : p.in, in ? bytes : 0);
+        }
+        if (++cs == ND) cs = 0;
+        if (++ck == p.nk) {
+          ck = 0;
+          ++ci;
+          copy_item();
         }
       }
       asm volatile("cp.async.commit_group;" ::: "memory");
     };
-    for (int q = 0; q < ND; ++q) issue(q);
-    for (int g = 0; g < nstages; ++g) {
-      const int s = g % NS, u = g / NS, kt = g % p.nk;
-      asm volatile("cp.async.wait_group %0;" ::"n"(ND - 1) : "memory");
-      __syncwarp();  // the warp's rows, copied by all of its lanes, are visible to each lane
-      if (u >= 1 && !pollw(sfree(s), (u - 1) & 1, fail, lane)) break;
-      const uint8_t* dslot = smem + OFF_D + (size_t)(g % ND) * D_STAGE + (size_t)r * 128;
-      uint8_t* sA = smem + OFF_A + s * A_STAGE;
-      const int k0 = kt * TC_KT;
+    for (int q = 0; q < ND; ++q) issue();
+    int s = 0, ds = 0;
+    uint32_t ph = 1;  // parity of the operand slot's last release (none yet: the wait passes)
+    bool ok = true;
+    for (int i = 0; i < nitems && ok; ++i) {
+      for (int kt = 0; kt < p.nk; ++kt) {
+        asm volatile("cp.async.wait_group %0;" ::"n"(ND - 1) : "memory");
+        __syncwarp();  // the warp's rows, copied by all of its lanes, are visible to each lane
+        const uint8_t* dslot = smem + OFF_D + (size_t)ds * D_STAGE + (size_t)r * 128;
+        const int k0 = kt * TC_KT;
+        uint4 hi[2], lo[2];
 #pragma unroll
-      for (int e = 0; e < 2; ++e) {
-        const int kg = 2 * hk + e;
-        const float4 a = *(const float4*)(dslot + (((2 * kg) ^ sw) << 4));
-        const float4 b = *(const float4*)(dslot + (((2 * kg + 1) ^ sw) << 4));
-        uint4 hi, lo;
-        split8(a, b, hi, lo);
-        const int off = kg * A_LBO + (r >> 3) * 128 + (r & 7) * 16;
-        *(uint4*)(sA + off) = hi;
-        *(uint4*)(sA + A_TILE + off) = lo;
-        if (TAIL && p.tail) {
+        for (int e = 0; e < 2; ++e) {
+          const int kg = 2 * hk + e;
+          const float4 a = *(const float4*)(dslot + (((2 * kg) ^ sw) << 4));
+          const float4 b = *(const float4*)(dslot + (((2 * kg + 1) ^ sw) << 4));
+          split8(a, b, hi[e], lo[e]);
+          if (TAIL && p.tail) {
 #pragma unroll
-          for (int c = 0; c < TC_TAILMAX; ++c) {
-            if (c < p.tail) {
-              const float4 w0 = *(const float4*)(sBt + c * TAIL_LD + k0 + 8 * kg);
-              const float4 w1 = *(const float4*)(sBt + c * TAIL_LD + k0 + 8 * kg + 4);
-              float acc = tacc[c];
-              acc = fmaf(a.x, w0.x, acc);
-              acc = fmaf(a.y, w0.y, acc);
-              acc = fmaf(a.z, w0.z, acc);
-              acc = fmaf(a.w, w0.w, acc);
-              acc = fmaf(b.x, w1.x, acc);
-              acc = fmaf(b.y, w1.y, acc);
-              acc = fmaf(b.z, w1.z, acc);
-              acc = fmaf(b.w, w1.w, acc);
-              tacc[c] = acc;
+            for (int c = 0; c < TC_TAILMAX; ++c) {
+              if (c < p.tail) {
+                const float4 w0 = *(const float4*)(sBt + c * TAIL_LD + k0 + 8 * kg);
+                const float4 w1 = *(const float4*)(sBt + c * TAIL_LD + k0 + 8 * kg + 4);
+                float acc = tacc[c];
+                acc = fmaf(a.x, w0.x, acc);
+                acc = fmaf(a.y, w0.y, acc);
+                acc = fmaf(a.z, w0.z, acc);
+                acc = fmaf(a.w, w0.w, acc);
+                acc = fmaf(b.x, w1.x, acc);
+                acc = fmaf(b.y, w1.y, acc);
+                acc = fmaf(b.z, w1.z, acc);
+                acc = fmaf(b.w, w1.w, acc);
+                tacc[c] = acc;
+              }
             }
           }
         }
+        __syncwarp();
+        issue();  // the ring slot just read is free again
+        if (++ds == ND) ds = 0;
+        if (!pollw(sfree(s), ph, fail)) {
+          ok = false;
+          break;
+        }
+        uint8_t* sA = smem + OFF_A + s * A_STAGE;
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+          const int off = (2 * hk + e) * A_LBO + (r >> 3) * 128 + (r & 7) * 16;
+          *(uint4*)(sA + off) = hi[e];
+          *(uint4*)(sA + A_TILE + off) = lo[e];
+        }
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        __syncwarp();
+        if (lane == 0) arrive(full(s));
+        if (++s == NS) {
+          s = 0;
+          ph ^= 1u;
+        }
       }
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-      __syncwarp();
-      if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(afull(s)) : "memory");
-      issue(g + ND);
-      if (TAIL && p.tail && kt == p.nk - 1) {
+      if (TAIL && p.tail && ok) {
         // the two k halves of a row are in lanes l and l + 16
 #pragma unroll
         for (int c = 0; c < TC_TAILMAX; ++c) tacc[c] += __shfl_xor_sync(0xffffffffu, tacc[c], 16);
-        const Item it = item(p, (int)blockIdx.x + (g / p.nk) * (int)gridDim.x);
+        const Item it = item_at(i);
         const int row = it.m0 + r;
         if (hk == 0 && row < p.M_total) {
           const int plane = row / p.R, rr = row - plane * p.R;
@@ -419,10 +467,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1) xform_tc_kernel(TcArgs p) {
     const int q = warp & 3, h = warp >> 2;
     float* stg = (float*)(smem + OFF_S) + warp * STG_FLOATS;
     for (int i = 0; i < nitems; ++i) {
-      const Item it = item(p, (int)blockIdx.x + i * (int)gridDim.x);
+      const Item it = item_at(i);
       const int b = i & 1, v = i >> 1;
-      if (!pollw(tfull(b), v & 1, fail, lane)) break;
-      asm volatile("tcgen05.fence::after_thread_sync;");
       const int row0 = it.m0 + 32 * q;
       const int row = row0 + lane;
       const bool live = row < p.M_total;
@@ -433,6 +479,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1) xform_tc_kernel(TcArgs p) {
         const int plane = row / p.R, rr = row - plane * p.R;
         obase = (int64_t)plane * p.ldo * p.P + rr;
       }
+      if (!pollw(tfull(b), v & 1, fail)) break;
+      asm volatile("tcgen05.fence::after_thread_sync;");
       // the tensor-memory load of the next chunk is in flight while a chunk is stored;
       // a chunk goes through the warp's staging area so that each store instruction writes
       // p.vec consecutive floats per lane (4 or 2 where the output pitch allows it)
@@ -530,7 +578,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) xform_tc_kernel(TcArgs p) {
       }
       asm volatile("tcgen05.fence::before_thread_sync;");
       __syncwarp();
-      if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tempty(b)) : "memory");
+      if (lane == 0) arrive(tempty(b));
     }
   }
 
@@ -654,7 +702,6 @@ void launch_xform_tc(const float* in, float* out, const uint8_t* W, int M_total,
   a.gcols = tc_gcols(P, K);
   a.tail = tc_tail(P, K);
   a.Bt = a.tail ? (const float*)(W + tc_tile_bytes(P, K)) : nullptr;
-  a.nwork = ((M_total + TC_M - 1) / TC_M) * a.ngroups;
   a.err = err;
   {
     // transposed: a lane stores vec consecutive rows of a column (R % vec == 0, so they
@@ -666,9 +713,10 @@ void launch_xform_tc(const float* in, float* out, const uint8_t* W, int M_total,
     a.vec = (!transposed && a.ldo % 4 == 0 && oa % 16 == 0) ? 4 : 1;
     if (!transposed && a.ngroups > 1 && (a.gcols % a.vec)) a.vec = 1;
   }
-  if (a.nwork == 0) return;
+  if (M_total <= 0) return;
   static int sms = 0;
   if (!sms) sms = device_sm_count();
+  a.nwork = ((M_total + TC_M - 1) / TC_M) * a.ngroups;
   const unsigned grid = (unsigned)std::min(a.nwork, sms);
   note_launch();
   const uintptr_t ia = (uintptr_t)in;
