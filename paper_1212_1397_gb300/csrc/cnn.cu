@@ -16,14 +16,15 @@
 //                   pre-activations kept) and its input gradients (the transpose of a
 //                   zero-padded correlation is the correlation with the flipped,
 //                   channel-transposed taps; the FP32 gradient split into BF16 hi + lo)
-//   wgrad_kernel    weight and bias gradients (SIMT, 32x4x2-point tiles with the input halo
-//                   staged in shared memory), block partials over persistent tiles
+//   wgrad_kernel    weight and bias gradients (SIMT, register tiles over 32x4x2-point tiles staged
+//                   with their halo in shared memory), block partials over persistent tiles
 //   mse_kernel, adam_kernel, prep_tc_kernel / prep_tcb_kernel (BF16 taps in the layouts the
 //   tensor-core kernel reads, from the master vector)
 #include <cuda_bf16.h>
 
 #include <cmath>
 #include <cstring>
+#include <type_traits>
 #include <utility>
 #include <vector>
 
@@ -38,12 +39,6 @@ constexpr int HX = TXc + 2, HY = TYc + 2, HZ = TZc + 2, HP = HX * HY * HZ;
 constexpr int NL = 4;
 // channels entering layer l (l = 0..3) and leaving the last one (l = 4)
 __host__ __device__ constexpr int ch(int l) { return (l == 0 || l == NL) ? 2 : 16; }
-
-// halo floats per point (16 channels padded to 20: conflict-free 16-byte shared loads)
-template <int C>
-struct PStride {
-  static constexpr int v = (C == 16) ? 20 : C;
-};
 
 // IN_G32 (tensor-core kernel only): FP32 gradients split into BF16 hi + lo operand copies
 enum { IN_F32 = 0, IN_BF16 = 1, IN_PLANAR = 2, IN_G32 = 3 };
@@ -85,117 +80,184 @@ __device__ __forceinline__ void tile_origin(const ConvArgs& a, int64_t tile, int
   z0 = bz * TZc;
 }
 
-// Stage the input halo of one tile into sx (HP points x PStride<CIN> floats).
-template <int CIN, int IN>
-__device__ __forceinline__ void load_halo(const ConvArgs& a, int img, int z0, int y0, int x0, float* sx) {
-  constexpr int PS = PStride<CIN>::v;
-  for (int i = threadIdx.x; i < HP; i += NT) {
-    const int hx = i % HX, r = i / HX, hy = r % HY, hz = r / HY;
-    const int gx = x0 + hx - 1, gy = y0 + hy - 1, gz = z0 + hz - 1;
-    const bool ok = gx >= 0 && gx < a.nx && gy >= 0 && gy < a.ny && gz >= 0 && gz < a.nz;
-    const int64_t p = (((int64_t)img * a.nz + gz) * a.ny + gy) * a.nx + gx;
-    float* d = sx + i * PS;
-    if constexpr (IN == IN_BF16) {
-      static_assert(IN != IN_BF16 || CIN == 16, "BF16 activations carry 16 channels");
-      uint4 q0 = make_uint4(0, 0, 0, 0), q1 = q0;
-      if (ok) {
-        const uint4* s = (const uint4*)a.in + 2 * p;
-        q0 = s[0];
-        q1 = s[1];
-      }
-      float4* d4 = (float4*)d;
-      d4[0] = make_float4(bf16_lo(q0.x), bf16_hi(q0.x), bf16_lo(q0.y), bf16_hi(q0.y));
-      d4[1] = make_float4(bf16_lo(q0.z), bf16_hi(q0.z), bf16_lo(q0.w), bf16_hi(q0.w));
-      d4[2] = make_float4(bf16_lo(q1.x), bf16_hi(q1.x), bf16_lo(q1.y), bf16_hi(q1.y));
-      d4[3] = make_float4(bf16_lo(q1.z), bf16_hi(q1.z), bf16_lo(q1.w), bf16_hi(q1.w));
-    } else {
-      const float* f = (const float*)a.in + p * CIN;
-      if constexpr (CIN == 16) {
-        float4* d4 = (float4*)d;
+// Weight and bias gradients of one layer: dW[t][ci][co] = sum_p in[p + d_t][ci] g[p][co],
+// db[co] = sum_p g[p][co].  Persistent blocks over tiles, one partial row per block.
+//
+// Bound by the FP32 pipe (27 c_in c_out multiply-adds per point), provided that shared memory
+// keeps up: it delivers one warp-wide word per clock where the pipe takes four multiply-adds.  So a
+// warp takes one (dz, dy) and all three dx: a thread holds 3 x CT x OT sums in registers, slides a
+// three-point window of CT input channels along a row of the tile, and one point costs it two vector
+// loads for 3 CT OT multiply-adds (48 at 16 x 16 channels; one output entry per thread and
+// iteration, as before, cost two loads per multiply-add).  Lanes with the same sums take different
+// rows; rows are padded to odd pitches, so neighbouring ones lie in different halves of the banks.
+// 32 images of 32^3: 16 x 16 channels 878 -> 340 us, 2 x 16 322 -> 81 us (ncu);
+// the whole gradient call 4.10 -> 2.38 ms.
+template <int CIN, int COUT>
+struct WgTile {
+  static constexpr int CT = CIN < 4 ? CIN : 4, OT = COUT < 4 ? COUT : 4;  // a thread's channels
+  static constexpr int NCO = COUT / OT, LG = (CIN / CT) * NCO;            // lanes that cover all channels
+  static constexpr int RS = 32 / LG;                                      // rows of the tile a warp takes at a time
+  static constexpr int PX = HX + 1, PG = TXc + 1;                         // row pitches (points), odd
+  static constexpr int XF = HY * HZ * PX * CIN, GF = TYc * TZc * PG * COUT;
+  static constexpr int PER_SM = CIN * COUT == 256 ? 2 : 3;  // blocks an SM holds (registers)
+  static constexpr size_t smem = sizeof(float) * (XF + GF);
+};
+constexpr int NTW = 288;  // nine warps: the (dz, dy) taps
+
+template <int N>
+__device__ __forceinline__ void ldv(const float* p, float (&v)[N]) {
+  if constexpr (N == 4) {
+    const float4 q = *(const float4*)p;
+    v[0] = q.x, v[1] = q.y, v[2] = q.z, v[3] = q.w;
+  } else {
+    static_assert(N == 2, "two or four channels");
+    const float2 q = *(const float2*)p;
+    v[0] = q.x, v[1] = q.y;
+  }
+}
+
+template <int CIN, int COUT, int IN>
+__global__ void __launch_bounds__(NTW, WgTile<CIN, COUT>::PER_SM)
+    wgrad_kernel(ConvArgs a, const float* __restrict__ g, float* __restrict__ partial, int64_t ntiles) {
+  using T = WgTile<CIN, COUT>;
+  constexpr int CT = T::CT, OT = T::OT, E = 27 * CIN * COUT;
+  extern __shared__ __align__(16) float smem[];
+  float* sx = smem;          // [HZ][HY][PX][CIN]
+  float* sg = smem + T::XF;  // [TZc * TYc][PG][COUT]
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int dz = warp / 3, dy = warp % 3;
+  const int rs = lane / T::LG, lg = lane % T::LG;
+  const int ci0 = (lg / T::NCO) * CT, co0 = (lg % T::NCO) * OT;
+  float acc[3][CT][OT];
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          float4 v = ok ? ((const float4*)f)[c] : make_float4(0.f, 0.f, 0.f, 0.f);
-          if (a.round_in) v = make_float4(bf16r(v.x), bf16r(v.y), bf16r(v.z), bf16r(v.w));
-          d4[c] = v;
-        }
+  for (int d = 0; d < 3; ++d)
+#pragma unroll
+    for (int c = 0; c < CT; ++c)
+#pragma unroll
+      for (int o = 0; o < OT; ++o) acc[d][c][o] = 0.f;
+  float bacc = 0.f;  // threads 0 .. NT-1: output channel tid % COUT, points tid / COUT, + NT / COUT, ...
+  for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+    int img, z0, y0, x0;
+    tile_origin(a, tile, img, z0, y0, x0);
+    // the tile's input with its halo, and its gradients
+    constexpr int PARTS = CIN == 16 ? 2 : 1;  // pieces of a point: 8 BF16 channels or 2 FP32 ones
+    for (int i = tid; i < HP * PARTS; i += NTW) {
+      const int h = i / PARTS, part = i % PARTS;
+      const int hx = h % HX, r = h / HX, hy = r % HY, hz = r / HY;
+      const int gx = x0 + hx - 1, gy = y0 + hy - 1, gz = z0 + hz - 1;
+      const bool ok = gx >= 0 && gx < a.nx && gy >= 0 && gy < a.ny && gz >= 0 && gz < a.nz;
+      const int64_t p = (((int64_t)img * a.nz + gz) * a.ny + gy) * a.nx + gx;
+      float* d = sx + ((size_t)r * T::PX + hx) * CIN + 8 * part;
+      if constexpr (IN == IN_BF16) {
+        static_assert(IN != IN_BF16 || CIN == 16, "BF16 activations carry 16 channels");
+        uint4 q = make_uint4(0, 0, 0, 0);
+        if (ok) q = ((const uint4*)a.in)[2 * p + part];
+        ((float4*)d)[0] = make_float4(bf16_lo(q.x), bf16_hi(q.x), bf16_lo(q.y), bf16_hi(q.y));
+        ((float4*)d)[1] = make_float4(bf16_lo(q.z), bf16_hi(q.z), bf16_lo(q.w), bf16_hi(q.w));
       } else {
+        static_assert(IN == IN_BF16 || CIN == 2, "FP32 input has two channels");
+        const float* f = (const float*)a.in + p * CIN;
 #pragma unroll
-        for (int c = 0; c < CIN; ++c) {
+        for (int c = 0; c < 2; ++c) {
           const float v = ok ? f[c] : 0.f;
           d[c] = a.round_in ? bf16r(v) : v;
         }
       }
     }
-  }
-}
-
-// Weight and bias gradients of one layer: dW[t][ci][co] = sum_p in[p + d_t][ci] g[p][co],
-// db[co] = sum_p g[p][co].  Persistent blocks over tiles, one partial row per block.
-template <int CIN, int COUT, int IN>
-__global__ void __launch_bounds__(NT) wgrad_kernel(ConvArgs a, const float* __restrict__ g,
-                                                   float* __restrict__ partial, int64_t ntiles) {
-  extern __shared__ __align__(16) float smem[];
-  constexpr int PS = PStride<CIN>::v;
-  constexpr int E = 27 * CIN * COUT;
-  constexpr int KE = (E + NT - 1) / NT;
-  float* sx = smem;            // HP * PS
-  float* sg = smem + HP * PS;  // NT * COUT
-  const int tid = threadIdx.x;
-  int xo[KE], go[KE];
-  float acc[KE];
-#pragma unroll
-  for (int k = 0; k < KE; ++k) {
-    const int e = (tid + k * NT < E) ? tid + k * NT : 0;  // entries past E read entry 0, unused
-    const int t = e / (CIN * COUT), r = e % (CIN * COUT);
-    const int ci = r / COUT, co = r % COUT;
-    const int dz = t / 9, dy = (t / 3) % 3, dx = t % 3;
-    xo[k] = ((dz * HY + dy) * HX + dx) * PS + ci;
-    go[k] = co;
-    acc[k] = 0.f;
-  }
-  float bacc = 0.f;
-  for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-    int img, z0, y0, x0;
-    tile_origin(a, tile, img, z0, y0, x0);
-    load_halo<CIN, IN>(a, img, z0, y0, x0, sx);
-    {
-      const int lx = tid % TXc, ly = (tid / TXc) % TYc, lz = tid / (TXc * TYc);
-      const int gx = x0 + lx, gy = y0 + ly, gz = z0 + lz;
+    constexpr int GP = COUT / OT;
+    for (int i = tid; i < NT * GP; i += NTW) {
+      const int q = i / GP, part = i % GP;
+      const int lx = q % TXc, row = q / TXc;
+      const int gx = x0 + lx, gy = y0 + row % TYc, gz = z0 + row / TYc;
       const bool ok = gx < a.nx && gy < a.ny && gz < a.nz;
       const int64_t p = (((int64_t)img * a.nz + gz) * a.ny + gy) * a.nx + gx;
+      float v[OT];
 #pragma unroll
-      for (int c = 0; c < COUT; ++c) sg[tid * COUT + c] = ok ? g[p * COUT + c] : 0.f;
+      for (int o = 0; o < OT; ++o) v[o] = 0.f;
+      if (ok) ldv<OT>(g + p * COUT + OT * part, v);
+      float* d = sg + ((size_t)row * T::PG + lx) * COUT + OT * part;
+      if constexpr (OT == 4)
+        *(float4*)d = make_float4(v[0], v[1], v[2], v[3]);
+      else
+        *(float2*)d = make_float2(v[0], v[1]);
     }
     __syncthreads();
-#pragma unroll 2
-    for (int q = 0; q < NT; ++q) {
-      const int hb = ((q / (TXc * TYc)) * HY + (q / TXc) % TYc) * HX + q % TXc;
-      const float* xq = sx + hb * PS;
-      const float* gq = sg + q * COUT;
+    const int xlim = min(TXc, a.nx - x0);
+    for (int row = rs; row < TYc * TZc; row += T::RS) {
+      const float* xi = sx + (((row / TYc + dz) * HY + row % TYc + dy) * T::PX) * CIN + ci0;
+      const float* gi = sg + row * T::PG * COUT + co0;
+      float w[3][CT];
+      ldv<CT>(xi, w[0]);
+      ldv<CT>(xi + CIN, w[1]);
+      auto step = [&](int x, auto J) {  // J = x % 3: the window's first point
+        constexpr int j = decltype(J)::value;
+        float gv[OT];
+        ldv<CT>(xi + (x + 2) * CIN, w[(j + 2) % 3]);
+        ldv<OT>(gi + x * COUT, gv);
 #pragma unroll
-      for (int k = 0; k < KE; ++k)
-        if (KE * NT == E || tid + k * NT < E) acc[k] = fmaf(xq[xo[k]], gq[go[k]], acc[k]);
+        for (int d = 0; d < 3; ++d)
+#pragma unroll
+          for (int c = 0; c < CT; ++c)
+#pragma unroll
+            for (int o = 0; o < OT; ++o) acc[d][c][o] = fmaf(w[(j + d) % 3][c], gv[o], acc[d][c][o]);
+      };
+      int x = 0;
+#pragma unroll 2
+      for (; x + 3 <= xlim; x += 3) {
+        step(x, std::integral_constant<int, 0>{});
+        step(x + 1, std::integral_constant<int, 1>{});
+        step(x + 2, std::integral_constant<int, 2>{});
+      }
+      if (x < xlim) step(x, std::integral_constant<int, 0>{});
+      if (x + 1 < xlim) step(x + 1, std::integral_constant<int, 1>{});
     }
-    if (tid < COUT)
-      for (int q = 0; q < NT; ++q) bacc += sg[q * COUT + tid];
+    if (tid < NT) {
+#pragma unroll 4
+      for (int q = tid / COUT; q < NT; q += NT / COUT) bacc += sg[((q / TXc) * T::PG + q % TXc) * COUT + tid % COUT];
+    }
     __syncthreads();
   }
   float* row = partial + (int64_t)blockIdx.x * (E + COUT);
 #pragma unroll
-  for (int k = 0; k < KE; ++k)
-    if (tid + k * NT < E) row[tid + k * NT] = acc[k];
-  if (tid < COUT) row[E + tid] = bacc;
+  for (int d = 0; d < 3; ++d)
+#pragma unroll
+    for (int c = 0; c < CT; ++c)
+#pragma unroll
+      for (int o = 0; o < OT; ++o) {
+        float v = acc[d][c][o];
+#pragma unroll
+        for (int m = T::LG; m < 32; m *= 2) v += __shfl_xor_sync(0xffffffffu, v, m);
+        if (rs == 0) row[((warp * 3 + d) * CIN + ci0 + c) * COUT + co0 + o] = v;
+      }
+  if (tid < NT) smem[tid] = bacc;  // (the tile buffers are free: every loop ends on a barrier)
+  __syncthreads();
+  if (tid < COUT) {
+    float v = 0.f;
+    for (int q = tid; q < NT; q += COUT) v += smem[q];
+    row[E + tid] = v;
+  }
 }
 
 // grad[flat] = sum over blocks of the partial rows, entries mapped from the kernel's
-// [t][ci][co] order to the parameter vector's [co][ci][t] order; biases follow.
-__global__ void wgrad_reduce_kernel(const float* __restrict__ partial, int nblk, int cin, int cout,
-                                    float* __restrict__ grad_w, float* __restrict__ grad_b) {
-  const int E = 27 * cin * cout;
-  const int e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= E + cout) return;
+// [t][ci][co] order to the parameter vector's [co][ci][t] order; biases follow.  A block sums 32
+// entries, its eight warps every eighth row each (a thread alone per entry waited for one row
+// after the other: 51 us for the 6928 x 304 sums of a 16 x 16 layer, 15 this way).
+constexpr int WR_WARPS = 8;
+__global__ void __launch_bounds__(32 * WR_WARPS)
+    wgrad_reduce_kernel(const float* __restrict__ partial, int nblk, int cin, int cout, float* __restrict__ grad_w,
+                        float* __restrict__ grad_b) {
+  __shared__ double part[WR_WARPS][32];
+  const int E = 27 * cin * cout, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int e = blockIdx.x * 32 + lane;
   double s = 0.0;
-  for (int b = 0; b < nblk; ++b) s += partial[(int64_t)b * (E + cout) + e];
+  if (e < E + cout) {
+#pragma unroll 8
+    for (int b = warp; b < nblk; b += WR_WARPS) s += partial[(int64_t)b * (E + cout) + e];
+  }
+  part[warp][lane] = s;
+  __syncthreads();
+  if (warp || e >= E + cout) return;
+  for (int w = 1; w < WR_WARPS; ++w) s += part[w][lane];
   if (e < E) {
     const int t = e / (cin * cout), r = e % (cin * cout), ci = r / cout, co = r % cout;
     grad_w[(co * cin + ci) * 27 + t] = (float)s;
@@ -638,14 +700,17 @@ __host__ __device__ inline LayerDims layer_dims() {
 constexpr int kWeights = 27 * (2 * 16 + 16 * 16 + 16 * 16 + 16 * 2);  // 15552 taps
 static_assert(kWeights + 16 + 16 + 16 + 2 == HELM6_CNN_NPARAMS, "parameter count");
 
+// blocks of a layer's weight gradient: what the SMs hold, at most one per tile
 template <int CIN, int COUT>
-constexpr size_t wgrad_smem() {
-  return sizeof(float) * (HP * PStride<CIN>::v + NT * COUT);
+int wgrad_blocks(const ConvArgs& a) {
+  const int64_t tiles = (int64_t)a.tx * a.ty * a.tz * a.nb;
+  return (int)std::min<int64_t>(tiles, (int64_t)WgTile<CIN, COUT>::PER_SM * device_sm_count());
 }
 
 template <int CIN, int COUT, int IN>
-cudaError_t launch_wgrad(const ConvArgs& a, const float* g, float* partial, int nblk, cudaStream_t s) {
-  const size_t sm = wgrad_smem<CIN, COUT>();
+cudaError_t launch_wgrad(const ConvArgs& a, const float* g, float* partial, float* grad_w, float* grad_b,
+                         cudaStream_t s) {
+  constexpr size_t sm = WgTile<CIN, COUT>::smem;
   static bool configured = false;
   if (!configured) {
     cudaError_t e =
@@ -654,8 +719,11 @@ cudaError_t launch_wgrad(const ConvArgs& a, const float* g, float* partial, int 
     configured = true;
   }
   const int64_t tiles = (int64_t)a.tx * a.ty * a.tz * a.nb;
-  note_launch();
-  wgrad_kernel<CIN, COUT, IN><<<nblk, NT, sm, s>>>(a, g, partial, tiles);
+  const int nblk = wgrad_blocks<CIN, COUT>(a);
+  note_launch(2);
+  wgrad_kernel<CIN, COUT, IN><<<nblk, NTW, sm, s>>>(a, g, partial, tiles);
+  wgrad_reduce_kernel<<<(27 * CIN * COUT + COUT + 31) / 32, 32 * WR_WARPS, 0, s>>>(partial, nblk, CIN, COUT, grad_w,
+                                                                                  grad_b);
   return cudaGetLastError();
 }
 
@@ -848,12 +916,6 @@ int tr_backward(helm6_cnn_trainer* tr, const float* x, const float* target) {
   }
   launch_reduce_sum(tr->lpart, tr->nloss, tr->loss, s);
   ConvArgs a = vol_args(tr->nb, tr->nz, tr->ny, tr->nx);
-  auto reduce = [&](int l) {
-    note_launch();
-    const int ne = 27 * d.cin[l] * d.cout[l] + d.cout[l];
-    wgrad_reduce_kernel<<<(ne + 255) / 256, 256, 0, s>>>(tr->partial, tr->nblk, d.cin[l], d.cout[l],
-                                                         tr->grad + d.toff[l], tr->grad + d.boff[l]);
-  };
   // input gradients on the tensor cores (the FP32 gradient split into BF16 hi + lo), weight
   // gradients by the SIMT reduction kernel
   TcConvArgs t = tr_tc_args(tr);
@@ -861,8 +923,8 @@ int tr_backward(helm6_cnn_trainer* tr, const float* x, const float* target) {
   t.bias = nullptr;
   // layer 4: dW from act3 and g4; g3 = (W4^T * g4) gelu'(pre3)
   a.in = tr->act[2];
-  if (launch_wgrad<16, 2, IN_BF16>(a, tr->g4, tr->partial, tr->nblk, s) != cudaSuccess) return HELM6_ERR_CUDA;
-  reduce(3);
+  if (launch_wgrad<16, 2, IN_BF16>(a, tr->g4, tr->partial, tr->grad + d.toff[3], tr->grad + d.boff[3], s) != cudaSuccess)
+    return HELM6_ERR_CUDA;
   t.in = tr->g4;
   t.cin = 2;
   t.w = tr->net.wtcb + (size_t)3 * 27 * 256;
@@ -875,8 +937,8 @@ int tr_backward(helm6_cnn_trainer* tr, const float* x, const float* target) {
   float* gnext = tr->gb;
   for (int l = 2; l >= 1; --l) {
     a.in = tr->act[l - 1];
-    if (launch_wgrad<16, 16, IN_BF16>(a, gcur, tr->partial, tr->nblk, s) != cudaSuccess) return HELM6_ERR_CUDA;
-    reduce(l);
+    if (launch_wgrad<16, 16, IN_BF16>(a, gcur, tr->partial, tr->grad + d.toff[l], tr->grad + d.boff[l], s) != cudaSuccess)
+      return HELM6_ERR_CUDA;
     t.in = gcur;
     t.cin = 16;
     t.w = tr->net.wtcb + (size_t)l * 27 * 256;
@@ -889,8 +951,8 @@ int tr_backward(helm6_cnn_trainer* tr, const float* x, const float* target) {
   // layer 1: dW from the BF16-rounded input and g1
   a.in = x;
   a.round_in = 1;
-  if (launch_wgrad<2, 16, IN_F32>(a, gcur, tr->partial, tr->nblk, s) != cudaSuccess) return HELM6_ERR_CUDA;
-  reduce(0);
+  if (launch_wgrad<2, 16, IN_F32>(a, gcur, tr->partial, tr->grad + d.toff[0], tr->grad + d.boff[0], s) != cudaSuccess)
+    return HELM6_ERR_CUDA;
   return HELM6_OK;
 }
 
