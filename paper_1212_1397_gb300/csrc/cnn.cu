@@ -385,14 +385,22 @@ __global__ void resid_loss_kernel(int nb, int nz, int ny, int nx, const float* _
 // every image face): its forward layers (FP32 pre-activations kept) and the input gradients
 // of the backward pass, whose FP32 gradient operand is split into BF16 hi + lo copies (two
 // more channel planes; 54 MMAs per tile) so that it keeps FP32-like accuracy.
-constexpr int BX = 30, BY = 4, BZ = 4;                       // output points of a brick
-constexpr int GX = BX + 2, GY = BY + 2, GZ = BZ + 2, GP = GX * GY * GZ;  // halo (GX = 32)
-constexpr int TC_TILES = BZ * BY / 4;                         // 128-point tiles of a brick
-constexpr int TC_TMEM = TC_TILES * 16 <= 32 ? 32 : TC_TILES * 16 <= 64 ? 64 : 128;  // TMEM columns
-constexpr int PLANE_B = (GP + 2) * 16;                        // one point of padding each end
+constexpr int BX = 30, BY = 4, BZ = 4;       // output points of a brick
+constexpr int GX = BX + 2, GY = BY + 2, GZ = BZ + 2;  // its halo (GX = 32)
+constexpr int RUN_NX = 32;                   // widest image that is taken in runs
+constexpr int LMAX = 128 + 2 * (RUN_NX + 2);  // halo points of a plane: GX GY = 192 (brick), at most 196 (run)
+static_assert(LMAX >= GX * GY && BY * GX == 128, "one 128-point tile per plane");
+constexpr int TC_TILES = BZ;                 // 128-point tiles of a CTA, one per plane
+constexpr int TC_TMEM = 64;                  // TMEM columns: 16 per tile
+constexpr int PLANE_B = (LMAX * GZ + 2) * 16;  // one point of padding each end
 constexpr int TCW_TAP = 512;                                  // bytes of one tap's 16 x 16 BF16
-constexpr size_t TC_SMEM = 1024 + 2 * (size_t)PLANE_B + 27 * TCW_TAP + 256;
-constexpr size_t TC_SMEM4 = 1024 + 4 * (size_t)PLANE_B + 27 * TCW_TAP + 256;  // IN_G32: hi and lo planes
+constexpr size_t TC_SMEM = 1024 + 2 * (size_t)PLANE_B + 27 * TCW_TAP + 64 + 8 * LMAX;
+constexpr size_t TC_SMEM4 = 1024 + 4 * (size_t)PLANE_B + 27 * TCW_TAP + 64 + 8 * LMAX;  // IN_G32: hi and lo planes
+// threads of a CTA: with four planes two CTAs share an SM, with two planes four
+template <int IN>
+constexpr int conv_threads() {
+  return IN == IN_G32 ? 256 : 128;
+}
 constexpr int kConvPolls = 1 << 22;
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -420,7 +428,8 @@ __device__ __forceinline__ void cp16(uint32_t dst, const void* src, bool ok) {
 struct TcConvArgs {
   int nb;                // images (1 for the field path)
   int nz, ny, nx;        // size of an image
-  int bx, by, bz;        // bricks per axis of an image
+  int bx, by, bz;        // bricks per axis of an image, or (run) by runs per plane, bx = 1
+  int run;               // whether a CTA takes runs of points rather than a brick
   const void* in;        // IN_BF16: [N][16] BF16; IN_PLANAR: planar FP32 complex field;
                          // IN_F32 (rounded to BF16) / IN_G32: [N][cin] FP32, channel-last
   int cin;               // IN_F32 / IN_G32: input channels (2 or 16)
@@ -435,18 +444,19 @@ struct TcConvArgs {
 };
 
 template <int IN, int OUT>
-__global__ void __launch_bounds__(128) conv_tc_kernel(TcConvArgs a) {
+__global__ void __launch_bounds__(conv_threads<IN>()) conv_tc_kernel(TcConvArgs a) {
   extern __shared__ uint8_t smem_raw[];
   constexpr int NPL = IN == IN_G32 ? 4 : 2;  // channel planes: 0-7, 8-15 (hi), then lo
+  constexpr int NTH = conv_threads<IN>();
   uint8_t* sm = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   uint8_t* plane0 = sm + 16;               // point -1 at sm, point 0 at sm + 16
-  uint8_t* plane1 = plane0 + PLANE_B;
   uint8_t* wts = sm + NPL * PLANE_B;       // 27 x 512 B (1024-aligned base + NPL * PLANE_B: 16-aligned)
   uint64_t* bar = (uint64_t*)(wts + 27 * TCW_TAP);
   uint32_t* tslot = (uint32_t*)(bar + 1);
   int* fail = (int*)(tslot + 1);
+  int64_t* tab = (int64_t*)(wts + 27 * TCW_TAP + 64);  // point of an image's plane at a halo position, or -1
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int64_t npts = (int64_t)a.nz * a.ny * a.nx;
+  const int64_t npts = (int64_t)a.nz * a.ny * a.nx, plane_pts = (int64_t)a.ny * a.nx;
 
   int64_t b = blockIdx.x;
   const int ibx = (int)(b % a.bx);
@@ -455,72 +465,102 @@ __global__ void __launch_bounds__(128) conv_tc_kernel(TcConvArgs a) {
   b /= a.by;
   const int ibz = (int)(b % a.bz);
   const int64_t img = b / a.bz;
-  const int x0 = ibx * BX - 1, y0 = iby * BY - 1, z0 = ibz * BZ - 1;  // global coordinate of halo (0,0,0)
+  const int z0 = ibz * BZ - 1;  // plane of halo plane 0
+  // halo positions of a plane: `len` of them, row pitch `pitch`; the tile's first output at `base`
+  const int len = a.run ? 128 + 2 * (a.nx + 2) : GX * GY, pitch = a.run ? a.nx + 1 : GX, base = a.run ? a.nx + 2 : GX;
 
   // weights: 27 x 512 B
-  for (int i = tid; i < 27 * TCW_TAP / 16; i += 128) cp16(smem_u32(wts) + 16u * i, (const uint4*)a.w + i, true);
-  // halo planes
-  float sc = 1.f;
+  for (int i = tid; i < 27 * TCW_TAP / 16; i += NTH) cp16(smem_u32(wts) + 16u * i, (const uint4*)a.w + i, true);
+  for (int l = tid; l < len; l += NTH) {
+    int64_t gx, gy;
+    if (a.run) {
+      const int64_t q = (int64_t)iby * 128 - base + l;  // rows of nx points and one zero
+      gy = q >= 0 ? q / pitch : -1;
+      gx = q - gy * pitch;
+    } else {
+      gx = ibx * BX - 1 + l % GX;
+      gy = iby * BY - 1 + l / GX;
+    }
+    tab[l] = gx >= 0 && gx < a.nx && gy >= 0 && gy < a.ny ? gy * a.nx + gx : -1;
+  }
+  __syncthreads();
+  // halo planes: consecutive lanes on consecutive 16-byte pieces of the image
   if constexpr (IN == IN_PLANAR) {
     const double ss = *a.sumsq;
-    sc = ss > 0.0 ? (float)(1.0 / sqrt(ss / (double)npts)) : 0.f;
-  }
-  if constexpr (IN == IN_PLANAR) {
-    // the planar FP32 field: every load of the thread's halo points issued before any is used
-    constexpr int PER = (GP + 127) / 128;
+    const float sc = ss > 0.0 ? (float)(1.0 / sqrt(ss / (double)npts)) : 0.f;
     const float* f = (const float*)a.in;
-    float re[PER], im[PER];
+    for (int l = tid; l < len; l += NTH) {
+      const int64_t t = tab[l];
+      float re[GZ], im[GZ];
 #pragma unroll
-    for (int k = 0; k < PER; ++k) {
-      const int i = tid + 128 * k;
-      const int hx = i % GX, r = i / GX, hy = r % GY, hz = r / GY;
-      const int gx = x0 + hx, gy = y0 + hy, gz = z0 + hz;
-      const bool ok = i < GP && gx >= 0 && gx < a.nx && gy >= 0 && gy < a.ny && gz >= 0 && gz < a.nz;
-      const int64_t p = ok ? ((img * a.nz + gz) * a.ny + gy) * a.nx + gx : 0;
-      re[k] = ok ? f[p] : 0.f;
-      im[k] = ok ? f[npts + p] : 0.f;
-    }
+      for (int hz = 0; hz < GZ; ++hz) {
+        const int gz = z0 + hz;
+        const bool ok = t >= 0 && gz >= 0 && gz < a.nz;
+        const int64_t p = (img * a.nz + gz) * plane_pts + t;
+        re[hz] = ok ? f[p] : 0.f;
+        im[hz] = ok ? f[npts + p] : 0.f;
+      }
 #pragma unroll
-    for (int k = 0; k < PER; ++k) {
-      const int i = tid + 128 * k;
-      if (i < GP) {
-        *(uint4*)(plane0 + 16 * i) = make_uint4(pack_bf16(re[k] * sc, im[k] * sc), 0u, 0u, 0u);
-        *(uint4*)(plane1 + 16 * i) = make_uint4(0u, 0u, 0u, 0u);
+      for (int hz = 0; hz < GZ; ++hz) {
+        uint8_t* d = plane0 + 16 * (hz * len + l);
+        *(uint4*)d = make_uint4(pack_bf16(re[hz] * sc, im[hz] * sc), 0u, 0u, 0u);
+        *(uint4*)(d + PLANE_B) = make_uint4(0u, 0u, 0u, 0u);
       }
     }
-  }
-  for (int i = tid; i < GP && IN != IN_PLANAR; i += 128) {
-    const int hx = i % GX, r = i / GX, hy = r % GY, hz = r / GY;
-    const int gx = x0 + hx, gy = y0 + hy, gz = z0 + hz;
-    const bool ok = gx >= 0 && gx < a.nx && gy >= 0 && gy < a.ny && gz >= 0 && gz < a.nz;
-    const int64_t p = ok ? ((img * a.nz + gz) * a.ny + gy) * a.nx + gx : 0;
-    if constexpr (IN == IN_BF16) {
-      const uint4* src = (const uint4*)a.in + 2 * p;
-      cp16(smem_u32(plane0) + 16u * i, src, ok);
-      cp16(smem_u32(plane1) + 16u * i, src + 1, ok);
-    } else if constexpr (IN == IN_F32 || IN == IN_G32) {
-      // channel-last FP32: BF16 (IN_F32), or BF16 hi + lo = the value to 16 bits (IN_G32)
-      const float* f = (const float*)a.in + p * a.cin;
-      float v[16];
+  } else if constexpr (IN == IN_BF16) {
+    const int half = tid & 1;
+    for (int l = tid >> 1; l < len; l += NTH / 2) {
+      const int64_t t = tab[l];
 #pragma unroll
-      for (int c = 0; c < 16; ++c) v[c] = (ok && c < a.cin) ? f[c] : 0.f;
-      uint32_t hi[8], lo[8];
-#pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        hi[q] = pack_bf16(v[2 * q], v[2 * q + 1]);
-        lo[q] = pack_bf16(v[2 * q] - bf16_lo(hi[q]), v[2 * q + 1] - bf16_hi(hi[q]));
+      for (int hz = 0; hz < GZ; ++hz) {
+        const int gz = z0 + hz;
+        const bool ok = t >= 0 && gz >= 0 && gz < a.nz;
+        const int64_t p = ok ? (img * a.nz + gz) * plane_pts + t : 0;
+        cp16(smem_u32(plane0) + (uint32_t)(half * PLANE_B + 16 * (hz * len + l)), (const uint4*)a.in + 2 * p + half, ok);
       }
-      *(uint4*)(plane0 + 16 * i) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
-      *(uint4*)(plane1 + 16 * i) = make_uint4(hi[4], hi[5], hi[6], hi[7]);
-      if constexpr (IN == IN_G32) {
-        *(uint4*)(plane0 + 2 * PLANE_B + 16 * i) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
-        *(uint4*)(plane0 + 3 * PLANE_B + 16 * i) = make_uint4(lo[4], lo[5], lo[6], lo[7]);
+    }
+  } else {
+    // channel-last FP32: BF16 (IN_F32), or BF16 hi + lo = the value to 16 bits (IN_G32); four channels
+    // of a point per thread where it has 16, else both of them and the zeros
+    const bool wide = a.cin == 16;
+    const int part = wide ? tid & 3 : 0;
+    for (int l = wide ? tid >> 2 : tid; l < len; l += wide ? NTH / 4 : NTH) {
+      const int64_t t = tab[l];
+      float4 v[GZ];
+#pragma unroll
+      for (int hz = 0; hz < GZ; ++hz) {
+        const int gz = z0 + hz;
+        const bool ok = t >= 0 && gz >= 0 && gz < a.nz;
+        const int64_t p = (img * a.nz + gz) * plane_pts + t;
+        v[hz] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (ok && wide) v[hz] = ((const float4*)a.in)[4 * p + part];
+        if (ok && !wide) v[hz] = make_float4(((const float*)a.in)[2 * p], ((const float*)a.in)[2 * p + 1], 0.f, 0.f);
+      }
+#pragma unroll
+      for (int hz = 0; hz < GZ; ++hz) {
+        const float4 w = v[hz];
+        const uint32_t h0 = pack_bf16(w.x, w.y), h1 = pack_bf16(w.z, w.w);
+        const uint32_t l0 = pack_bf16(w.x - bf16_lo(h0), w.y - bf16_hi(h0));
+        const uint32_t l1 = pack_bf16(w.z - bf16_lo(h1), w.w - bf16_hi(h1));
+        uint8_t* d = plane0 + 16 * (hz * len + l);
+        if (wide) {
+          d += (part >> 1) * PLANE_B + 8 * (part & 1);
+          *(uint2*)d = make_uint2(h0, h1);
+          if constexpr (IN == IN_G32) *(uint2*)(d + 2 * PLANE_B) = make_uint2(l0, l1);
+        } else {
+          *(uint4*)d = make_uint4(h0, 0u, 0u, 0u);
+          *(uint4*)(d + PLANE_B) = make_uint4(0u, 0u, 0u, 0u);
+          if constexpr (IN == IN_G32) {
+            *(uint4*)(d + 2 * PLANE_B) = make_uint4(l0, 0u, 0u, 0u);
+            *(uint4*)(d + 3 * PLANE_B) = make_uint4(0u, 0u, 0u, 0u);
+          }
+        }
       }
     }
   }
   if (tid < NPL) {  // the padding points before and after each plane
     *(uint4*)(sm + tid * PLANE_B) = make_uint4(0u, 0u, 0u, 0u);
-    *(uint4*)(plane0 + tid * PLANE_B + 16 * GP) = make_uint4(0u, 0u, 0u, 0u);
+    *(uint4*)(plane0 + tid * PLANE_B + 16 * len * GZ) = make_uint4(0u, 0u, 0u, 0u);
   }
   if (tid == 0) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(1));
@@ -544,11 +584,10 @@ __global__ void __launch_bounds__(128) conv_tc_kernel(TcConvArgs a) {
     const uint32_t id = (1u << 4) | (1u << 7) | (1u << 10) | (2u << 17) | (8u << 24);
     const uint32_t p0 = smem_u32(plane0);
     for (int tile = 0; tile < TC_TILES; ++tile) {
-      const int hz = 1 + tile / (BY / 4), hy = 1 + 4 * (tile % (BY / 4));
-      const int q0 = (hz * GY + hy) * GX;
+      const int q0 = (1 + tile) * len + base;
       for (int t = 0; t < 27; ++t) {
         const int dz = t / 9 - 1, dy = (t / 3) % 3 - 1, dx = t % 3 - 1;
-        const int q = q0 + (dz * GY + dy) * GX + dx;  // in [-1, GP - 128]: the padding covers -1 and GP
+        const int q = q0 + dz * len + dy * pitch + dx;  // in [-1, len GZ - 127]: the padding covers -1 and len GZ
         const uint64_t ad = desc_noswz(p0 + (uint32_t)(q * 16), PLANE_B, 128);
         const uint64_t bd = desc_noswz(smem_u32(wts) + (uint32_t)(t * TCW_TAP), 128, 256);
         mma_bf16(tmem + 16u * tile, ad, bd, id, t > 0 ? 1u : 0u);
@@ -578,62 +617,71 @@ __global__ void __launch_bounds__(128) conv_tc_kernel(TcConvArgs a) {
   if (!ok) {
     *fail = 1;
   } else {
-    float bias[16];
+    float bias[4];  // of the lane's channels: 4 (lane & 3) .. + 3, or 0 and 1
 #pragma unroll
-    for (int c = 0; c < 16; ++c) bias[c] = (a.bias && (OUT == OUT_HIDDEN || c < 2)) ? a.bias[c] : 0.f;
+    for (int c = 0; c < 4; ++c) bias[c] = (a.bias && (OUT == OUT_HIDDEN || c < 2)) ? a.bias[(OUT == OUT_HIDDEN ? 4 * (lane & 3) : 0) + c] : 0.f;
     float cs = 0.f;
     if constexpr (OUT == OUT_FIELD) {
       const double ss = *a.sumsq;
       cs = ss > 0.0 ? a.out_scale * (float)sqrt(ss / (double)npts) : 0.f;
     }
-    for (int tile = 0; tile < TC_TILES; ++tile) {
+    // the products have read the halo: its place takes the warp's 32 x 16 results, so that the
+    // global accesses of 16-channel layers run over whole points (16-byte chunks swizzled by row)
+    uint8_t* stg = sm + warp * 2048;
+    for (int tile = warp >> 2; tile < TC_TILES; tile += NTH / 128) {
       uint32_t v[16];
       asm volatile(
           "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
           : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
             "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
-          : "r"(tmem + ((uint32_t)(32 * warp) << 16) + 16u * tile));
+          : "r"(tmem + ((uint32_t)(32 * (warp & 3)) << 16) + 16u * tile));
       asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-      const int r = 32 * warp + lane;  // row of the tile: halo x = r % 32, y = hy + r / 32
-      const int hx = r % GX, hz = 1 + tile / (BY / 4), hy = 1 + 4 * (tile % (BY / 4)) + r / GX;
-      const int gx = x0 + hx, gy = y0 + hy, gz = z0 + hz;
-      if (hx < 1 || hx > BX || gx >= a.nx || gy >= a.ny || gz >= a.nz) continue;
-      const int64_t p = ((img * a.nz + gz) * a.ny + gy) * a.nx + gx;
-      if constexpr (OUT == OUT_HIDDEN) {
-        if (a.pre) {
-          float4* pr = (float4*)(a.pre + p * 16);
+      const int gz = z0 + 1 + tile;
+      // row r of the tile: its point, or -1 (halo columns of a brick, beyond the image)
+      auto point = [&](int r) -> int64_t {
+        if (gz >= a.nz || (!a.run && (r % GX < 1 || r % GX > BX))) return -1;
+        const int64_t t = tab[base + r];
+        return t < 0 ? -1 : (img * a.nz + gz) * plane_pts + t;
+      };
+      if constexpr (OUT == OUT_HIDDEN || OUT == OUT_GRAD) {
+        __syncwarp();
 #pragma unroll
-          for (int q = 0; q < 4; ++q)
-            pr[q] = make_float4(__uint_as_float(v[4 * q]) + bias[4 * q], __uint_as_float(v[4 * q + 1]) + bias[4 * q + 1],
-                                __uint_as_float(v[4 * q + 2]) + bias[4 * q + 2],
-                                __uint_as_float(v[4 * q + 3]) + bias[4 * q + 3]);
-        }
-        uint32_t pk[8];
+        for (int q = 0; q < 4; ++q)
+          *(uint4*)(stg + lane * 64 + ((q ^ ((lane >> 1) & 3)) << 4)) =
+              make_uint4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+        __syncwarp();
+        const int q = lane & 3;  // this lane's four channels of rows lane / 4, + 8, ...
+        const float4 bq = make_float4(bias[0], bias[1], bias[2], bias[3]);
 #pragma unroll
-        for (int q = 0; q < 8; ++q)
-          pk[q] = pack_bf16(gelu_f(__uint_as_float(v[2 * q]) + bias[2 * q]),
-                            gelu_f(__uint_as_float(v[2 * q + 1]) + bias[2 * q + 1]));
-        uint4* o4 = (uint4*)a.out + 2 * p;
-        o4[0] = make_uint4(pk[0], pk[1], pk[2], pk[3]);
-        o4[1] = make_uint4(pk[4], pk[5], pk[6], pk[7]);
-      } else if constexpr (OUT == OUT_F32) {
-        float* o = (float*)a.out + p * 2;
-        o[0] = __uint_as_float(v[0]) + bias[0];
-        o[1] = __uint_as_float(v[1]) + bias[1];
-      } else if constexpr (OUT == OUT_GRAD) {
-        const float4* pr = (const float4*)(a.pre + p * 16);
-        float4* o = (float4*)((float*)a.out + p * 16);
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const float4 pv = pr[q];
-          o[q] = make_float4(__uint_as_float(v[4 * q]) * gelu_df(pv.x), __uint_as_float(v[4 * q + 1]) * gelu_df(pv.y),
-                             __uint_as_float(v[4 * q + 2]) * gelu_df(pv.z),
-                             __uint_as_float(v[4 * q + 3]) * gelu_df(pv.w));
+        for (int k = 0; k < 4; ++k) {
+          const int rw = 8 * k + (lane >> 2);
+          const int64_t p = point(32 * (warp & 3) + rw);
+          if (p < 0) continue;  // (no warp-wide step follows within this loop)
+          float4 d = *(const float4*)(stg + rw * 64 + ((q ^ ((rw >> 1) & 3)) << 4));
+          if constexpr (OUT == OUT_HIDDEN) {
+            d = make_float4(d.x + bq.x, d.y + bq.y, d.z + bq.z, d.w + bq.w);
+            if (a.pre) ((float4*)a.pre)[4 * p + q] = d;
+            ((uint2*)a.out)[4 * p + q] = make_uint2(pack_bf16(gelu_f(d.x), gelu_f(d.y)), pack_bf16(gelu_f(d.z), gelu_f(d.w)));
+          } else {
+            const float4 pv = ((const float4*)a.pre)[4 * p + q];
+            ((float4*)a.out)[4 * p + q] =
+                make_float4(d.x * gelu_df(pv.x), d.y * gelu_df(pv.y), d.z * gelu_df(pv.z), d.w * gelu_df(pv.w));
+          }
         }
       } else {
-        float* z = (float*)a.out;
-        z[p] = fmaf(cs, __uint_as_float(v[0]) + bias[0], z[p]);
-        z[npts + p] = fmaf(cs, __uint_as_float(v[1]) + bias[1], z[npts + p]);
+        const int64_t p = point(32 * (warp & 3) + lane);
+        if (p >= 0) {
+          if constexpr (OUT == OUT_F32) {
+            float* o = (float*)a.out + p * 2;
+            o[0] = __uint_as_float(v[0]) + bias[0];
+            o[1] = __uint_as_float(v[1]) + bias[1];
+          } else {
+            float* z = (float*)a.out;
+            z[p] = fmaf(cs, __uint_as_float(v[0]) + bias[0], z[p]);
+            z[npts + p] = fmaf(cs, __uint_as_float(v[1]) + bias[1], z[npts + p]);
+          }
+        }
+        __syncwarp();
       }
     }
   }
@@ -641,6 +689,18 @@ __global__ void __launch_bounds__(128) conv_tc_kernel(TcConvArgs a) {
   __syncthreads();
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TC_TMEM));
   if (tid == 0 && *fail) atomicExch(a.err, 1);
+}
+
+// Bricks or runs.  An image up to 32 points wide is taken as runs of 128 points of its planes' rows
+// joined by one zero point each (the right neighbour of a row's end and the left one of the next
+// row's beginning): a run's halo is no larger than a brick's, a row of nx points costs nx + 1 places
+// of a tile and not 32 ceil(nx / 30) (33 instead of 64 at nx = 32), and nothing is dropped but the
+// zeros.  Wider images would need wider halos for that.
+void conv_tiling(TcConvArgs& a) {
+  a.run = a.nx <= RUN_NX;
+  a.bx = a.run ? 1 : (a.nx + BX - 1) / BX;
+  a.by = a.run ? (int)(((int64_t)a.ny * (a.nx + 1) - 1 + 127) / 128) : (a.ny + BY - 1) / BY;
+  a.bz = (a.nz + BZ - 1) / BZ;
 }
 
 // Canonical tensor-core taps of every layer: layer l, tap t, 16 x 16 BF16 with c_out rows
@@ -794,9 +854,7 @@ int cnn_apply_field(const CnnNet& net, int nz, int ny, int nx, const float* t, c
   a.nz = nz;
   a.ny = ny;
   a.nx = nx;
-  a.bx = (nx + BX - 1) / BX;
-  a.by = (ny + BY - 1) / BY;
-  a.bz = (nz + BZ - 1) / BZ;
+  conv_tiling(a);
   a.sumsq = sumsq;
   a.out_scale = out_scale;
   a.err = err;
@@ -856,9 +914,7 @@ TcConvArgs tr_tc_args(const helm6_cnn_trainer* tr) {
   a.nz = tr->nz;
   a.ny = tr->ny;
   a.nx = tr->nx;
-  a.bx = (tr->nx + BX - 1) / BX;
-  a.by = (tr->ny + BY - 1) / BY;
-  a.bz = (tr->nz + BZ - 1) / BZ;
+  conv_tiling(a);
   a.err = tr->tcerr;
   return a;
 }
@@ -931,7 +987,7 @@ int tr_backward(helm6_cnn_trainer* tr, const float* x, const float* target) {
   t.pre = tr->pre[2];
   t.out = tr->ga;
   note_launch();
-  conv_tc_kernel<IN_G32, OUT_GRAD><<<tgrid, 128, TC_SMEM4, s>>>(t);
+  conv_tc_kernel<IN_G32, OUT_GRAD><<<tgrid, conv_threads<IN_G32>(), TC_SMEM4, s>>>(t);
   // layers 3 and 2
   float* gcur = tr->ga;
   float* gnext = tr->gb;
@@ -945,7 +1001,7 @@ int tr_backward(helm6_cnn_trainer* tr, const float* x, const float* target) {
     t.pre = tr->pre[l - 1];
     t.out = gnext;
     note_launch();
-    conv_tc_kernel<IN_G32, OUT_GRAD><<<tgrid, 128, TC_SMEM4, s>>>(t);
+    conv_tc_kernel<IN_G32, OUT_GRAD><<<tgrid, conv_threads<IN_G32>(), TC_SMEM4, s>>>(t);
     std::swap(gcur, gnext);
   }
   // layer 1: dW from the BF16-rounded input and g1

@@ -47,3 +47,20 @@ def test_weight_gradient_at_tile_edges(shape):
             b = slice(o, o + size)
             assert np.linalg.norm(g[b] - ref[b]) < 3e-3 * np.linalg.norm(ref[b]), (ci, co, size)
             o += size
+
+
+@pytest.mark.parametrize("shape", [(1, 1, 130, 1), (2, 3, 64, 3), (1, 4, 9, 30), (2, 5, 31, 31), (1, 5, 8, 32),
+                                   (1, 2, 3, 33), (2, 9, 32, 32)])
+def test_forward_at_run_and_brick_edges(shape):
+    """Layers at the edges of the convolution kernel's tiles: images up to 32 points wide are taken as
+    runs of 128 points of rows joined by a zero point, wider ones as 30 x 4 x 4 bricks.  The bound is
+    that of the ordinary sizes: FP32 sums and single BF16 rounding flips (2^-8 of a value)."""
+    from paper_1212_1397_gb300 import build, helm6
+    build.build()
+    th = cnn.init_params(inputs.standard_normal(31, cnn.n_params())).astype(np.float32)
+    x = inputs.standard_normal(32, int(np.prod(shape)) * 2).reshape(shape + (2,)).astype(np.float32)
+    with helm6.Trainer(*shape, th) as tr:
+        y = tr.forward(torch.from_numpy(x).cuda()).cpu().numpy().astype(np.float64)
+    ref = cnn.forward(th.astype(np.float64), x.astype(np.float64), bf16=True)
+    assert np.linalg.norm(y - ref) < 1e-3 * np.linalg.norm(ref)
+    assert np.abs(y - ref).max() < 1e-2 * np.abs(ref).max()
