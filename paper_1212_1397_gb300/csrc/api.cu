@@ -1582,6 +1582,16 @@ int helm6_apply_A(helm6_ctx* c, const void* x, void* y) {
   if (!c || !x || !y) return HELM6_ERR_INVALID;
   cudaStream_t s = c->stream;
   const int64_t N = c->g.N;
+  // FP64 with the caller's axis order: straight on the caller's arrays, unless they overlap (two
+  // conversion passes less: 16 bytes per point read and written each)
+  const char *xb = (const char*)x, *yb = (const char*)y;
+  if (c->opts.precision == HELM6_FP64 && c->xaxis < 0 && (xb + 16 * N <= yb || yb + 16 * N <= xb)) {
+    cudaEvent_t e = prof_start(c);
+    launch_apply64_il(c->g, c->coef, (const double*)x, (double*)y, s);
+    prof_stop(c, HELM6_PH_STENCIL, e);
+    CK(cudaGetLastError());
+    return HELM6_OK;
+  }
   launch_caller_to_planar(c->g, c->xaxis, (const double*)x, c->R64, s);
   if (c->opts.precision == HELM6_FP64) {
     cudaEvent_t e = prof_start(c);

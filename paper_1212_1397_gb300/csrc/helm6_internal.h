@@ -98,7 +98,14 @@ template <typename T>
 void launch_stencil(const Geom& g, const StencilCoef& c, const T* x, T* y, const T* f, T* r,
                     int mode, double* sumsq, int* nblk, cudaStream_t s, int share = 1);
 
-// Number of blocks (and fused-norm partials) of launch_stencil for this geometry.
+// The FP64 operator on interleaved complex128 arrays (16-byte aligned): y = A x, x and y apart;
+// r = F - A u with the blocks' sums of |r|^2 in partials (u and r apart; the number of blocks is
+// returned).
+void launch_apply64_il(const Geom& g, const StencilCoef& c, const double* x, double* y, cudaStream_t s);
+int launch_residual64_il(const Geom& g, const StencilCoef& c, const double* F, const double* u, double* r,
+                         double* partials, cudaStream_t s);
+
+// Number of blocks (and fused-norm partials) of the operator's kernels for this geometry.
 int stencil_blocks(const Geom& g);
 
 // Batched strided real GEMM on planar data, C = A * B per batch:

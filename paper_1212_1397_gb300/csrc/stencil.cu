@@ -9,11 +9,10 @@
 // across x/y faces and across Neumann z faces are even reflections (U_{-1} = U_1);
 // across Dirichlet faces they are zero.
 //
-// Thread block: a 32 x 8 (x, y) tile marching over a chunk of up to 32 z planes.  Each plane
-// tile plus a one-point halo is staged in shared memory by asynchronous copies issued
-// three planes ahead into a ring of five buffers (one barrier per plane); each thread
-// keeps the three plane sums (C, Nb, Dg) of planes l-1, l, l+1 in registers, so every
-// input value is read from global memory once per chunk.
+// A thread block takes an (x, y) tile and marches over a chunk of z planes.  Each plane tile plus a
+// one-point halo is staged in shared memory by asynchronous copies issued two or three planes ahead
+// into a ring of buffers (one barrier per plane), and the plane's sums are combined with those of its
+// neighbours in registers, so every input value is read from global memory once per chunk.
 #include <algorithm>
 
 #include "helm6_internal.h"
@@ -22,16 +21,14 @@ namespace helm6 {
 
 namespace {
 
-constexpr int TX = 32, TY = 8;
 constexpr int ZCH = 32;  // most z planes per block
 
-// Planes per block for `tiles` (x, y) tiles of mz planes: 32 where that leaves `per_sm` blocks per
+// FP32: planes per block for `tiles` (x, y) tiles of mz planes: 32 where that leaves `per_sm` blocks per
 // SM, else half as many, down to 2 (a block reads two planes more than it computes).  A block
 // marches plane by plane, so on small grids its length is the kernel's time; on large ones longer
-// blocks read less twice.  Measured, 32 planes a block against this rule: FP32 34 -> 9 us at 32^3,
-// 35 -> 19 at 128^3, unchanged at 256^3 (16 planes there: 85 against 82); FP64 87 -> 12 and
-// 164 -> 157 us.
-constexpr int ZB32 = 3, ZB64 = 6;  // blocks per SM asked for: FP32, FP64 (best of 2 to 32 planes at 64^3 to 256^3)
+// blocks read less twice.  Measured, 32 planes a block against this rule: 34 -> 9 us at 32^3,
+// 35 -> 19 at 128^3, unchanged at 256^3 (16 planes there: 85 against 82).
+constexpr int ZB32 = 3;  // blocks per SM asked for (best of 2 to 32 planes at 64^3 to 256^3)
 // share: problems running side by side, which fill the SMs together (6 problems of 96 to 160
 // points a side in one batch: 26.5 ms with each block length chosen as if alone, 25.3 so).
 int z_chunk(int tiles, int mz, int per_sm, int share = 1) {
@@ -63,61 +60,71 @@ __device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_grou
 template <int N>
 __device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
 
-// RW: the interior class weights are real (a real wavenumber); their products with the
-// plane sums then take two FMAs instead of four (identical results: the imaginary parts
-// that drop out are exact zeros).
-template <typename T, int MODE, bool NORM, bool RW>
-__global__ void __launch_bounds__(TX* TY)
-    stencil_kernel(Geom g, StencilCoef coef, const T* __restrict__ x, T* __restrict__ y,
-                   const T* __restrict__ f, double* __restrict__ sumsq, int zch) {
-  // ring of NBUF staged planes; plane p + DIST is requested while plane p is used
-  constexpr int DIST = 3, NBUF = DIST + 2;
-  __shared__ T sre[NBUF][TY + 2][TX + 2];
-  __shared__ T sim[NBUF][TY + 2][TX + 2];
-  __shared__ double red[TX * TY / 32];
+__device__ __forceinline__ int ghost_index(int gi, int m, int lo_neumann, int hi_neumann) {
+  if (gi < 0) return lo_neumann ? 1 : -1;
+  if (gi >= m) return (hi_neumann && gi == m) ? m - 2 : -1;
+  return gi;
+}
 
-  const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * TX + tx;
-  const int i = blockIdx.x * TX + tx, j = blockIdx.y * TY + ty;
+// FP64: a 16 x 32 (x, y) tile, 16 x 16 threads with 2 y-adjacent points each.
+//
+// Bound by the FP64 pipe (two operations per clock and SM), so what counts is operations per
+// point, those of idle lanes included.  The x-neighbour sums of the four halo rows are shared by
+// the thread's two points (5 operations per point and component for the in-plane sums), and the
+// planes are combined as they arrive: plane p gives
+//     G(p) = c1 C + c2 Nb + c3 Dg   to rows p - 1 and p + 1,   c0 C + c1 Nb + c2 Dg   to row p,
+// so a row is one sum of three fused chains, 7 operations with real weights, instead of the nine
+// of adding up its 27 points class by class; two values per point and component are kept instead of
+// three planes' sums.  Tiles are 16 points wide and a warp (4 rows) beyond the grid's edge skips the
+// arithmetic, so little of it is spent on padding.  15 -> 12 operations; with the
+// blocks chosen below, on a caller's arrays: A x 1214 -> 837 us at 256^3 (FP64 pipe at 12 operations:
+// 745), 529 -> 394 at 192^3, 189 -> 107 at 100^3 (complex k); F - A x with its norm 1520 -> 1015 at 256^3.
+//
+// IL: x, f and y are interleaved complex arrays (a caller's own, or of a call without workspace)
+// instead of planar ones.  RW: the interior class weights are real (a real wavenumber); the products
+// with the imaginary parts, exact zeros, then drop out.
+constexpr int DX = 16, DTY = 16, DLD = DX + 2, DNT = DX * DTY;
+
+template <bool RW>
+__device__ __forceinline__ cpx<double> wfma(const cpx<double>& c, const cpx<double>& v, const cpx<double>& a) {
+  if constexpr (RW)
+    return mk(fmx(c.re, v.re, a.re), fmx(c.re, v.im, a.im));
+  else
+    return cfma(c, v, a);
+}
+template <int MODE, bool NORM, bool RW, bool IL, int DR>
+__global__ void __launch_bounds__(DNT, 3)
+    stencil64_kernel(Geom g, const __grid_constant__ StencilCoef coef, const double* __restrict__ x,
+                     double* __restrict__ y, const double* f, double* __restrict__ sumsq, int zch) {
+  using Z = cpx<double>;
+  // ring of NBUF staged planes; plane p + DIST is requested while plane p is used
+  constexpr int DY = DTY * DR, DROWS = DY + 2;
+  constexpr int DIST = 2, NBUF = DIST + 2, HALO = DROWS * DLD, PER = (HALO + DNT - 1) / DNT;
+  __shared__ __align__(16) double2 sb[NBUF][DROWS][DLD];
+  __shared__ double red[DNT / 32];
+
+  const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * DX + tx;
+  const int i = blockIdx.x * DX + tx, j0 = blockIdx.y * DY + DR * ty;
   const int l0 = blockIdx.z * zch;
   const int l1 = min(l0 + zch, g.mz);
   const int64_t plane = (int64_t)g.mx * g.my;
-  const bool active = (i < g.mx) && (j < g.my);
 
-  const cpx<T> c0 = cast<T>(coef.interior.w[1][0]);
-  const cpx<T> c1 = cast<T>(coef.interior.w[1][1]);
-  const cpx<T> c2 = cast<T>(coef.interior.w[1][2]);
-  const cpx<T> c3 = cast<T>(coef.interior.w[0][2]);
-
-  // Halo tile element t = tid + k * TX*TY (k = 0, 1) of every plane: its in-plane source
-  // offset (reflection across Neumann x/y faces) or -1 for a zero ghost, computed once.
-  constexpr int HALO = (TX + 2) * (TY + 2);
-  int hoff[2];
+  // halo elements tid, tid + DNT, ... of every plane: the in-plane source (reflection across
+  // Neumann x/y faces) or -1 for a zero ghost, computed once
+  int hoff[PER];
 #pragma unroll
-  for (int k = 0; k < 2; ++k) {
-    const int t = tid + k * TX * TY;
+  for (int k = 0; k < PER; ++k) {
+    const int t = tid + k * DNT;
     hoff[k] = -1;
     if (t < HALO) {
-      const int sy = t / (TX + 2), sx = t - sy * (TX + 2);
-      int gi = blockIdx.x * TX + sx - 1, gj = blockIdx.y * TY + sy - 1;
-      bool ok = true;
-      if (gi < 0) {
-        if (g.face[0] == HELM6_NEUMANN) gi = 1; else ok = false;
-      } else if (gi >= g.mx) {
-        if (g.face[1] == HELM6_NEUMANN && gi == g.mx) gi = g.mx - 2; else ok = false;
-      }
-      if (gj < 0) {
-        if (g.face[2] == HELM6_NEUMANN) gj = 1; else ok = false;
-      } else if (gj >= g.my) {
-        if (g.face[3] == HELM6_NEUMANN && gj == g.my) gj = g.my - 2; else ok = false;
-      }
-      if (ok) hoff[k] = gj * g.mx + gi;
+      const int sy = t / DLD, sx = t - sy * DLD;
+      const int gi = ghost_index(blockIdx.x * DX + sx - 1, g.mx, g.face[0] == HELM6_NEUMANN, g.face[1] == HELM6_NEUMANN);
+      const int gj = ghost_index(blockIdx.y * DY + sy - 1, g.my, g.face[2] == HELM6_NEUMANN, g.face[3] == HELM6_NEUMANN);
+      if (gi >= 0 && gj >= 0) hoff[k] = gj * g.mx + gi;
     }
   }
-  T* sre_flat = &sre[0][0][0];
-  T* sim_flat = &sim[0][0][0];
-
-  // stage the halo tile of the plane feeding position p (ghost planes: reflection across a
-  // Neumann z face, zero otherwise) into ring slot `slot`
+  // the halo tile of the plane feeding position p (ghost planes: reflection across a Neumann z
+  // face, zero otherwise) into ring slot `slot`
   auto stage = [&](int p, int slot) {
     int src = p;
     bool zplane = false;
@@ -127,21 +134,41 @@ __global__ void __launch_bounds__(TX* TY)
       if (g.face[5] == HELM6_NEUMANN) src = g.mz - 2; else zplane = true;
     }
     const int64_t pbase = (int64_t)src * plane;
+    double2* d = &sb[slot][0][0];
 #pragma unroll
-    for (int k = 0; k < 2; ++k) {
-      const int t = tid + k * TX * TY;
+    for (int k = 0; k < PER; ++k) {
+      const int t = tid + k * DNT;
       if (t < HALO) {
         const bool ok = !zplane && hoff[k] >= 0;
         const int64_t idx = ok ? pbase + hoff[k] : 0;
-        cp_async<sizeof(T)>(sre_flat + slot * HALO + t, x + idx, ok ? (int)sizeof(T) : 0);
-        cp_async<sizeof(T)>(sim_flat + slot * HALO + t, x + g.N + idx, ok ? (int)sizeof(T) : 0);
+        if constexpr (IL) {
+          const uint32_t da = (uint32_t)__cvta_generic_to_shared(d + t);
+          asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(da), "l"((const double2*)x + idx),
+                       "r"(ok ? 16 : 0)
+                       : "memory");
+        } else {
+          cp_async<8>(&d[t].x, x + idx, ok ? 8 : 0);
+          cp_async<8>(&d[t].y, x + g.N + idx, ok ? 8 : 0);
+        }
       }
     }
   };
 
-  Sums<T> P0, P1, P2;  // planes l-1, l, l+1 as the march proceeds
-  const cpx<T> zero = {T(0), T(0)};
-  P0 = P1 = P2 = Sums<T>{zero, zero, zero};
+  const Z c0 = cast<double>(coef.interior.w[1][0]), c1 = cast<double>(coef.interior.w[1][1]);
+  const Z c2 = cast<double>(coef.interior.w[1][2]);
+  const double c3 = coef.interior.w[0][2].re;  // 1/30: real whatever the wavenumber
+  // the Sommerfeld-like face rows, with weights of their own: 1 (low), 2 (high); 0 any other row
+  auto face_row = [&](int l) {
+    if (l == 0 && g.face[4] == HELM6_SOMMERFELD) return 1;
+    if (l == g.mz - 1 && g.face[5] == HELM6_SOMMERFELD) return 2;
+    return 0;
+  };
+  // whether any of the warp's rows (its lanes take two thread rows) lies in the grid
+  const bool warp_on = (int)(blockIdx.y * DY + DR * (ty & ~1)) < g.my;
+  const Z zero = {0.0, 0.0};
+  Z below[DR], part[DR];  // G of the last plane; the row of the last plane without what is above it
+#pragma unroll
+  for (int q = 0; q < DR; ++q) below[q] = part[q] = zero;
   double acc = 0.0;
 
   const int pfirst = l0 - 1;
@@ -150,68 +177,60 @@ __global__ void __launch_bounds__(TX* TY)
     cp_commit();
   }
   for (int p = pfirst; p <= l1; ++p) {
-    const int k = p - pfirst;
+    const int k = p - pfirst, l = p - 1;  // row l is complete with plane p
     if (p + DIST <= l1) stage(p + DIST, (k + DIST) % NBUF);
     cp_commit();
+    Z fv[DR];
+    if constexpr (MODE != 0) {
+#pragma unroll
+      for (int q = 0; q < DR; ++q) {
+        fv[q] = zero;
+        if (l >= l0 && i < g.mx && j0 + q < g.my) {
+          const int64_t idx = (int64_t)l * plane + (int64_t)(j0 + q) * g.mx + i;
+          if constexpr (IL) {
+            const double2 v = ((const double2*)f)[idx];
+            fv[q] = mk(v.x, v.y);
+          } else {
+            fv[q] = mk(f[idx], f[g.N + idx]);
+          }
+        }
+      }
+    }
     cp_wait<DIST>();  // the group of plane p has landed
     __syncthreads();
-    const int buf = k % NBUF;
-
-    // ---- in-plane sums of plane p at (i, j) ----
-    Sums<T> cur;
-    {
-      const int a = ty + 1, b = tx + 1;
-      cur.c = mk(sre[buf][a][b], sim[buf][a][b]);
-      cur.n = mk(sre[buf][a][b - 1] + sre[buf][a][b + 1] + sre[buf][a - 1][b] + sre[buf][a + 1][b],
-                 sim[buf][a][b - 1] + sim[buf][a][b + 1] + sim[buf][a - 1][b] + sim[buf][a + 1][b]);
-      cur.d = mk(sre[buf][a - 1][b - 1] + sre[buf][a - 1][b + 1] + sre[buf][a + 1][b - 1] +
-                     sre[buf][a + 1][b + 1],
-                 sim[buf][a - 1][b - 1] + sim[buf][a - 1][b + 1] + sim[buf][a + 1][b - 1] +
-                     sim[buf][a + 1][b + 1]);
+    if (!warp_on) continue;
+    const double2* t0 = &sb[k % NBUF][DR * ty][tx];
+    Z c[DR + 2], h[DR + 2];
+#pragma unroll
+    for (int q = 0; q < DR + 2; ++q) {
+      const double2 a = t0[q * DLD], b = t0[q * DLD + 1], e = t0[q * DLD + 2];
+      c[q] = mk(b.x, b.y);
+      h[q] = mk(a.x + e.x, a.y + e.y);
     }
-    P0 = P1;
-    P1 = P2;
-    P2 = cur;
-
-    const int l = p - 1;  // row whose three planes are now in P0, P1, P2
-    if (l >= l0 && active) {
-      cpx<T> out;
-      const bool slo = (l == 0) && (g.face[4] == HELM6_SOMMERFELD);
-      const bool shi = (l == g.mz - 1) && (g.face[5] == HELM6_SOMMERFELD);
-      if (!slo && !shi) {
-        // interior class form: c0 C + c1 (Nb + C-+C+) + c2 (Dg + Nb-+Nb+) + c3 (Dg-+Dg+)
-        const cpx<T> s1 = P1.n + P0.c + P2.c, s2 = P1.d + P0.n + P2.n, s3 = P0.d + P2.d;
-        if constexpr (RW) {
-          out.re = fmx(c3.re, s3.re, fmx(c2.re, s2.re, fmx(c1.re, s1.re, c0.re * P1.c.re)));
-          out.im = fmx(c3.re, s3.im, fmx(c2.re, s2.im, fmx(c1.re, s1.im, c0.re * P1.c.im)));
+    const int fl = face_row(l), fp = face_row(p), fn = face_row(p + 1);
+#pragma unroll
+    for (int q = 0; q < DR; ++q) {
+      const Z C = c[q + 1], n = h[q + 1] + (c[q] + c[q + 2]), d = h[q] + h[q + 2];
+      const Z G = wfma<RW>(c2, n, wfma<RW>(c1, C, c3 * d));
+      auto face = [&](int fc, int a, const Z& base) {  // plane p's part of a face row
+        const RowWeights& W = fc == 1 ? coef.s_lo : coef.s_hi;
+        return cfma(cast<double>(W.w[a][2]), d, cfma(cast<double>(W.w[a][1]), n, cfma(cast<double>(W.w[a][0]), C, base)));
+      };
+      Z out = fl ? face(fl, 2, part[q]) : part[q] + G;
+      if (p >= l0 && p < l1) part[q] = fp ? face(fp, 1, below[q]) : wfma<RW>(c2, d, wfma<RW>(c1, n, wfma<RW>(c0, C, below[q])));
+      below[q] = fn ? face(fn, 0, zero) : G;
+      if (l >= l0 && i < g.mx && j0 + q < g.my) {
+        const int64_t idx = (int64_t)l * plane + (int64_t)(j0 + q) * g.mx + i;
+        if (MODE == 1) out = fv[q] - out;
+        if (MODE == 2) out = fv[q] + out;
+        if constexpr (IL) {
+          ((double2*)y)[idx] = make_double2(out.re, out.im);
         } else {
-          out = c0 * P1.c;
-          out = cfma(c1, s1, out);
-          out = cfma(c2, s2, out);
-          out = cfma(c3, s3, out);
+          y[idx] = out.re;
+          y[g.N + idx] = out.im;
         }
-      } else {
-        const RowWeights& W = slo ? coef.s_lo : coef.s_hi;
-        out = zero;
-        out = cfma(cast<T>(W.w[0][0]), P0.c, out);
-        out = cfma(cast<T>(W.w[0][1]), P0.n, out);
-        out = cfma(cast<T>(W.w[0][2]), P0.d, out);
-        out = cfma(cast<T>(W.w[1][0]), P1.c, out);
-        out = cfma(cast<T>(W.w[1][1]), P1.n, out);
-        out = cfma(cast<T>(W.w[1][2]), P1.d, out);
-        out = cfma(cast<T>(W.w[2][0]), P2.c, out);
-        out = cfma(cast<T>(W.w[2][1]), P2.n, out);
-        out = cfma(cast<T>(W.w[2][2]), P2.d, out);
+        if (NORM) acc += out.re * out.re + out.im * out.im;
       }
-      const int64_t idx = (int64_t)l * plane + (int64_t)j * g.mx + i;
-      if (MODE == 1) {
-        out = mk(f[idx] - out.re, f[g.N + idx] - out.im);
-      } else if (MODE == 2) {
-        out = mk(f[idx] + out.re, f[g.N + idx] + out.im);
-      }
-      y[idx] = out.re;
-      y[g.N + idx] = out.im;
-      if (NORM) acc += (double)out.re * out.re + (double)out.im * out.im;
     }
   }
   cp_wait<0>();
@@ -221,7 +240,7 @@ __global__ void __launch_bounds__(TX* TY)
     if ((tid & 31) == 0) red[tid >> 5] = acc;
     __syncthreads();
     if (tid < 32) {
-      double v = (tid < TX * TY / 32) ? red[tid] : 0.0;
+      double v = (tid < DNT / 32) ? red[tid] : 0.0;
       v = warp_sum(v);
       if (tid == 0) {
         const int64_t b = ((int64_t)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
@@ -239,12 +258,6 @@ __global__ void __launch_bounds__(TX* TY)
 // cross the field's x extent, are copied element by element with the ghost rules.
 constexpr int T4X = 32, T4Y = 16, T4R = 4, T4ROWS = T4Y + 2, T4LD = 40;
 constexpr int T4SLOTS = 2 * T4ROWS * 10;  // components x rows x (8 chunks + 2 edges)
-
-__device__ __forceinline__ int ghost_index(int gi, int m, int lo_neumann, int hi_neumann) {
-  if (gi < 0) return lo_neumann ? 1 : -1;
-  if (gi >= m) return (hi_neumann && gi == m) ? m - 2 : -1;
-  return gi;
-}
 
 // The FP32 kernel's weights, rounded to FP32 once on the host (a conversion per thread and
 // weight would run on the FP64 pipe): the four interior class weights and the two
@@ -467,11 +480,90 @@ __global__ void __launch_bounds__(T4X* T4Y / T4R)
 
 }  // namespace
 
+namespace {
+
+// Points per thread (1 or 2) and planes per block: the pair with the least arithmetic on the fullest
+// SM.  The FP64 pipe is the bound however many blocks share it, so what counts is whole blocks per SM,
+// times planes (a block's first and last plane take half the work), times 13 or 23 operations per
+// thread; partial tiles and the last chunk fill the SMs left over by the whole ones or add to
+// them (a partial tile of at most four warps 0.6 of a whole one), and no SM does less than the mean.
+// Against the best of all pairs tried at eight sizes from 32^3 to 300^3 (apply_A): within 2.6 %; 32
+// planes, halved until every SM had four blocks of two points per thread, was up to 60 % off (21 us
+// instead of 13 at 32^3, 45 instead of 30 at 64^3, 123 instead of 111 at 100^3).
+struct Grid64 {
+  int dr, zch;
+  dim3 grid;
+};
+Grid64 grid64(const Geom& g) {
+  static int sms = 0;
+  if (!sms) sms = device_sm_count();
+  auto up = [](int64_t a, int64_t b) { return (a + b - 1) / b; };
+  Grid64 b{};
+  double best = 1e300;
+  for (int dr = 1; dr <= 2; ++dr) {
+    const int dy = DTY * dr;
+    const int64_t tx = up(g.mx, DX), left_rows = g.my % dy;
+    const bool part = left_rows > 0 && left_rows <= dy / 2;  // a tile of at most four warps
+    const int64_t ty = g.my / dy + (left_rows > dy / 2), tyf = std::max<int64_t>(1, ty);
+    for (int z = 1; z <= 64 && (z == 1 || z < 2 * g.mz); ++z) {
+      const int64_t nzf = std::max(1, g.mz / z), rz = g.mz > z ? g.mz % z : 0;
+      const double whole = std::min(z, g.mz) + 1, rest = rz ? rz + 1 : 0;
+      const int64_t n1 = tx * tyf * nzf, n2 = (rz ? tx * tyf : 0) + (part && ty ? tx * nzf : 0);
+      const int64_t rounds = up(n1, sms), spare = rounds * sms - n1;
+      const double extra = std::max(rest, part && ty ? 0.6 * whole : 0.0);
+      const double full = rounds * whole + (n2 > spare ? extra * up(n2 - spare, sms) : 0.0);
+      const double mean = tx * (tyf + (part && ty ? 0.5 : 0.0)) * (nzf * whole + rest) / sms;
+      const double cost = std::max(full, mean) * (dr == 1 ? 13 : 23);
+      if (cost < best) {
+        best = cost;
+        b.dr = dr;
+        b.zch = z;
+        b.grid = dim3((unsigned)tx, (unsigned)up(g.my, dy), (unsigned)up(g.mz, z));
+      }
+    }
+  }
+  return b;
+}
+
+bool real_weights(const StencilCoef& c) {
+  return c.interior.w[1][0].im == 0.0 && c.interior.w[1][1].im == 0.0 && c.interior.w[1][2].im == 0.0;
+}
+
+template <int MODE, bool NORM, bool IL>
+int run64(const Geom& g, const StencilCoef& c, const double* x, double* y, const double* f, double* sumsq,
+          cudaStream_t s) {
+  const Grid64 b = grid64(g);
+  const dim3 block(DX, DTY);
+  const bool rw = real_weights(c);
+  note_launch();
+  if (rw && b.dr == 1)
+    stencil64_kernel<MODE, NORM, true, IL, 1><<<b.grid, block, 0, s>>>(g, c, x, y, f, sumsq, b.zch);
+  else if (rw)
+    stencil64_kernel<MODE, NORM, true, IL, 2><<<b.grid, block, 0, s>>>(g, c, x, y, f, sumsq, b.zch);
+  else if (b.dr == 1)
+    stencil64_kernel<MODE, NORM, false, IL, 1><<<b.grid, block, 0, s>>>(g, c, x, y, f, sumsq, b.zch);
+  else
+    stencil64_kernel<MODE, NORM, false, IL, 2><<<b.grid, block, 0, s>>>(g, c, x, y, f, sumsq, b.zch);
+  return (int)(b.grid.x * b.grid.y * b.grid.z);
+}
+
+}  // namespace
+
 int stencil_blocks(const Geom& g) {
-  // the larger of the two kernels' grids (FP64: 32 x 8 tiles, FP32: 32 x 16 tiles)
-  const int t8 = ((g.mx + TX - 1) / TX) * ((g.my + TY - 1) / TY), t16 = ((g.mx + T4X - 1) / T4X) * ((g.my + T4Y - 1) / T4Y);
-  const int z8 = z_chunk(t8, g.mz, ZB64), z16 = z_chunk(t16, g.mz, ZB32);
-  return std::max(t8 * ((g.mz + z8 - 1) / z8), t16 * ((g.mz + z16 - 1) / z16));
+  // the larger of the two kernels' grids
+  const dim3 d = grid64(g).grid;
+  const int t16 = ((g.mx + T4X - 1) / T4X) * ((g.my + T4Y - 1) / T4Y);
+  const int z16 = z_chunk(t16, g.mz, ZB32);
+  return std::max((int)(d.x * d.y * d.z), t16 * ((g.mz + z16 - 1) / z16));
+}
+
+void launch_apply64_il(const Geom& g, const StencilCoef& c, const double* x, double* y, cudaStream_t s) {
+  run64<0, false, true>(g, c, x, y, nullptr, nullptr, s);
+}
+
+int launch_residual64_il(const Geom& g, const StencilCoef& c, const double* F, const double* u, double* r,
+                         double* partials, cudaStream_t s) {
+  return run64<1, true, true>(g, c, u, r, F, partials, s);
 }
 
 template <typename T>
@@ -520,33 +612,16 @@ void launch_stencil(const Geom& g, const StencilCoef& c, const T* x, T* y, const
 #undef HELM6_S4
     return;
   }
-  dim3 block(TX, TY);
-  dim3 grid((g.mx + TX - 1) / TX, (g.my + TY - 1) / TY);
-  const int zch = z_chunk((int)(grid.x * grid.y), g.mz, ZB64);
-  grid.z = (g.mz + zch - 1) / zch;
-  if (nblk) *nblk = (int)(grid.x * grid.y * grid.z);
-  note_launch();
-  const bool nrm = sumsq != nullptr;
-  const bool rw = c.interior.w[1][0].im == 0.0 && c.interior.w[1][1].im == 0.0 &&
-                  c.interior.w[1][2].im == 0.0 && c.interior.w[0][2].im == 0.0;
-#define HELM6_SG(M, N)                                                                        \
-  do {                                                                                        \
-    if (rw)                                                                                   \
-      stencil_kernel<T, M, N, true><<<grid, block, 0, s>>>(g, c, x, y, f, N ? sumsq : nullptr, zch);  \
-    else                                                                                      \
-      stencil_kernel<T, M, N, false><<<grid, block, 0, s>>>(g, c, x, y, f, N ? sumsq : nullptr, zch); \
-  } while (0)
-  if (mode == 0 && !nrm)
-    HELM6_SG(0, false);
-  else if (mode == 0)
-    HELM6_SG(0, true);
-  else if (mode == 1 && !nrm)
-    HELM6_SG(1, false);
+  const double *xd = (const double*)x, *fd = (const double*)f;
+  double* yd = (double*)y;
+  int nb;
+  if (mode == 0)
+    nb = sumsq ? run64<0, true, false>(g, c, xd, yd, fd, sumsq, s) : run64<0, false, false>(g, c, xd, yd, fd, nullptr, s);
   else if (mode == 1)
-    HELM6_SG(1, true);
+    nb = sumsq ? run64<1, true, false>(g, c, xd, yd, fd, sumsq, s) : run64<1, false, false>(g, c, xd, yd, fd, nullptr, s);
   else
-    HELM6_SG(2, false);
-#undef HELM6_SG
+    nb = run64<2, false, false>(g, c, xd, yd, fd, nullptr, s);
+  if (nblk) *nblk = nb;
 }
 
 template void launch_stencil<float>(const Geom&, const StencilCoef&, const float*, float*,
