@@ -197,7 +197,11 @@ __global__ void reduce_sum_kernel(const double* __restrict__ partial, int n, dou
 // ---- Arnoldi with delayed classical Gram-Schmidt (one reduction + one update per step) ----
 // Vector traits for 2-point loads of a planar field.
 
-constexpr int CHD = 8;  // most basis vectors per warp group of the reduction pass (4 accumulators each)
+// Most basis vectors per warp group of the reduction pass (4 accumulators each).  FP64: 4, so that two
+// blocks share an SM, one's loads behind the other's arithmetic (eight vectors, one block: 341 us
+// instead of 301 per pass at 127^3, 198 and 183 at 101^3, 756 either way at 192^3).
+template <typename T>
+constexpr int CHD = sizeof(T) == 8 ? 4 : 8;
 
 // P consecutive values of one plane, starting at point q * P, widened to the arithmetic
 // type T.  S is the storage type: T itself (P = 1, 2, or 4 for float) or __half (P = 1, 2
@@ -339,6 +343,27 @@ __device__ __forceinline__ T round_to(T x) {
     return __half2float(__float2half_rn(x));
 }
 
+// The warp's sums of M values per lane (M a power of two up to 32): value c in lane c (and c + M, ...).
+// Each exchange halves the values a lane is left with: M - 1 additions and a few for M < 32,
+// instead of 5 M (in FP64 an addition takes a warp's scheduler 64 cycles: 35 sums by five additions
+// each were 12 us per block of a reduction pass).
+template <typename T, int M>
+__device__ __forceinline__ T warp_sums(T (&r)[M], int lane) {
+#pragma unroll
+  for (int h = M / 2; h > 0; h /= 2) {
+    const bool up = lane & h;
+#pragma unroll
+    for (int c = 0; c < h; ++c) {
+      const T give = up ? r[c] : r[c + h], keep = up ? r[c + h] : r[c];
+      r[c] = keep + __shfl_xor_sync(0xffffffffu, give, h);
+    }
+  }
+  T v = r[0];
+#pragma unroll
+  for (int o = M; o < 32; o *= 2) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
 // One reduction pass over the basis V_0..V_{count-1}, u and (optionally) w.  Per block:
 //   s_i = sum conj(V_i) u,  t_i = sum conj(V_i) w  (i < count),
 //   a = sum |u|^2,  b = sum conj(u) w.
@@ -352,7 +377,7 @@ __device__ __forceinline__ T round_to(T x) {
 // end of a round every accumulator is reduced by warp shuffles and one shared-memory
 // exchange.
 template <typename T, int PTS, typename TV, int CH>
-__global__ void __launch_bounds__(RB, sizeof(T) == 8 ? 1 : 2) dcgs_dot_kernel(const TV* __restrict__ V, int64_t vs, int count,
+__global__ void __launch_bounds__(RB, 2) dcgs_dot_kernel(const TV* __restrict__ V, int64_t vs, int count,
                                                          const T* __restrict__ u, const T* __restrict__ w,
                                                          int64_t N, double* __restrict__ partial, double vinv) {
   constexpr int NW = RB / 32;
@@ -423,11 +448,23 @@ __global__ void __launch_bounds__(RB, sizeof(T) == 8 ? 1 : 2) dcgs_dot_kernel(co
         }
       }
     }
+    {
+      constexpr int M = 4 * CH <= 4 ? 4 : 4 * CH <= 8 ? 8 : 4 * CH <= 16 ? 16 : 32;
+      T r[M];
 #pragma unroll
-    for (int c = 0; c < NACC; ++c) {
-      T v = acc[c];
-      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-      if (lane == 0) sh[warp][c] = v;
+      for (int c = 0; c < M; ++c) r[c] = c < 4 * CH ? acc[c] : T(0);
+      const T v = warp_sums<T, M>(r, lane);
+      if (lane < 4 * CH) sh[warp][lane] = v;
+      if (own) {
+#pragma unroll
+        for (int c = 4 * CH; c < NACC; ++c) {
+          T v3 = acc[c];
+          for (int o = 16; o > 0; o >>= 1) v3 += __shfl_xor_sync(0xffffffffu, v3, o);
+          if (lane == 0) sh[warp][c] = v3;
+        }
+      } else if (lane < 3) {
+        sh[warp][4 * CH + lane] = T(0);
+      }
     }
     __syncthreads();
     // group gg's sums over its wpg warps; column c of its accumulators
@@ -1054,14 +1091,14 @@ void launch_dcgs_dot(const TV* V, int64_t vs, int count, const T* u, const T* w,
       }
     }
     if (cgs_pts<TV>(N, vs) == 4) {
-      dcgs_dot_kernel<T, 4, TV, CHD><<<nblocks, RB, 0, s>>>(V, vs, count, u, w, N, partial, vinv);
+      dcgs_dot_kernel<T, 4, TV, CHD<T>><<<nblocks, RB, 0, s>>>(V, vs, count, u, w, N, partial, vinv);
       return;
     }
   }
   if (cgs_pts<TV>(N, vs) == 2)
-    dcgs_dot_kernel<T, 2, TV, CHD><<<nblocks, RB, 0, s>>>(V, vs, count, u, w, N, partial, vinv);
+    dcgs_dot_kernel<T, 2, TV, CHD<T>><<<nblocks, RB, 0, s>>>(V, vs, count, u, w, N, partial, vinv);
   else
-    dcgs_dot_kernel<T, 1, TV, CHD><<<nblocks, RB, 0, s>>>(V, vs, count, u, w, N, partial, vinv);
+    dcgs_dot_kernel<T, 1, TV, CHD<T>><<<nblocks, RB, 0, s>>>(V, vs, count, u, w, N, partial, vinv);
 }
 
 // Blocks of the reduction pass: two per SM (its per-block epilogue favours few blocks).
