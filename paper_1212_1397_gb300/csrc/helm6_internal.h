@@ -134,9 +134,9 @@ void launch_xform_tc(const float* in, float* out, const uint8_t* W, int M_total,
 // FP64 x/y transform in exact integer slices on the tensor cores (xform64.cu): one basis matrix
 // (m x m) as digit planes, and the same for symmetric (fold) bases over half the points.
 struct X64Basis {
-  uint8_t* dev = nullptr;  // digit planes (device)
-  size_t bytes = 0;
-  int m = 0, fold = 0, nk = 0, nch = 0, gcols = 0, ngroups = 0, eb = 0;
+  uint8_t* dev = nullptr;  // digit planes, then the FP64 rows of the last `tail` modes (device)
+  size_t bytes = 0, planes = 0;
+  int m = 0, fold = 0, nk = 0, nch = 0, gcols = 0, ngroups = 0, eb = 0, tail = 0;
 };
 X64Basis x64_plan(int n, int lo, int hi);
 void x64_trig(int n, int lo, int hi, std::vector<double>& trig);

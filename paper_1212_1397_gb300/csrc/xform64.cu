@@ -35,6 +35,8 @@
 //     release it, then round and store them while the next group runs;
 //   * two scanner warps find the row exponents of the next unit's rows (which also brings those
 //     rows into L2).
+// One or two modes beyond whole groups (258 points: 129 of each parity) are formed in FP64 by a
+// kernel of their own.
 // All arithmetic on data points and sums is 32-bit integer or FP32, most of it on the FMA pipe
 // (multiply-adds, FP32 sums as integer conversions): an FP64 operation or conversion takes a
 // scheduler 64 cycles, an FP32-to-integer conversion 8, a logic operation or a carry 2, an
@@ -94,6 +96,8 @@ struct X64Args {
   int ngroups, gcols, nch, npad;  // groups, columns per group, groups per parity, padded columns
   int split, nunits;              // units per tile and in all
   int transposed, R, ldin, ldo;
+  int tail;          // last modes, formed in FP64 from the rows Bt
+  const double* Bt;  // [tail][K]
   int* err;
 };
 
@@ -260,6 +264,52 @@ struct Unit {
 __device__ __forceinline__ Unit unit(const X64Args& p, int u, int rank) {
   const int part = u % p.split;
   return Unit{(u / p.split) * 2 * X_M + rank * X_M, part * p.ngroups / p.split, (part + 1) * p.ngroups / p.split};
+}
+
+// The last p.tail modes in FP64, two modes of four rows at a time per warp, the lanes' shares of a row
+// added pairwise.  Bound by the FP64 pipe: two products per data point at 258 points.
+constexpr int TM_BLOCK = 256;
+__global__ void __launch_bounds__(TM_BLOCK, 6) x64_tail_modes_kernel(X64Args p) {
+  const int lane = threadIdx.x & 31;
+  const int r0 = (int)((blockIdx.x * TM_BLOCK + threadIdx.x) >> 5) * 4, nr = min(4, p.M_total - r0);
+  if (nr <= 0) return;
+  const double* x = p.in + (int64_t)r0 * p.ldin;
+  for (int t = 0; t < p.tail; t += 2) {
+    const bool two = t + 1 < p.tail;
+    const double *b0 = p.Bt + (int64_t)t * p.K, *b1 = two ? b0 + p.K : b0;
+    double a[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) a[e] = 0.0;
+#pragma unroll 1
+    for (int k = lane; k < p.K; k += 32) {
+      const double u = b0[k], v = b1[k];
+#pragma unroll
+      for (int e = 0; e < 4; ++e)
+        if (e < nr) {
+          const double w = x[(int64_t)e * p.ldin + k];
+          a[2 * e] = fma(u, w, a[2 * e]);
+          if (two) a[2 * e + 1] = fma(v, w, a[2 * e + 1]);
+        }
+    }
+    // sum c of the eight to lane c: exchanges that halve what a lane is left with
+#pragma unroll
+    for (int h = 4; h > 0; h /= 2) {
+      const bool up = lane & h;
+#pragma unroll
+      for (int c = 0; c < h; ++c) {
+        const double give = up ? a[c] : a[c + h], keep = up ? a[c + h] : a[c];
+        a[c] = keep + __shfl_xor_sync(0xffffffffu, give, h);
+      }
+    }
+    double v = a[0];
+    v += __shfl_xor_sync(0xffffffffu, v, 8);
+    v += __shfl_xor_sync(0xffffffffu, v, 16);
+    const int row = r0 + lane / 2, m = p.P - p.tail + t + (lane & 1);
+    if (lane < 2 * nr && m < p.P) {
+      const int plane = row / p.R, rr = row - plane * p.R;
+      p.out[p.transposed ? ((int64_t)plane * p.P + m) * p.ldo + rr : (int64_t)row * p.ldo + m] = v;
+    }
+  }
 }
 
 template <int VEC, bool FOLD>
@@ -683,6 +733,12 @@ __device__ __forceinline__ double basis_entry(const X64Axis& a, const double* tr
   return a.sc * w * v;
 }
 
+// FP64 rows of the last modes (or nodes) of an axis, first m - tail.
+__global__ void x64_tail_kernel(X64Axis a, X64Basis h, const double* __restrict__ trig) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < h.tail * a.m) ((double*)(h.dev + h.planes))[i] = basis_entry(a, trig, a.m - h.tail + i / a.m, i % a.m);
+}
+
 // Digit planes of one column (mode or node p) per block, in the transform kernel's layout.  *over is
 // set when an accumulator could leave the integers that FP32 holds exactly: level l sums the basis
 // digits 0..l times data digits of at most 128.
@@ -725,10 +781,17 @@ X64Basis x64_plan(int n, int lo, int hi) {
   h.fold = nlo == nhi;
   const int Kf = h.fold ? (h.m + 1) / 2 : h.m, cnt = Kf;  // points of a product; modes of the larger parity
   h.nk = (Kf + X_KT - 1) / X_KT;
-  h.nch = (cnt + X_NMAX - 1) / X_NMAX;
-  h.gcols = round32((cnt + h.nch - 1) / h.nch);
+  // One or two modes more than the groups hold would split them into twice as many, and each group
+  // turns its tile's points into digits again, the slowest role: they are formed apart (258
+  // points, four groups of 96 columns: 682 and 631 us for the two transforms of a 256^3 field; two
+  // groups of 128 and two modes apart: 565 and 534).  Each further pair of modes would cost 160.
+  const int whole = (h.fold ? 2 : 1) * (cnt / X_NMAX) * X_NMAX;
+  h.tail = whole > 0 && h.m > whole && h.m - whole <= 2 ? h.m - whole : 0;
+  h.nch = h.tail ? cnt / X_NMAX : (cnt + X_NMAX - 1) / X_NMAX;
+  h.gcols = h.tail ? X_NMAX : round32((cnt + h.nch - 1) / h.nch);
   h.ngroups = (h.fold && h.m > 1 ? 2 : 1) * h.nch;
-  h.bytes = (size_t)h.ngroups * h.nk * 2 * DG * h.gcols * X_KT;
+  h.planes = (size_t)h.ngroups * h.nk * 2 * DG * h.gcols * X_KT;
+  h.bytes = h.planes + (size_t)h.tail * h.m * sizeof(double);
   return h;
 }
 
@@ -771,6 +834,10 @@ void launch_x64_digits(int n, int lo, int hi, int inverse, X64Basis& h, const do
   if (!inverse && a.sc > 1.0) h.eb = 1;
   note_launch();
   x64_digits_kernel<<<h.ngroups * h.gcols, 128, 0, s>>>(a, h, trig, std::ldexp(1.0, 55 - h.eb), over);
+  if (h.tail) {
+    note_launch();
+    x64_tail_kernel<<<(h.tail * h.m + 127) / 128, 128, 0, s>>>(a, h, trig);
+  }
 }
 
 int x64_configure() {
@@ -805,6 +872,8 @@ void launch_xform64(const X64Basis& b, const double* in, double* out, int M_tota
   a.R = R;
   a.ldin = ldin;
   a.ldo = ldo;
+  a.tail = b.tail;
+  a.Bt = (const double*)(b.dev + b.planes);
   a.err = err;
   static int sms = 0;
   if (!sms) sms = device_sm_count();
@@ -826,6 +895,10 @@ void launch_xform64(const X64Basis& b, const double* in, double* out, int M_tota
       xform64_kernel<16, false><<<grid, X_THREADS, X_SMEM, s>>>(a);
     else
       xform64_kernel<8, false><<<grid, X_THREADS, X_SMEM, s>>>(a);
+  }
+  if (a.tail) {
+    note_launch();
+    x64_tail_modes_kernel<<<(unsigned)(((int64_t)M_total + 4 * TM_BLOCK / 32 - 1) / (4 * TM_BLOCK / 32)), TM_BLOCK, 0, s>>>(a);
   }
 }
 

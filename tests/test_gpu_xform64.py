@@ -80,3 +80,20 @@ def test_non_finite_rows_stay_non_finite(H, bad):
     x = inputs.complex_normal(5, O.Problem(n, k, faces).shape)
     x[4, 5, 6] = bad
     assert not np.isfinite(pinv(H, n, k, faces, x)).all()
+
+
+@pytest.mark.parametrize("n,faces", [(127, "DNNDSS"), (128, "DNNDDD"), (129, "NDNDSS"), (131, "NDNDSS"), (255, "NNDDSS"), (256, "DDNNSS"),
+                                     (258, "NNNNSD"), (259, "NNDDSS")])
+def test_modes_beyond_whole_groups(H, n, faces):
+    """Axes one to five modes longer than whole groups of 128 (128, 130 and 132 modes of a quarter-wave axis, 257,
+    258, 260 and 261 of a cosine one): up to two are formed apart in FP64."""
+    k = 0.2 * (n + 1) * (1 + 0.3j)
+    prob = O.Problem(n, k, faces)
+    gen = torch.Generator(device="cuda").manual_seed(n)
+    x = torch.view_as_complex(torch.randn(prob.shape + (2,), dtype=torch.float64, device="cuda", generator=gen))
+    out = []
+    for form in ("auto", "fft"):
+        with H.Solver(n, k, faces, precision=H.FP64, method=H.SKS, transform=form) as s:
+            out.append(s.apply_Pinv(x))
+    # as above: the dense form's basis entries carry an argument rounding
+    assert float((out[0] - out[1]).abs().max()) <= 1e-11 * float(out[1].abs().max())
