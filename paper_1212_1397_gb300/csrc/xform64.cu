@@ -245,16 +245,19 @@ __device__ __forceinline__ int64_t level_sum(const float (&a)[DG]) {
 }
 
 // t 2^sc for an integer |t| < 2^63 and a scale that keeps every such result a normal number;
-// ebase = 1085 + sc.  `small`: 0 < |t| < 2^32, which the caller does another way.
-__device__ __forceinline__ double to_double(int64_t t, int ebase, bool& small) {
+// ebase = 1085 + sc.  (Integers below 2^32 by a shift, not by conversions: in a solve the high modes of
+// a smooth residual are that small against their row, and with FP64 conversions for them the x
+// transform of a smooth 255^3 field took 507 us instead of 412.)
+__device__ __forceinline__ double to_double(int64_t t, int ebase) {
   const int m = (int)(t >> 63);
-  const uint64_t u = (uint64_t)(t ^ m) - (int64_t)m;
+  const uint64_t w = (uint64_t)(t ^ m) - (int64_t)m;
+  const bool low = (uint32_t)(w >> 32) == 0;
+  const uint64_t u = low ? w << 31 : w;
   const uint32_t uh = (uint32_t)(u >> 32), ul = (uint32_t)u;
-  small = uh == 0 && ul != 0;
   const int lz = __clz((int)uh), sh = lz - 1;  // leading bit to 62
   const uint64_t n = ((uint64_t)__funnelshift_l(ul, uh, sh) << 32 | (ul << (sh & 31))) + 0x200u;
-  const uint32_t hi = (uint32_t)(n >> 42) + (uint32_t)(lz * -(1 << 20)) + ((uint32_t)ebase << 20);
-  return uh ? __hiloint2double((int)(hi | ((uint32_t)m & 0x80000000u)), (int)(uint32_t)(n >> 10)) : 0.0;
+  const uint32_t hi = (uint32_t)(n >> 42) + (uint32_t)((lz + (low ? 31 : 0)) * -(1 << 20)) + ((uint32_t)ebase << 20);
+  return w ? __hiloint2double((int)(hi | ((uint32_t)m & 0x80000000u)), (int)(uint32_t)(n >> 10)) : 0.0;
 }
 
 // The unit's tile (this CTA's first row) and group range.
@@ -639,13 +642,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(X_THREADS, 1) xform6
             float f[4][DG], big = 0.f;
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
-              float sum = 0.f;
 #pragma unroll
               for (int l = 0; l < DG; ++l) {
                 f[j][l] = __uint_as_float(a[l][j]);
-                sum += fabsf(f[j][l]);
+                big = fmaxf(big, fabsf(f[j][l]));
               }
-              big = fmaxf(big, sum);
             }
             if (!__any_sync(0xffffffffu, big > 4194304.f)) {
 #pragma unroll
@@ -664,14 +665,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(X_THREADS, 1) xform6
         for (int c = 0; c < X_NMAX / 4; c += 8) {
           if (c >= ncol) continue;
           double v[8];
-          bool any = false;
+          if (plain) {
 #pragma unroll
-          for (int j = 0; j < 8; ++j) {
-            bool small;
-            v[j] = to_double(T[c + j], 1085 + sc, small);
-            any = any || small;
-          }
-          if (any || !plain) {  // zeros and near zeros, rows at the ends of the exponent range, NaN and Inf
+            for (int j = 0; j < 8; ++j) v[j] = to_double(T[c + j], 1085 + sc);
+          } else {  // rows at the ends of the exponent range, NaN and Inf
 #pragma unroll
             for (int j = 0; j < 8; ++j)
               v[j] = nonfinite ? __longlong_as_double(0x7ff8000000000000ll) : scalbn(__ll2double_rn(T[c + j]), sc);

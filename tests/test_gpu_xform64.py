@@ -97,3 +97,17 @@ def test_modes_beyond_whole_groups(H, n, faces):
             out.append(s.apply_Pinv(x))
     # as above: the dense form's basis entries carry an argument rounding
     assert float((out[0] - out[1]).abs().max()) <= 1e-11 * float(out[1].abs().max())
+
+
+@pytest.mark.parametrize("eps", [0.0, 1e-18, 1e-9, 1e-4])
+def test_smooth_rows(H, eps):
+    """Rows of one low mode (and eps of noise): nearly all results are integers far below a row's scale,
+    down to single units and zeros; to a few roundings of the largest, like any other row."""
+    n, k, faces = 63, 12 + 4j, "DDNNSS"
+    prob = O.Problem(n, k, faces)
+    mz, my, mx = prob.shape
+    x = (np.sin(np.pi * np.arange(1, mx + 1) / (n + 1))[None, None, :] * np.cos(np.pi * np.arange(my) / (n + 1))[None, :, None]
+         * np.exp(-np.arange(mz) / 9.0)[:, None, None]).astype(np.complex128) * (1 - 0.5j)
+    x = x + eps * inputs.complex_normal(7, prob.shape)
+    ref = O.Preconditioner(prob)(x)
+    assert np.abs(pinv(H, n, k, faces, x) - ref).max() <= 1e-12 * np.abs(ref).max()
