@@ -67,12 +67,12 @@ KERNEL_OF = {
     "stencil": "stencil4_kernel",
     "xform_x_fwd": "xform_tc_kernel",
     "xform_y_fwd": "xform_tc_kernel",
-    "ztri": "ztri_lines_kernel<8>",
+    "ztri": "ztri_lines_kernel",
     "xform_y_inv": "xform_tc_kernel",
     "xform_x_inv": "xform_tc_kernel",
     "gs_dot": "dcgs_dot_kernel<float,{p},{tv}{dch}>",
     "gs_update": "dcgs_update_kernel<float,{p},{tv}{uch}>",
-    "resid64": "stencil_kernel<double,1>",
+    "resid64": "stencil64_kernel",
 }
 
 # DRAM bytes (ncu dram__bytes_read.sum + dram__bytes_write.sum) per launch and unknown of a
@@ -83,9 +83,9 @@ KERNEL_OF = {
 # DRAM bytes fall below the 16 B per unknown it reads and writes; the z lines read their input,
 # the pivot table twice (once per sweep) and their own forward results back.
 NCU_DRAM_BYTES_PER_UNKNOWN = {
-    "xform_tc_kernel": 12.736,
-    "ztri_lines_kernel<8>": 40.786,
-    "stencil4_kernel": 13.844,
+    "xform_tc_kernel": 12.690,
+    "ztri_lines_kernel": 40.730,
+    "stencil4_kernel": 13.794,
 }
 
 
