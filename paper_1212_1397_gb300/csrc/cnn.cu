@@ -16,6 +16,7 @@
 //                   pre-activations kept) and its input gradients (the transpose of a
 //                   zero-padded correlation is the correlation with the flipped,
 //                   channel-transposed taps; the FP32 gradient split into BF16 hi + lo)
+//   conv_brick_kernel  the same for the field path's layers on grids wider than 32 points
 //   wgrad_kernel    weight and bias gradients (SIMT, register tiles over 32x4x2-point tiles staged
 //                   with their halo in shared memory), block partials over persistent tiles
 //   mse_kernel, adam_kernel, prep_tc_kernel / prep_tcb_kernel (BF16 taps in the layouts the
@@ -402,6 +403,7 @@ constexpr int TC_TMEM = 64;                  // TMEM columns: 16 per tile
 constexpr int PLANE_B = (LMAX * GZ + 2) * 16;  // one point of padding each end
 constexpr int TCW_TAP = 512;                                  // bytes of one tap's 16 x 16 BF16
 constexpr size_t TC_SMEM = 1024 + 2 * (size_t)PLANE_B + 27 * TCW_TAP + 64 + 8 * LMAX;
+constexpr size_t BRICK_SMEM = 1024 + 2 * (size_t)(GX * GY * GZ + 2) * 16 + 27 * TCW_TAP + 256;
 constexpr size_t TC_SMEM4 = 1024 + 4 * (size_t)PLANE_B + 27 * TCW_TAP + 64 + 8 * LMAX;  // IN_G32: hi and lo planes
 // threads of a CTA: with four planes two CTAs share an SM, with two planes four
 template <int IN>
@@ -698,6 +700,177 @@ __global__ void __launch_bounds__(conv_threads<IN>()) conv_tc_kernel(TcConvArgs 
   if (tid == 0 && *fail) atomicExch(a.err, 1);
 }
 
+// The field path's layers on wide grids: bricks only, one thread per halo point and per output row,
+// results stored as they come (layers in and out in 16-byte pieces already).  On 256^3 fields the
+// general kernel costs more (4.74 ms for the two-stage preconditioner against 4.29 with
+// this one); on FP32 layers and narrow images that one is faster.
+template <int IN, int OUT>
+__global__ void __launch_bounds__(128) conv_brick_kernel(TcConvArgs a) {
+  extern __shared__ uint8_t smem_raw[];
+  constexpr int GP = GX * GY * GZ, PB = (GP + 2) * 16;  // halo points; bytes of a channel plane
+  uint8_t* sm = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+  uint8_t* plane0 = sm + 16;               // point -1 at sm, point 0 at sm + 16
+  uint8_t* plane1 = plane0 + PB;
+  uint8_t* wts = sm + 2 * PB;       // 27 x 512 B (1024-aligned base + 2 * PB: 16-aligned)
+  uint64_t* bar = (uint64_t*)(wts + 27 * TCW_TAP);
+  uint32_t* tslot = (uint32_t*)(bar + 1);
+  int* fail = (int*)(tslot + 1);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int64_t npts = (int64_t)a.nz * a.ny * a.nx;
+
+  int64_t b = blockIdx.x;
+  const int ibx = (int)(b % a.bx);
+  b /= a.bx;
+  const int iby = (int)(b % a.by);
+  b /= a.by;
+  const int ibz = (int)(b % a.bz);
+  const int64_t img = b / a.bz;
+  const int x0 = ibx * BX - 1, y0 = iby * BY - 1, z0 = ibz * BZ - 1;  // global coordinate of halo (0,0,0)
+
+  // weights: 27 x 512 B
+  for (int i = tid; i < 27 * TCW_TAP / 16; i += 128) cp16(smem_u32(wts) + 16u * i, (const uint4*)a.w + i, true);
+  // halo planes
+  float sc = 1.f;
+  if constexpr (IN == IN_PLANAR) {
+    const double ss = *a.sumsq;
+    sc = ss > 0.0 ? (float)(1.0 / sqrt(ss / (double)npts)) : 0.f;
+  }
+  if constexpr (IN == IN_PLANAR) {
+    // the planar FP32 field: every load of the thread's halo points issued before any is used
+    constexpr int PER = (GP + 127) / 128;
+    const float* f = (const float*)a.in;
+    float re[PER], im[PER];
+#pragma unroll
+    for (int k = 0; k < PER; ++k) {
+      const int i = tid + 128 * k;
+      const int hx = i % GX, r = i / GX, hy = r % GY, hz = r / GY;
+      const int gx = x0 + hx, gy = y0 + hy, gz = z0 + hz;
+      const bool ok = i < GP && gx >= 0 && gx < a.nx && gy >= 0 && gy < a.ny && gz >= 0 && gz < a.nz;
+      const int64_t p = ok ? ((img * a.nz + gz) * a.ny + gy) * a.nx + gx : 0;
+      re[k] = ok ? f[p] : 0.f;
+      im[k] = ok ? f[npts + p] : 0.f;
+    }
+#pragma unroll
+    for (int k = 0; k < PER; ++k) {
+      const int i = tid + 128 * k;
+      if (i < GP) {
+        *(uint4*)(plane0 + 16 * i) = make_uint4(pack_bf16(re[k] * sc, im[k] * sc), 0u, 0u, 0u);
+        *(uint4*)(plane1 + 16 * i) = make_uint4(0u, 0u, 0u, 0u);
+      }
+    }
+  }
+  for (int i = tid; i < GP && IN != IN_PLANAR; i += 128) {
+    const int hx = i % GX, r = i / GX, hy = r % GY, hz = r / GY;
+    const int gx = x0 + hx, gy = y0 + hy, gz = z0 + hz;
+    const bool ok = gx >= 0 && gx < a.nx && gy >= 0 && gy < a.ny && gz >= 0 && gz < a.nz;
+    const int64_t p = ok ? ((img * a.nz + gz) * a.ny + gy) * a.nx + gx : 0;
+    if constexpr (IN == IN_BF16) {
+      const uint4* src = (const uint4*)a.in + 2 * p;
+      cp16(smem_u32(plane0) + 16u * i, src, ok);
+      cp16(smem_u32(plane1) + 16u * i, src + 1, ok);
+    }
+  }
+  if (tid < 2) {  // the padding points before and after each plane
+    *(uint4*)(sm + tid * PB) = make_uint4(0u, 0u, 0u, 0u);
+    *(uint4*)(plane0 + tid * PB + 16 * GP) = make_uint4(0u, 0u, 0u, 0u);
+  }
+  if (tid == 0) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(1));
+    asm volatile("fence.mbarrier_init.release.cluster;");
+    *fail = 0;
+  }
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tslot)),
+                 "r"(TC_TMEM));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+  }
+  asm volatile("cp.async.wait_all;" ::: "memory");
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  asm volatile("tcgen05.fence::before_thread_sync;");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;");
+  const uint32_t tmem = *tslot;
+
+  if (tid == 0) {
+    // kind::f16, D = F32, A = B = BF16, K-major, M = 128, N = 16
+    const uint32_t id = (1u << 4) | (1u << 7) | (1u << 10) | (2u << 17) | (8u << 24);
+    const uint32_t p0 = smem_u32(plane0);
+    for (int tile = 0; tile < TC_TILES; ++tile) {
+      const int hz = 1 + tile / (BY / 4), hy = 1 + 4 * (tile % (BY / 4));
+      const int q0 = (hz * GY + hy) * GX;
+      for (int t = 0; t < 27; ++t) {
+        const int dz = t / 9 - 1, dy = (t / 3) % 3 - 1, dx = t % 3 - 1;
+        const int q = q0 + (dz * GY + dy) * GX + dx;  // in [-1, GP - 128]: the padding covers -1 and GP
+        const uint64_t ad = desc_noswz(p0 + (uint32_t)(q * 16), PB, 128);
+        const uint64_t bd = desc_noswz(smem_u32(wts) + (uint32_t)(t * TCW_TAP), 128, 256);
+        mma_bf16(tmem + 16u * tile, ad, bd, id, t > 0 ? 1u : 0u);
+      }
+    }
+    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
+                 : "memory");
+  }
+  __syncthreads();
+  bool ok = false;
+  for (int it = 0; it < kConvPolls; ++it) {
+    uint32_t r;
+    asm volatile(
+        "{\n .reg .pred P1;\n mbarrier.try_wait.parity.shared::cta.b64 P1, [%1], %2;\n"
+        " selp.b32 %0, 1, 0, P1;\n}\n"
+        : "=r"(r)
+        : "r"(smem_u32(bar)), "r"(0)
+        : "memory");
+    if (r) {
+      ok = true;
+      break;
+    }
+  }
+  asm volatile("tcgen05.fence::after_thread_sync;");
+  if (!ok) {
+    *fail = 1;
+  } else {
+    float bias[16];
+#pragma unroll
+    for (int c = 0; c < 16; ++c) bias[c] = (OUT == OUT_HIDDEN || c < 2) ? a.bias[c] : 0.f;
+    float cs = 0.f;
+    if constexpr (OUT == OUT_FIELD) {
+      const double ss = *a.sumsq;
+      cs = ss > 0.0 ? a.out_scale * (float)sqrt(ss / (double)npts) : 0.f;
+    }
+    for (int tile = 0; tile < TC_TILES; ++tile) {
+      uint32_t v[16];
+      asm volatile(
+          "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+          : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
+            "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
+          : "r"(tmem + ((uint32_t)(32 * warp) << 16) + 16u * tile));
+      asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+      const int r = 32 * warp + lane;  // row of the tile: halo x = r % 32, y = hy + r / 32
+      const int hx = r % GX, hz = 1 + tile / (BY / 4), hy = 1 + 4 * (tile % (BY / 4)) + r / GX;
+      const int gx = x0 + hx, gy = y0 + hy, gz = z0 + hz;
+      if (hx < 1 || hx > BX || gx >= a.nx || gy >= a.ny || gz >= a.nz) continue;
+      const int64_t p = ((img * a.nz + gz) * a.ny + gy) * a.nx + gx;
+      if constexpr (OUT == OUT_HIDDEN) {
+        uint32_t pk[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+          pk[q] = pack_bf16(gelu_f(__uint_as_float(v[2 * q]) + bias[2 * q]),
+                            gelu_f(__uint_as_float(v[2 * q + 1]) + bias[2 * q + 1]));
+        uint4* o4 = (uint4*)a.out + 2 * p;
+        o4[0] = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+        o4[1] = make_uint4(pk[4], pk[5], pk[6], pk[7]);
+      } else {
+        float* z = (float*)a.out;
+        z[p] = fmaf(cs, __uint_as_float(v[0]) + bias[0], z[p]);
+        z[npts + p] = fmaf(cs, __uint_as_float(v[1]) + bias[1], z[npts + p]);
+      }
+    }
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;");
+  __syncthreads();
+  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TC_TMEM));
+  if (tid == 0 && *fail) atomicExch(a.err, 1);
+}
+
 // Bricks or runs.  An image up to 32 points wide is taken as runs of 128 points of its planes' rows
 // joined by one zero point each (the right neighbour of a row's end and the left one of the next
 // row's beginning): a run's halo is no larger than a brick's, a row of nx points costs nx + 1 places
@@ -836,6 +1009,9 @@ int cnn_configure() {
       {(const void*)conv_tc_kernel<IN_PLANAR, OUT_HIDDEN>, TC_SMEM},
       {(const void*)conv_tc_kernel<IN_BF16, OUT_HIDDEN>, TC_SMEM},
       {(const void*)conv_tc_kernel<IN_BF16, OUT_FIELD>, TC_SMEM},
+      {(const void*)conv_brick_kernel<IN_PLANAR, OUT_HIDDEN>, BRICK_SMEM},
+      {(const void*)conv_brick_kernel<IN_BF16, OUT_HIDDEN>, BRICK_SMEM},
+      {(const void*)conv_brick_kernel<IN_BF16, OUT_FIELD>, BRICK_SMEM},
       // the trainer's layers
       {(const void*)conv_tc_kernel<IN_F32, OUT_HIDDEN>, TC_SMEM},
       {(const void*)conv_tc_kernel<IN_BF16, OUT_F32>, TC_SMEM},
@@ -866,6 +1042,7 @@ int cnn_apply_field(const CnnNet& net, int nz, int ny, int nx, const float* t, c
   a.out_scale = out_scale;
   a.err = err;
   const unsigned grid = (unsigned)((int64_t)a.bx * a.by * a.bz);
+  const size_t sm = a.run ? TC_SMEM : BRICK_SMEM;
   const uint16_t* in[4] = {nullptr, act0, act1, act0};
   void* out[4] = {act0, act1, act0, z};
   note_launch(4);
@@ -875,11 +1052,11 @@ int cnn_apply_field(const CnnNet& net, int nz, int ny, int nx, const float* t, c
     a.bias = net.theta + d.boff[l];
     a.out = out[l];
     if (l == 0)
-      conv_tc_kernel<IN_PLANAR, OUT_HIDDEN><<<grid, 128, TC_SMEM, s>>>(a);
+      (a.run ? conv_tc_kernel<IN_PLANAR, OUT_HIDDEN> : conv_brick_kernel<IN_PLANAR, OUT_HIDDEN>)<<<grid, 128, sm, s>>>(a);
     else if (l < NL - 1)
-      conv_tc_kernel<IN_BF16, OUT_HIDDEN><<<grid, 128, TC_SMEM, s>>>(a);
+      (a.run ? conv_tc_kernel<IN_BF16, OUT_HIDDEN> : conv_brick_kernel<IN_BF16, OUT_HIDDEN>)<<<grid, 128, sm, s>>>(a);
     else
-      conv_tc_kernel<IN_BF16, OUT_FIELD><<<grid, 128, TC_SMEM, s>>>(a);
+      (a.run ? conv_tc_kernel<IN_BF16, OUT_FIELD> : conv_brick_kernel<IN_BF16, OUT_FIELD>)<<<grid, 128, sm, s>>>(a);
   }
   return cudaGetLastError() == cudaSuccess ? HELM6_OK : HELM6_ERR_CUDA;
 }
