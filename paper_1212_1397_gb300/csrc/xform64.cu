@@ -28,7 +28,8 @@
 //   * eight converter warps in two groups taking alternate stages copy a stage's row segments
 //     (the mirrored ones too) into an FP64 ring with cp.async and turn them into the seven FP16
 //     digit planes of the A operand;
-//   * a producer thread streams its CTA's half of the basis' digit planes (cp.async.bulk);
+//   * a producer thread streams its CTA's half of the basis' digit planes (cp.async.bulk) and passes
+//     each landed copy on to the stage's barrier (the MMA warp's waiting on both took 4 % of A_p^-1);
 //   * the MMA warp of the first CTA issues the 28 products of a stage for both; the second one's passes
 //     its operands' barrier on to the first one's, so that each waits once per stage;
 //   * eight epilogue warps take the finished sums out of tensor memory as 64-bit integers,
@@ -41,8 +42,8 @@
 // (multiply-adds, FP32 sums as integer conversions): an FP64 operation or conversion takes a
 // scheduler 64 cycles, an FP32-to-integer conversion 8, a logic operation or a carry 2, an
 // integer or FP32 multiply-add 1 (measured).
-// Every wait is bounded; a timeout sets *err, and each CTA still waits for the MMAs and copies in
-// flight before it frees tensor memory.
+// Every wait is bounded; a timeout sets *err, and each CTA still waits (bounded, whatever the other
+// roles do) for the MMAs and copies in flight before it frees tensor memory.
 #include <cuda_fp16.h>
 
 #include <algorithm>
@@ -50,6 +51,7 @@
 #include <cstring>
 
 #include "helm6_internal.h"
+#include "waits.h"
 
 namespace helm6 {
 
@@ -79,7 +81,7 @@ constexpr int O_D = O_B + X_NS * B_BYTES;
 constexpr int O_S = O_D + X_ND * D_BYTES;
 constexpr int O_E = O_S + X_EPI * STG_BYTES;   // row exponents, two units
 constexpr int O_BAR = O_E + 2 * X_M * 4;
-constexpr int X_NBAR = 2 * X_NS + 7;
+constexpr int X_NBAR = 3 * X_NS + 7;
 constexpr int O_MISC = O_BAR + X_NBAR * 8;
 constexpr int X_SMEM = O_MISC + 16 + 1024;
 static_assert(X_SMEM <= 232448, "shared memory per CTA");
@@ -123,18 +125,30 @@ __device__ __forceinline__ bool try_wait(uint32_t bar, uint32_t parity) {
   return ok != 0;
 }
 
+// One look at a phase, without the suspension of try_wait.
+__device__ __forceinline__ bool test_wait(uint32_t bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n .reg .pred P1;\n mbarrier.test_wait.parity.shared::cta.b64 P1, [%1], %2;\n"
+      " selp.b32 %0, 1, 0, P1;\n}\n"
+      : "=r"(ok)
+      : "r"(bar), "r"(parity)
+      : "memory");
+  return ok != 0;
+}
+
 // Bounded wait by one thread; gives up when the flag is raised by another role.  It sleeps between
 // polls: a spinning warp's issue slots are the converters' and the epilogue's (measured: half of
 // all instructions were polls).
 template <int NAP>
 __device__ __forceinline__ bool poll1(uint32_t bar, uint32_t parity, volatile int* fail) {
-  for (int it = 0; it < kPolls; ++it) {
-    if (try_wait(bar, parity)) return true;
-    if ((it & 63) == 63 && *fail) return false;
-    __nanosleep(NAP);
-  }
-  *fail = 1;
-  return false;
+  return wait_role([=] { return try_wait(bar, parity); }, [] { __nanosleep(NAP); }, fail, kPolls, 64);
+}
+
+// Bounded wait for products or copies under way, whatever the other roles do.  (In the second CTA the
+// products' barrier also waits for the first one's MMA warp to end, after one bounded wait at most.)
+__device__ __forceinline__ void poll_flight(uint32_t bar, uint32_t parity, volatile int* fail) {
+  wait_flight([=] { return try_wait(bar, parity); }, [] { __nanosleep(100); }, fail, 4ll * kPolls);
 }
 
 // Warp-uniform bounded wait: every lane polls.  (Lane 0 alone and a shuffle of its answer: the warp
@@ -331,17 +345,19 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(X_THREADS, 1) xform6
   const uint32_t bar0 = s_addr(smem + O_BAR);
   auto full = [&](int s) { return bar0 + 8u * s; };            // the stage's operands are there (first CTA: in both)
   auto sfree = [&](int s) { return bar0 + 8u * (X_NS + s); };  // the stage's MMAs completed
-  const uint32_t tfull = bar0 + 8u * (2 * X_NS);                   // the group's accumulators complete
-  const uint32_t tempty = bar0 + 8u * (2 * X_NS + 1);              // first CTA: ... and drained in both
-  auto efull = [&](int b) { return bar0 + 8u * (2 * X_NS + 2 + b); };  // row exponents of a unit known
-  auto efree = [&](int b) { return bar0 + 8u * (2 * X_NS + 5 + b); };  // ... and read by everybody
-  const uint32_t drain = bar0 + 8u * (2 * X_NS + 4);               // every MMA issued completed
+  auto bfull = [&](int s) { return bar0 + 8u * (2 * X_NS + s); };  // its basis digits are (its copy alone completes it)
+  const uint32_t tfull = bar0 + 8u * (3 * X_NS);                   // the group's accumulators complete
+  const uint32_t tempty = bar0 + 8u * (3 * X_NS + 1);              // first CTA: ... and drained in both
+  auto efull = [&](int b) { return bar0 + 8u * (3 * X_NS + 2 + b); };  // row exponents of a unit known
+  auto efree = [&](int b) { return bar0 + 8u * (3 * X_NS + 5 + b); };  // ... and read by everybody
+  const uint32_t drain = bar0 + 8u * (3 * X_NS + 4);               // every MMA issued completed
 
   if (tid == 0) {
     auto init = [](uint32_t b, int n) { asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(b), "r"(n)); };
     for (int s = 0; s < X_NS; ++s) {
       init(full(s), 4 + (rank ? 1 : 2));  // a converter group, the producer; first CTA: the relay
       init(sfree(s), 1);
+      init(bfull(s), 1);
     }
     init(tfull, 1);
     init(tempty, 2 * X_EPI);
@@ -368,28 +384,47 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(X_THREADS, 1) xform6
   const uint32_t bplane = (uint32_t)p.npad * X_KT, bstage = DG * bplane;  // this CTA's half of the modes
 
   if (warp == X_WPROD) {
-    // ---- basis producer ----
+    // ---- basis producer: copies as slots come free, and each landed copy passed on to the stage's
+    // barrier ----
     if (lane == 0) {
-      int q = 0, last = -1;
-      for (int i = 0; i < nun && !*fail; ++i) {
-        const Unit un = unit_at(i);
-        for (int g = un.g0; g < un.g1 && !*fail; ++g) {
-          const uint8_t* Wg = p.W + ((size_t)g * p.nk * 2 + rank) * bstage;
-          for (int kt = 0; kt < p.nk; ++kt, ++q) {
-            const int s = q % X_NS, u = q / X_NS;
-            if (u >= 1 && !poll1<100>(sfree(s), (u - 1) & 1, fail)) break;
-            const uint32_t bar = full(s);
-            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bstage) : "memory");
-            asm volatile(
-                "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                    s_addr(smem + O_B + s * B_BYTES)),
-                "l"(Wg + (size_t)kt * 2 * bstage), "r"(bstage), "r"(bar)
-                : "memory");
-            last = q;
+      // unit, group and K stage of copy q; copies before r have landed
+      int i = 0, g = 0, kt = 0, q = 0, r = 0, idle = 0;
+      Unit un = unit_at(0);
+      while ((i < nun || r < q) && idle < kPolls) {
+        bool step = false;
+        if (i < nun && (q < X_NS || test_wait(sfree(q % X_NS), (q / X_NS - 1) & 1))) {
+          const uint8_t* src = p.W + (((size_t)(un.g0 + g) * p.nk + kt) * 2 + rank) * bstage;
+          const uint32_t bar = bfull(q % X_NS);
+          asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bstage) : "memory");
+          asm volatile(
+              "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                  s_addr(smem + O_B + (q % X_NS) * B_BYTES)),
+              "l"(src), "r"(bstage), "r"(bar)
+              : "memory");
+          ++q;
+          if (++kt == p.nk) {
+            kt = 0;
+            if (un.g0 + ++g == un.g1) {
+              g = 0;
+              un = unit_at(++i);
+            }
           }
+          step = true;
+        }
+        if (r < q && test_wait(bfull(r % X_NS), (r / X_NS) & 1)) {
+          arrive(full(r % X_NS));
+          ++r;
+          step = true;
+        }
+        if (step) {
+          idle = 0;
+        } else {
+          if ((++idle & 63) == 0 && *fail) break;
+          __nanosleep(50);
         }
       }
-      if (last >= 0) poll1<100>(full(last % X_NS), (last / X_NS) & 1, fail);  // the last copy has landed
+      if (idle == kPolls) *fail = 1;
+      for (; r < q; ++r) poll_flight(bfull(r % X_NS), (r / X_NS) & 1, fail);  // every copy has landed before the CTA ends
     }
     __syncwarp();
   } else if (warp == X_WMMA) {
@@ -438,7 +473,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(X_THREADS, 1) xform6
     }
     // every MMA issued above has completed before either CTA frees its tensor memory
     if (rank == 0) commit(drain);
-    poll1<20>(drain, 0, fail);
+    poll_flight(drain, 0, fail);
     __syncwarp();
   } else if (warp > X_WMMA) {
     // ---- scanners: the largest |x| high word of each row, four rows at a time (the loads in flight,

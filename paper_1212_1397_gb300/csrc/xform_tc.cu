@@ -19,7 +19,9 @@
 //     the 258-point Neumann axes) are accumulated in FP32 by the same threads from the values
 //     they already hold, and written by them;
 //   * one producer thread streams the basis stage (hi and lo tiles, prepared on the host) into the
-//     basis ring with cp.async.bulk, completing on `full` too: the MMA warp waits once per stage;
+//     basis ring with cp.async.bulk, completing on `bfull`, a barrier that waits for nothing else, and
+//     passes each landed copy on to `full`, so that the MMA warp waits once per stage (its waiting on
+//     both took 1 % of a solve);
 //   * one MMA warp issues the tcgen05.mma's (one elected lane, operands in uniform registers) into
 //     one of two 256-column tensor-memory accumulators and commits them to `sfree` (which
 //     releases the stage's operand slots) and, after a tile's last stage, to `tfull`;
@@ -38,15 +40,16 @@
 // (20/19/21/16).  CTA pairs (cta_group::2, half the shared-memory traffic per product) measured
 // the same at 256^3 and 1.5 to 2 us slower per transform below 160^3.
 // Every mbarrier wait is bounded and warp-uniform; a timeout sets a shared flag that ends
-// every role's loop, and *err for the host.  Whatever the path, the CTA waits (bounded) for its committed
-// MMAs, the producer for its last bulk copy and the converters for their cp.async groups before
-// the tensor memory is freed.
+// every role's loop, and *err for the host.  Whatever the path, the CTA waits (bounded, and the flag
+// does not end these waits) for its committed MMAs, the producer for its bulk copies and the
+// converters for their cp.async groups before the tensor memory is freed.
 #include <cuda_bf16.h>
 
 #include <algorithm>
 #include <cstring>
 
 #include "helm6_internal.h"
+#include "waits.h"
 
 namespace helm6 {
 
@@ -79,7 +82,7 @@ constexpr int OFF_D = OFF_B + NS * B_STAGE;
 constexpr int OFF_T = OFF_D + ND * D_STAGE;
 constexpr int OFF_S = OFF_T + TAIL_FLOATS * 4;
 constexpr int OFF_BAR = OFF_S + EPI_WARPS * STG_FLOATS * 4;
-constexpr int NBAR = 2 * NS + 5;  // full, sfree per stage; tfull, tempty per buffer; drain
+constexpr int NBAR = 3 * NS + 5;  // full, bfull, sfree per stage; tfull, tempty per buffer; drain
 constexpr int OFF_MISC = OFF_BAR + NBAR * 8;
 constexpr int SMEM_BYTES = OFF_MISC + 16 + 1024;  // + alignment of the base to 1024
 static_assert(SMEM_BYTES <= 232448, "shared memory per CTA");
@@ -126,14 +129,26 @@ __device__ __forceinline__ bool try_wait(uint32_t bar, uint32_t parity) {
   return ok != 0;
 }
 
+// One look at a phase, without the suspension of try_wait.
+__device__ __forceinline__ bool test_wait(uint32_t bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n .reg .pred P1;\n mbarrier.test_wait.parity.shared::cta.b64 P1, [%1], %2;\n"
+      " selp.b32 %0, 1, 0, P1;\n}\n"
+      : "=r"(ok)
+      : "r"(bar), "r"(parity)
+      : "memory");
+  return ok != 0;
+}
+
 // Bounded wait by one thread; gives up when the flag is raised by another role.
 __device__ __forceinline__ bool poll1(uint32_t bar, uint32_t parity, volatile int* fail) {
-  for (int it = 0; it < kMaxPolls; ++it) {
-    if (try_wait(bar, parity)) return true;
-    if ((it & 255) == 255 && *fail) return false;
-  }
-  *fail = 1;
-  return false;
+  return wait_role([=] { return try_wait(bar, parity); }, [] {}, fail, kMaxPolls, 256);
+}
+
+// Bounded wait for products or copies under way, whatever the other roles do.
+__device__ __forceinline__ void poll_flight(uint32_t bar, uint32_t parity, volatile int* fail) {
+  wait_flight([=] { return try_wait(bar, parity); }, [] {}, fail, kMaxPolls);
 }
 
 // Warp-uniform bounded wait: every lane polls.  With lane 0 alone polling and a shuffle of its
@@ -233,15 +248,17 @@ __global__ void __launch_bounds__(TC_THREADS, 1) xform_tc_kernel(TcArgs p) {
   uint32_t* tslot = (uint32_t*)(smem + OFF_MISC);
   volatile int* fail = (volatile int*)(tslot + 1);
   const uint32_t bar0 = s_addr(bars);
-  auto full = [&](int s) { return bar0 + 8u * s; };          // the stage's operands are there
-  auto sfree = [&](int s) { return bar0 + 8u * (NS + s); };  // the stage's MMAs completed
-  auto tfull = [&](int b) { return bar0 + 8u * (2 * NS + b); };  // accumulator b complete
-  auto tempty = [&](int b) { return bar0 + 8u * (2 * NS + 2 + b); };  // accumulator b drained
-  const uint32_t drain = bar0 + 8u * (2 * NS + 4);                 // every MMA issued completed
+  auto full = [&](int s) { return bar0 + 8u * s; };              // the stage's operands are there
+  auto bfull = [&](int s) { return bar0 + 8u * (NS + s); };      // basis stage arrived (its copy alone completes it)
+  auto sfree = [&](int s) { return bar0 + 8u * (2 * NS + s); };  // the stage's MMAs completed
+  auto tfull = [&](int b) { return bar0 + 8u * (3 * NS + b); };  // accumulator b complete
+  auto tempty = [&](int b) { return bar0 + 8u * (3 * NS + 2 + b); };  // accumulator b drained
+  const uint32_t drain = bar0 + 8u * (3 * NS + 4);                 // every MMA issued completed
 
   if (tid == 0) {
     for (int s = 0; s < NS; ++s) {
       asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(full(s)), "r"(CONV_WARPS + 1));
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bfull(s)), "r"(1));
       asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(sfree(s)), "r"(1));
     }
     for (int b = 0; b < 2; ++b) {
@@ -271,27 +288,40 @@ __global__ void __launch_bounds__(TC_THREADS, 1) xform_tc_kernel(TcArgs p) {
   auto item_at = [&](int i) { return item(p, (int)blockIdx.x + i * (int)gridDim.x); };
 
   if (warp == W_PROD) {
-    // ---- basis producer ----
-    int last = -1;
+    // ---- basis producer: copies as slots come free, and each landed copy passed on to the stage's
+    // barrier ----
     if (lane == 0) {
-      int g = 0;
-      for (int i = 0; i < nitems && !*fail; ++i) {
-        const Item it = item_at(i);
-        const int bterm = TC_KC * it.npad * 16;
-        const int btx = (p.terms == 3 ? 2 : 1) * bterm;
-        const uint8_t* Wg = p.W + (size_t)it.grp * p.nk * 2 * TC_KC * p.gcols * 16;
-        for (int kt = 0; kt < p.nk; ++kt, ++g) {
-          const int s = g % NS, u = g / NS;
-          if (u >= 1 && !poll1(sfree(s), (u - 1) & 1, fail)) break;
-          const uint32_t dst = s_addr(smem + OFF_B + s * B_STAGE), bar = full(s);
+      int i = 0, kt = 0, q = 0, r = 0, idle = 0;  // item and K stage of copy q; copies before r have landed
+      while ((i < nitems || r < q) && idle < kMaxPolls) {
+        bool step = false;
+        if (i < nitems && (q < NS || test_wait(sfree(q % NS), (q / NS - 1) & 1))) {
+          const Item it = item_at(i);
+          const int bterm = TC_KC * it.npad * 16, btx = (p.terms == 3 ? 2 : 1) * bterm;
+          const uint8_t* Wg = p.W + (size_t)it.grp * p.nk * 2 * TC_KC * p.gcols * 16;
+          const uint32_t bar = bfull(q % NS);
           asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(btx) : "memory");
-          bulk(dst, Wg + (size_t)kt * 2 * bterm, btx, bar);
-          last = g;
+          bulk(s_addr(smem + OFF_B + (q % NS) * B_STAGE), Wg + (size_t)kt * 2 * bterm, btx, bar);
+          ++q;
+          if (++kt == p.nk) {
+            kt = 0;
+            ++i;
+          }
+          step = true;
         }
-        if (*fail) break;
+        if (r < q && test_wait(bfull(r % NS), (r / NS) & 1)) {
+          arrive(full(r % NS));
+          ++r;
+          step = true;
+        }
+        if (step) {
+          idle = 0;
+        } else {
+          if ((++idle & 63) == 0 && *fail) break;
+          __nanosleep(50);
+        }
       }
-      // the last copy must have landed before the CTA ends
-      if (last >= 0) poll1(full(last % NS), (last / NS) & 1, fail);
+      if (idle == kMaxPolls) *fail = 1;
+      for (; r < q; ++r) poll_flight(bfull(r % NS), (r / NS) & 1, fail);  // every copy has landed before the CTA ends
     }
     __syncwarp();
   } else if (warp == W_MMA) {
@@ -332,7 +362,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) xform_tc_kernel(TcArgs p) {
     }
     // every MMA issued above has completed before the tensor memory is freed
     commit(drain);
-    poll1(drain, 0, fail);
+    poll_flight(drain, 0, fail);
     __syncwarp();
   } else if (warp >= EPI_WARPS) {
     // ---- converters: warp cw copies rows 16 cw .. 16 cw + 15 of each stage into the FP32
