@@ -65,6 +65,22 @@ struct TermRange {
   int lo[3], hi[3];
 };
 
+// Element idx of a complex array: 16 bytes at once where the arrays are aligned to that, else (a caller's
+// own buffers may be aligned to a double only) two doubles.
+__device__ __forceinline__ Z ldc(const double* p, int64_t idx, bool wide) {
+  if (!wide) return Z{p[2 * idx], p[2 * idx + 1]};
+  const double2 v = ((const double2*)p)[idx];
+  return Z{v.x, v.y};
+}
+__device__ __forceinline__ void stc(double* p, int64_t idx, const Z& v, bool wide) {
+  if (wide) {
+    ((double2*)p)[idx] = make_double2(v.re, v.im);
+  } else {
+    p[2 * idx] = v.re;
+    p[2 * idx + 1] = v.im;
+  }
+}
+
 constexpr int RHS_WARPS = 4, RHS_ROWS = 16, RHS_TERMS = 32;  // warps and x rows of a block, terms per pass
 
 // A Neumann or Sommerfeld-like face's data term is, per separable term with normal factor
@@ -113,7 +129,7 @@ __global__ void __launch_bounds__(32 * RHS_WARPS) rhs_kernel(Geom g, RhsCoef c, 
                                                              const double* __restrict__ tab,
                                                              const double* __restrict__ amps,
                                                              const TermRange* __restrict__ rng,
-                                                             const double* __restrict__ noise, double2* __restrict__ F) {
+                                                             const double* __restrict__ noise, double* __restrict__ F, bool wide) {
   using TT = TabT<REAL>;
   __shared__ Z sA[RHS_ROWS][RHS_TERMS], sB[RHS_ROWS][RHS_TERMS], sC[RHS_ROWS][RHS_TERMS], sE[RHS_ROWS][2][RHS_TERMS];
   __shared__ short2 sR[RHS_ROWS][RHS_TERMS];  // the term's nonzero x nodes (empty: skipped on this row)
@@ -171,13 +187,10 @@ __global__ void __launch_bounds__(32 * RHS_WARPS) rhs_kernel(Geom g, RhsCoef c, 
       for (int i = lane; i < g.mx; i += 32) {
         const int64_t idx = (row0 + r) * g.mx + i;
         Z v{0.0, 0.0};
-        if (t0 > 0) {
-          const double2 f = F[idx];
-          v = Z{f.x, f.y};
-        } else if (noise) {
-          const double2 q = ((const double2*)noise)[idx];
-          v = h2cf * Z{q.x, q.y};
-        }
+        if (t0 > 0)
+          v = ldc(F, idx, wide);
+        else if (noise)
+          v = h2cf * ldc(noise, idx, wide);
         for (int s = 0; s < nt; ++s) {
           const short2 q = sR[r][s];
           if (i < q.x || i >= q.y) continue;
@@ -188,7 +201,7 @@ __global__ void __launch_bounds__(32 * RHS_WARPS) rhs_kernel(Geom g, RhsCoef c, 
           if (i == 0) v = v - sE[r][0][s];
           if (i == g.mx - 1) v = v - sE[r][1][s];
         }
-        F[idx] = make_double2(v.re, v.im);
+        stc(F, idx, v, wide);
       }
     }
     __syncthreads();
@@ -268,11 +281,12 @@ int launch_rhs(const Geom& g, double h, cd k, int nterm, int mmax, const double*
   const unsigned grid = (unsigned)((rows + RHS_ROWS - 1) / RHS_ROWS);
   const double* damp = dbuf + ntab;
   const TermRange* drng = (const TermRange*)(damp + 2 * (size_t)nterm);
+  const bool wide = ((uintptr_t)F | (uintptr_t)noise) % 16 == 0;
   note_launch();
   if (real)
-    rhs_kernel<true><<<grid, 32 * RHS_WARPS, 0, s>>>(g, c, nterm, mmax, dbuf, damp, drng, noise, (double2*)F);
+    rhs_kernel<true><<<grid, 32 * RHS_WARPS, 0, s>>>(g, c, nterm, mmax, dbuf, damp, drng, noise, F, wide);
   else
-    rhs_kernel<false><<<grid, 32 * RHS_WARPS, 0, s>>>(g, c, nterm, mmax, dbuf, damp, drng, noise, (double2*)F);
+    rhs_kernel<false><<<grid, 32 * RHS_WARPS, 0, s>>>(g, c, nterm, mmax, dbuf, damp, drng, noise, F, wide);
   cudaFreeAsync(dbuf, s);
   return cudaGetLastError() == cudaSuccess ? HELM6_OK : HELM6_ERR_CUDA;
 }
