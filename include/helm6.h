@@ -359,7 +359,10 @@ int helm6_apply_stage2(helm6_ctx* ctx, const void* x, void* y);
  * stored channel-last as DEVICE float arrays [batch][nz][ny][nx][2].  Zero padding at every
  * image's border.  The gradient is that of the rounded network with each rounding taken
  * as the identity (straight-through) and the GELU differentiated at its FP32 input.
- * theta0: HOST initial parameters.  All work is on `stream` (NULL = default). */
+ * theta0: HOST initial parameters.  All work is on `stream` (NULL = default).
+ * Where a bounded wait on the GPU runs out, a call that synchronises returns HELM6_ERR_CUDA, the
+ * arrays that the call writes hold NaN, and no Adam step is taken; a step not taken in a call
+ * without a loss is reported by the next call that synchronises. */
 typedef struct helm6_cnn_trainer helm6_cnn_trainer;
 int helm6_cnn_trainer_create(helm6_cnn_trainer** out, int batch, int nz, int ny, int nx,
                              const float* theta0, void* stream);

@@ -30,6 +30,7 @@
 #include <vector>
 
 #include "helm6_internal.h"
+#include "waits.h"
 
 namespace helm6 {
 
@@ -289,9 +290,14 @@ __global__ void mse_kernel(const float* __restrict__ y, const float* __restrict_
 }
 
 // Adam (beta1 0.9, beta2 0.999, eps 1e-8) with bias corrections c1 = 1 - beta1^t, c2 = 1 - beta2^t.
+// Where a layer's wait has timed out (err[0]) the gradient is not one: no step is taken, and err[1] keeps that.
 __global__ void adam_kernel(float* __restrict__ theta, float* __restrict__ m, float* __restrict__ v,
-                            const float* __restrict__ g, int n, float lr, float c1, float c2) {
+                            const float* __restrict__ g, int n, float lr, float c1, float c2, int* err) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (err[0]) {
+    if (i == 0) err[1] = 1;
+    return;
+  }
   if (i >= n) return;
   const float gi = g[i];
   const float mi = 0.9f * m[i] + 0.1f * gi;
@@ -299,6 +305,20 @@ __global__ void adam_kernel(float* __restrict__ theta, float* __restrict__ m, fl
   m[i] = mi;
   v[i] = vi;
   theta[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + 1e-8f);
+}
+
+// A call's result to the caller's array: src, or NaN throughout where a layer's wait has timed out (a
+// call that does not synchronise has no other way to say so).  Four loads of a thread in flight.
+__global__ void __launch_bounds__(256) result_copy_kernel(const float* __restrict__ src, float* __restrict__ dst,
+                                                          int64_t n, const int* __restrict__ err) {
+  const bool bad = *err != 0;
+  const int64_t i0 = (int64_t)blockIdx.x * 1024 + threadIdx.x;
+  float v[4];
+#pragma unroll
+  for (int e = 0; e < 4; ++e) v[e] = i0 + 256 * e < n ? src[i0 + 256 * e] : 0.f;
+#pragma unroll
+  for (int e = 0; e < 4; ++e)
+    if (i0 + 256 * e < n) dst[i0 + 256 * e] = bad ? __int_as_float(0x7fc00000) : v[e];
 }
 
 // Interior 27-point operator on channel-last complex patches [pts][2] with zero values
@@ -410,7 +430,7 @@ template <int IN>
 constexpr int conv_threads() {
   return IN == IN_G32 ? 256 : 128;
 }
-constexpr int kConvPolls = 1 << 22;
+constexpr int kConvPolls = 1 << 22;  // limit of a wait for products
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -428,6 +448,24 @@ __device__ __forceinline__ void mma_bf16(uint32_t tmem, uint64_t a, uint64_t b, 
       "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
       " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem),
       "l"(a), "l"(b), "r"(id), "r"(acc));
+}
+
+// Every thread's wait for the CTA's products: false, for the whole warp, once `polls` polls have gone
+// by.  The products are then waited for all the same before the CTA gives up what they read and write.
+__device__ __forceinline__ bool conv_wait(uint32_t bar, int polls, volatile int* fail) {
+  auto done = [=] {
+    uint32_t r;
+    asm volatile(
+        "{\n .reg .pred P1;\n mbarrier.try_wait.parity.shared::cta.b64 P1, [%1], %2;\n"
+        " selp.b32 %0, 1, 0, P1;\n}\n"
+        : "=r"(r)
+        : "r"(bar), "r"(0)
+        : "memory");
+    return r != 0;
+  };
+  const bool ok = __all_sync(0xffffffffu, wait_flight(done, [] {}, fail, polls));
+  if (!ok) wait_flight(done, [] {}, fail, kConvPolls);
+  return ok;
 }
 
 __device__ __forceinline__ void cp16(uint32_t dst, const void* src, bool ok) {
@@ -450,6 +488,7 @@ struct TcConvArgs {
   const double* sumsq;   // IN_PLANAR / OUT_FIELD: sum |t|^2
   float out_scale;
   int* err;              // set if the MMA completion wait timed out
+  int polls;             // that wait's limit
 };
 
 template <int IN, int OUT>
@@ -608,24 +647,9 @@ __global__ void __launch_bounds__(conv_threads<IN>()) conv_tc_kernel(TcConvArgs 
                  : "memory");
   }
   __syncthreads();
-  bool ok = false;
-  for (int it = 0; it < kConvPolls; ++it) {
-    uint32_t r;
-    asm volatile(
-        "{\n .reg .pred P1;\n mbarrier.try_wait.parity.shared::cta.b64 P1, [%1], %2;\n"
-        " selp.b32 %0, 1, 0, P1;\n}\n"
-        : "=r"(r)
-        : "r"(smem_u32(bar)), "r"(0)
-        : "memory");
-    if (r) {
-      ok = true;
-      break;
-    }
-  }
+  const bool ok = conv_wait(smem_u32(bar), a.polls, fail);
   asm volatile("tcgen05.fence::after_thread_sync;");
-  if (!ok) {
-    *fail = 1;
-  } else {
+  if (ok) {
     float bias[4];  // of the lane's channels: 4 (lane & 3) .. + 3, or 0 and 1
 #pragma unroll
     for (int c = 0; c < 4; ++c) bias[c] = (a.bias && (OUT == OUT_HIDDEN || c < 2)) ? a.bias[(OUT == OUT_HIDDEN ? 4 * (lane & 3) : 0) + c] : 0.f;
@@ -810,24 +834,9 @@ __global__ void __launch_bounds__(128) conv_brick_kernel(TcConvArgs a) {
                  : "memory");
   }
   __syncthreads();
-  bool ok = false;
-  for (int it = 0; it < kConvPolls; ++it) {
-    uint32_t r;
-    asm volatile(
-        "{\n .reg .pred P1;\n mbarrier.try_wait.parity.shared::cta.b64 P1, [%1], %2;\n"
-        " selp.b32 %0, 1, 0, P1;\n}\n"
-        : "=r"(r)
-        : "r"(smem_u32(bar)), "r"(0)
-        : "memory");
-    if (r) {
-      ok = true;
-      break;
-    }
-  }
+  const bool ok = conv_wait(smem_u32(bar), a.polls, fail);
   asm volatile("tcgen05.fence::after_thread_sync;");
-  if (!ok) {
-    *fail = 1;
-  } else {
+  if (ok) {
     float bias[16];
 #pragma unroll
     for (int c = 0; c < 16; ++c) bias[c] = (OUT == OUT_HIDDEN || c < 2) ? a.bias[c] : 0.f;
@@ -1041,6 +1050,7 @@ int cnn_apply_field(const CnnNet& net, int nz, int ny, int nx, const float* t, c
   a.sumsq = sumsq;
   a.out_scale = out_scale;
   a.err = err;
+  a.polls = kConvPolls;
   const unsigned grid = (unsigned)((int64_t)a.bx * a.by * a.bz);
   const size_t sm = a.run ? TC_SMEM : BRICK_SMEM;
   const uint16_t* in[4] = {nullptr, act0, act1, act0};
@@ -1081,7 +1091,9 @@ struct helm6_cnn_trainer {
   float* partial = nullptr;
   double *lpart = nullptr, *loss = nullptr;
   double* pinned = nullptr;
-  int* tcerr = nullptr;     // set by a tensor-core layer whose MMA wait timed out
+  int* tcerr = nullptr;     // [0] set by a tensor-core layer of the running call whose MMA wait timed out,
+                            // [1] by an Adam step not taken for that, until a call reports it
+  int polls = kConvPolls;   // limit of the layers' waits
   int nblk = 0, nloss = 0;
   long long step = 0;
   bool residual = false;    // loss mean|A_h y - x|^2 over interior points (else MSE)
@@ -1100,6 +1112,7 @@ TcConvArgs tr_tc_args(const helm6_cnn_trainer* tr) {
   a.nx = tr->nx;
   conv_tiling(a);
   a.err = tr->tcerr;
+  a.polls = tr->polls;
   return a;
 }
 
@@ -1112,6 +1125,7 @@ int tr_forward(helm6_cnn_trainer* tr, const float* x) {
   cudaStream_t s = tr->stream;
   TcConvArgs a = tr_tc_args(tr);
   const unsigned grid = tr_tc_grid(a);
+  if (cudaMemsetAsync(tr->tcerr, 0, sizeof(int), s) != cudaSuccess) return HELM6_ERR_CUDA;
   note_launch(NL);
   for (int l = 0; l < NL; ++l) {
     a.w = tr->net.wtc + (size_t)l * 27 * 256;
@@ -1196,16 +1210,39 @@ int tr_backward(helm6_cnn_trainer* tr, const float* x, const float* target) {
   return HELM6_OK;
 }
 
-int read_loss(helm6_cnn_trainer* tr, double* loss) {
-  if (!loss) return HELM6_OK;
-  if (cudaMemcpyAsync(tr->pinned, tr->loss, sizeof(double), cudaMemcpyDeviceToHost, tr->stream) != cudaSuccess)
+// Synchronises and reads the flags and the loss: HELM6_ERR_CUDA where a wait of this call timed out, or where an
+// earlier step was not taken for that (reported once).
+int sync_status(helm6_cnn_trainer* tr, double* loss) {
+  cudaStream_t s = tr->stream;
+  int flag[2];
+  if (loss && cudaMemcpyAsync(tr->pinned, tr->loss, sizeof(double), cudaMemcpyDeviceToHost, s) != cudaSuccess)
     return HELM6_ERR_CUDA;
-  if (cudaStreamSynchronize(tr->stream) != cudaSuccess) return HELM6_ERR_CUDA;
-  *loss = tr->pinned[0] / tr->loss_div;
+  if (cudaMemcpyAsync(tr->pinned + 1, tr->tcerr, sizeof(flag), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+      cudaStreamSynchronize(s) != cudaSuccess)
+    return HELM6_ERR_CUDA;
+  std::memcpy(flag, tr->pinned + 1, sizeof(flag));
+  if (flag[0] || flag[1]) {
+    cudaMemsetAsync(tr->tcerr, 0, 2 * sizeof(int), s);
+    return HELM6_ERR_CUDA;
+  }
+  if (loss) *loss = tr->pinned[0] / tr->loss_div;
   return HELM6_OK;
 }
 
+int read_loss(helm6_cnn_trainer* tr, double* loss) { return loss ? sync_status(tr, loss) : (int)HELM6_OK; }
+
+// A call's result to the caller's array.
+int copy_result(helm6_cnn_trainer* tr, const float* src, float* dst, int64_t n) {
+  note_launch();
+  result_copy_kernel<<<(unsigned)((n + 1023) / 1024), 256, 0, tr->stream>>>(src, dst, n, tr->tcerr);
+  return cudaGetLastError() == cudaSuccess ? HELM6_OK : HELM6_ERR_CUDA;
+}
+
 }  // namespace
+
+namespace helm6 {
+void cnn_wait_limit(helm6_cnn_trainer* tr, int polls) { tr->polls = polls; }
+}  // namespace helm6
 
 extern "C" {
 
@@ -1246,7 +1283,8 @@ int helm6_cnn_trainer_create(helm6_cnn_trainer** out, int batch, int nz, int ny,
   const size_t np = HELM6_CNN_NPARAMS;
   if (cnn_configure() != HELM6_OK) return fail(HELM6_ERR_CUDA);
   if (cnn_alloc(tr->net, true) != HELM6_OK) return fail(HELM6_ERR_NOMEM);
-  if (cudaMalloc((void**)&tr->tcerr, sizeof(int)) != cudaSuccess || cudaMemset(tr->tcerr, 0, sizeof(int)) != cudaSuccess)
+  if (cudaMalloc((void**)&tr->tcerr, 2 * sizeof(int)) != cudaSuccess ||
+      cudaMemset(tr->tcerr, 0, 2 * sizeof(int)) != cudaSuccess)
     return fail(HELM6_ERR_NOMEM);
   bool ok = al((void**)&tr->m, np * 4) && al((void**)&tr->v, np * 4) && al((void**)&tr->grad, np * 4) &&
             al((void**)&tr->y, npts * 8) && al((void**)&tr->g4, npts * 8) && al((void**)&tr->ga, npts * 64) &&
@@ -1269,9 +1307,7 @@ int helm6_cnn_forward(helm6_cnn_trainer* tr, const float* x, float* y) {
   if (!tr || !x || !y) return HELM6_ERR_INVALID;
   int rc = tr_forward(tr, x);
   if (rc) return rc;
-  if (cudaMemcpyAsync(y, tr->y, tr->npts * 8, cudaMemcpyDeviceToDevice, tr->stream) != cudaSuccess)
-    return HELM6_ERR_CUDA;
-  return HELM6_OK;
+  return copy_result(tr, tr->y, y, tr->npts * 2);
 }
 
 int helm6_cnn_gradient(helm6_cnn_trainer* tr, const float* x, const float* target, float* grad, double* loss) {
@@ -1279,9 +1315,7 @@ int helm6_cnn_gradient(helm6_cnn_trainer* tr, const float* x, const float* targe
   int rc = tr_forward(tr, x);
   if (!rc) rc = tr_backward(tr, x, target);
   if (rc) return rc;
-  if (cudaMemcpyAsync(grad, tr->grad, sizeof(float) * HELM6_CNN_NPARAMS, cudaMemcpyDeviceToDevice, tr->stream) !=
-      cudaSuccess)
-    return HELM6_ERR_CUDA;
+  if ((rc = copy_result(tr, tr->grad, grad, HELM6_CNN_NPARAMS))) return rc;
   return read_loss(tr, loss);
 }
 
@@ -1295,7 +1329,7 @@ int helm6_cnn_train_step(helm6_cnn_trainer* tr, const float* x, const float* tar
   const float c2 = (float)(1.0 - std::pow(0.999, (double)tr->step));
   note_launch();
   adam_kernel<<<(HELM6_CNN_NPARAMS + 255) / 256, 256, 0, tr->stream>>>(tr->net.theta, tr->m, tr->v, tr->grad,
-                                                                     HELM6_CNN_NPARAMS, lr, c1, c2);
+                                                                     HELM6_CNN_NPARAMS, lr, c1, c2, tr->tcerr);
   cnn_prepare(tr->net, tr->stream);
   if (cudaGetLastError() != cudaSuccess) return HELM6_ERR_CUDA;
   return read_loss(tr, loss);
@@ -1321,10 +1355,9 @@ int helm6_cnn_set_residual_loss(helm6_cnn_trainer* tr, helm6_c64 k, double h) {
 int helm6_cnn_get_params(helm6_cnn_trainer* tr, float* theta) {
   if (!tr || !theta) return HELM6_ERR_INVALID;
   if (cudaMemcpyAsync(theta, tr->net.theta, sizeof(float) * HELM6_CNN_NPARAMS, cudaMemcpyDeviceToHost,
-                      tr->stream) != cudaSuccess ||
-      cudaStreamSynchronize(tr->stream) != cudaSuccess)
+                      tr->stream) != cudaSuccess)
     return HELM6_ERR_CUDA;
-  return HELM6_OK;
+  return sync_status(tr, nullptr);
 }
 
 }  // extern "C"

@@ -302,6 +302,10 @@ int cnn_configure();  // kernel attributes of the field path (before any capture
 int cnn_apply_field(const CnnNet& net, int nz, int ny, int nx, const float* t, const double* sumsq,
                     uint16_t* act0, uint16_t* act1, float out_scale, float* z, int* err, cudaStream_t s);
 
+// Limit, in polls, of a trainer's waits for its layers' products (failure detection: 0 lets each run out
+// at once; the products are still waited for before their memory is given up).
+void cnn_wait_limit(::helm6_cnn_trainer* tr, int polls);
+
 int device_sm_count();
 
 // Device-driven solve (one CUDA graph per solve, convergence decided on the device through
