@@ -1448,7 +1448,7 @@ int helm6_create(helm6_ctx** out, int n, double h, helm6_c64 k, const int faces[
     fp.d.gidx = gi;
     c->fft[a] = fp.d;
     c->xform[a] = HELM6_XFORM_FFT;
-    fft_configure();
+    if (fft_configure() != HELM6_OK) return fail(HELM6_ERR_CUDA);
   }
 
   // workspace

@@ -30,6 +30,7 @@
 #include <vector>
 
 #include "helm6_internal.h"
+#include "per_device.h"
 #include "waits.h"
 
 namespace helm6 {
@@ -960,13 +961,13 @@ template <int CIN, int COUT, int IN>
 cudaError_t launch_wgrad(const ConvArgs& a, const float* g, float* partial, float* grad_w, float* grad_b,
                          cudaStream_t s) {
   constexpr size_t sm = WgTile<CIN, COUT>::smem;
-  static bool configured = false;
-  if (!configured) {
-    cudaError_t e =
-        cudaFuncSetAttribute(wgrad_kernel<CIN, COUT, IN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (e != cudaSuccess) return e;
-    configured = true;
-  }
+  static OncePerDevice once;
+  cudaError_t e = cudaSuccess;
+  if (!once(current_device(), [&] {
+        e = cudaFuncSetAttribute(wgrad_kernel<CIN, COUT, IN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        return e == cudaSuccess;
+      }))
+    return e;
   const int64_t tiles = (int64_t)a.tx * a.ty * a.tz * a.nb;
   const int nblk = wgrad_blocks<CIN, COUT>(a);
   note_launch(2);
@@ -1010,10 +1011,9 @@ void cnn_free(CnnNet& net) {
 }
 
 int cnn_configure() {
-  // the field kernels' shared-memory limits, set once before any launch (and so never
+  // the field kernels' shared-memory limits, set once per device before any launch (and so never
   // inside a stream capture)
-  static bool done = false;
-  if (done) return HELM6_OK;
+  static OncePerDevice once;
   const std::pair<const void*, size_t> ks[] = {
       {(const void*)conv_tc_kernel<IN_PLANAR, OUT_HIDDEN>, TC_SMEM},
       {(const void*)conv_tc_kernel<IN_BF16, OUT_HIDDEN>, TC_SMEM},
@@ -1025,11 +1025,13 @@ int cnn_configure() {
       {(const void*)conv_tc_kernel<IN_F32, OUT_HIDDEN>, TC_SMEM},
       {(const void*)conv_tc_kernel<IN_BF16, OUT_F32>, TC_SMEM},
       {(const void*)conv_tc_kernel<IN_G32, OUT_GRAD>, TC_SMEM4}};
-  for (const auto& k : ks)
-    if (cudaFuncSetAttribute(k.first, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)k.second) != cudaSuccess)
-      return HELM6_ERR_CUDA;
-  done = true;
-  return HELM6_OK;
+  const bool ok = once(current_device(), [&] {
+    for (const auto& k : ks)
+      if (cudaFuncSetAttribute(k.first, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)k.second) != cudaSuccess)
+        return false;
+    return true;
+  });
+  return ok ? HELM6_OK : HELM6_ERR_CUDA;
 }
 
 void cnn_prepare(const CnnNet& net, cudaStream_t s) {

@@ -33,6 +33,7 @@
 // precomputed spectrum of the kernel w_Q^{g^-q}.  Everything between the load and the store
 // runs in shared memory; the DRAM traffic is one read and one write of each line.
 #include "helm6_internal.h"
+#include "per_device.h"
 
 #include <cmath>
 #include <cstring>
@@ -543,14 +544,18 @@ int fft_lines_per_cta(const FftDev& f, int elem_bytes) {
 
 size_t fft_smem_bytes(const FftDev& f, int B, int elem_bytes) { return smem_of(f, B, elem_bytes); }
 
-void fft_configure() {
-  static bool done = false;
-  if (done) return;
-  cudaFuncSetAttribute(fft_axis_kernel<double, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFftSmemMax);
-  cudaFuncSetAttribute(fft_axis_kernel<double, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFftSmemMax);
-  cudaFuncSetAttribute(fft_axis_kernel<float, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFftSmemMax);
-  cudaFuncSetAttribute(fft_axis_kernel<float, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFftSmemMax);
-  done = true;
+int fft_configure() {
+  static OncePerDevice once;
+  auto set = [](auto* k) {
+    return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFftSmemMax) == cudaSuccess;
+  };
+  return once(current_device(),
+              [&] {
+                return set(fft_axis_kernel<double, true>) && set(fft_axis_kernel<double, false>) &&
+                       set(fft_axis_kernel<float, true>) && set(fft_axis_kernel<float, false>);
+              })
+             ? HELM6_OK
+             : HELM6_ERR_CUDA;
 }
 
 // axis 0: lines along x (contiguous), one per (z, y); axis 1: lines along y, one per (z, x).

@@ -198,7 +198,7 @@ struct FftHostPlan {
 // factorisation of the form above or a line does not fit in shared memory.  tables = false:
 // the sizes only.
 bool fft_make_plan(int n, int lo, int hi, bool half, FftHostPlan& plan, bool tables = true);
-void fft_configure();  // once per process: the kernels' dynamic shared memory limit
+int fft_configure();  // once per device: the kernels' dynamic shared memory limit
 // out = W in (inv = 0, forward) or V in (inv = 1) along axis 0 (x) or 1 (y) of the planar
 // field (same layout in and out; out may not alias in).
 template <typename T>
@@ -307,6 +307,7 @@ int cnn_apply_field(const CnnNet& net, int nz, int ny, int nx, const float* t, c
 void cnn_wait_limit(::helm6_cnn_trainer* tr, int polls);
 
 int device_sm_count();
+int current_device();  // -1 where it cannot be told
 
 // Device-driven solve (one CUDA graph per solve, convergence decided on the device through
 // conditional nodes): parameters written by the host before the launch, state kept by the

@@ -51,6 +51,7 @@
 #include <cstring>
 
 #include "helm6_internal.h"
+#include "per_device.h"
 #include "waits.h"
 
 namespace helm6 {
@@ -877,16 +878,17 @@ void launch_x64_digits(int n, int lo, int hi, int inverse, X64Basis& h, const do
 }
 
 int x64_configure() {
-  static int done = 0;
-  if (done) return HELM6_OK;
+  static OncePerDevice once;
   auto set = [](auto* k) {
-    return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, X_SMEM) != cudaSuccess;
+    return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, X_SMEM) == cudaSuccess;
   };
-  if (set(xform64_kernel<16, true>) || set(xform64_kernel<16, false>) || set(xform64_kernel<8, true>) ||
-      set(xform64_kernel<8, false>))
-    return HELM6_ERR_CUDA;
-  done = 1;
-  return HELM6_OK;
+  return once(current_device(),
+              [&] {
+                return set(xform64_kernel<16, true>) && set(xform64_kernel<16, false>) && set(xform64_kernel<8, true>) &&
+                       set(xform64_kernel<8, false>);
+              })
+             ? HELM6_OK
+             : HELM6_ERR_CUDA;
 }
 
 void launch_xform64(const X64Basis& b, const double* in, double* out, int M_total, int transposed, int R, int* err,

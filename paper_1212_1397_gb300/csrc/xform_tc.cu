@@ -49,6 +49,7 @@
 #include <cstring>
 
 #include "helm6_internal.h"
+#include "per_device.h"
 #include "waits.h"
 
 namespace helm6 {
@@ -706,11 +707,9 @@ void launch_vec(const TcArgs& a, unsigned grid, cudaStream_t s) {
 }  // namespace
 
 int tc_configure() {
-  static int done = 0;
-  if (done) return HELM6_OK;
-  if (set_smem<16>() || set_smem<8>() || set_smem<4>()) return HELM6_ERR_CUDA;
-  done = 1;
-  return HELM6_OK;
+  static OncePerDevice once;
+  return once(current_device(), [] { return !(set_smem<16>() || set_smem<8>() || set_smem<4>()); }) ? HELM6_OK
+                                                                                                   : HELM6_ERR_CUDA;
 }
 
 void launch_xform_tc(const float* in, float* out, const uint8_t* W, int M_total, int K, int P, int terms,
