@@ -505,8 +505,11 @@ __device__ __forceinline__ float cut32(double x) {
 // form sum_i V_i s_i, the correction of a vector that is orthogonal to the basis up to rounding
 // already: |s_i| is around 2^-52 of the vector.  Where every |s_i| is below 2^-36 of it (else
 // the general form runs), that sum is formed in FP32 from the vectors' leading 24 bits, cut by
-// integer operations: each term's error is below 2^-23 2^-36 of the vector, well under the
-// rounding of the subtraction that follows (2^-53).  192^3 FP64 GMRES: 908 -> 667 us.
+// integer operations, and taken from u once: a term's error is below 2^-23 2^-36 of the vector,
+// where the general form rounds u itself (2^-53) with every term.  FP32's exponents reach all that
+// counts for alpha from 2^-64 to 2^64 (other alpha, and a breakdown: the general form).  Error of v
+// against extended precision, in 2^-53 |u|, largest of 4096 points: 1.6 with 30 and with 64 vectors, the
+// general form 12 and 20.  192^3 FP64 GMRES: 908 -> 667 us.
 template <typename T, int PTS, typename TV, int UB = 8>
 __global__ void __launch_bounds__(RB) dcgs_update_kernel(const TV* __restrict__ V, int64_t vs, int count,
                                                          T* u, const T* __restrict__ w, TV* __restrict__ v_out,
@@ -528,8 +531,8 @@ __global__ void __launch_bounds__(RB) dcgs_update_kernel(const TV* __restrict__ 
   bool low = false;  // the correction of u is small enough for FP32
   __shared__ float s32[sizeof(T) == 8 ? 64 : 1][2];
   if constexpr (sizeof(T) == 8) {
-    const double alpha = 1.0 / coef[4 * count + 2];  // (a breakdown's 0: inf or NaN, either form will do)
-    bool ok = true;
+    const double alpha = 1.0 / coef[4 * count + 2];
+    bool ok = alpha >= 5.421010862427522e-20 && alpha <= 18446744073709551616.0;  // 2^-64 .. 2^64
     for (int c = threadIdx.x; c < count; c += blockDim.x) {
       ok = ok && fabs(s_r[c]) + fabs(s_i[c]) < 1.4551915228366852e-11 * alpha;  // 2^-36
       s32[c][0] = (float)s_r[c];
