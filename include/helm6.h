@@ -78,11 +78,15 @@ enum { HELM6_BASIS_AUTO = 0, /* the default below */
    post-processing) or 4(n+1) (D-N, N-D: the line's odd or even extension); it exists when
    n + 1 = 2^a * Q with Q = 1 or a prime with Q - 1 a power of two (Q <= 257): n + 1 a power
    of two, or 257, 17, 5, 3 times a power of two. */
-enum { HELM6_XFORM_AUTO = 0,   /* FP64: FFT on every axis that has one, else dense; from 8,192
-                                  unknowns on, while the axes' products stay exact (up to 320
-                                  points of a folded axis), the same basis applied on the
-                                  tensor cores in exact integer slices (errors at or below the
-                                  FFT's; helm6_transform reports the form it stands for).
+enum { HELM6_XFORM_AUTO = 0,   /* FP64: FFT on every axis that has one, else dense.  From 8,192
+                                  unknowns on the same bases are applied on the tensor cores
+                                  in integer slices, where both axes' sums stay exact (checked
+                                  at creation: for n up to about 460 with alike faces on an
+                                  axis, 248 with unlike ones; never from 569 and 279; single
+                                  lengths in between).  An error is then relative to the
+                                  largest value of the row (line) being transformed, as with
+                                  the FFT: values below 2^-54 of it count as zero.
+                                  helm6_transform reports the form that this one stands for.
                                   MIXED: dense on tensor cores while both axes fit them
                                   (<= 264 unknowns), else FFT where it exists, else dense FP32 */
        HELM6_XFORM_DENSE = 1,  /* the dense m x m basis matrices (tensor cores where MIXED and

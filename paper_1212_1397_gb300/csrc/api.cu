@@ -1367,28 +1367,39 @@ int helm6_create(helm6_ctx** out, int n, double h, helm6_c64 k, const int faces[
   // against 17 us per transform; n = 20, dense: 40 against 16).
   if (o.precision == HELM6_FP64 && o.transform == HELM6_XFORM_AUTO && c->g.N >= 8192) {
     X64Basis* X[4] = {&c->Wx6, &c->Vx6, &c->Wy6, &c->Vy6};
-    double* trig = nullptr;  // the two axes' tables
-    int* over = nullptr;
-    std::vector<double> tx, ty;
-    x64_trig(n, c->g.face[0], c->g.face[1], tx);
-    x64_trig(n, c->g.face[2], c->g.face[3], ty);
-    const size_t nx = tx.size();
-    tx.insert(tx.end(), ty.begin(), ty.end());
-    if (x64_configure() != HELM6_OK) return fail(HELM6_ERR_CUDA);
-    if ((rc = dalloc(c, &trig, tx.size())) || (rc = dalloc(c, &over, 1))) return fail(rc);
-    if (cudaMemcpy(trig, tx.data(), tx.size() * sizeof(double), cudaMemcpyHostToDevice) != cudaSuccess ||
-        cudaMemset(over, 0, sizeof(int)) != cudaSuccess)
-      return fail(HELM6_ERR_CUDA);
+    const size_t held = c->allocs.size();
+    bool fits = true;
     for (int a = 0; a < 4; ++a) {
-      const int lo = c->g.face[2 * (a / 2)], hi = c->g.face[2 * (a / 2) + 1];
-      *X[a] = x64_plan(n, lo, hi);
-      if (X[a]->nk * 16 > 320) break;  // far beyond what an accumulator holds
-      if ((rc = dalloc(c, &X[a]->dev, X[a]->bytes))) return fail(rc);
-      launch_x64_digits(n, lo, hi, a % 2, *X[a], a < 2 ? trig : trig + nx, over, 0);
+      *X[a] = x64_plan(n, c->g.face[2 * (a / 2)], c->g.face[2 * (a / 2) + 1]);
+      fits = fits && x64_may_fit(*X[a]);
     }
-    int out_of_range = 0;
-    if (cudaMemcpy(&out_of_range, over, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess) return fail(HELM6_ERR_CUDA);
-    c->x64 = !out_of_range && c->Vy6.dev;
+    if (fits) {
+      double* trig = nullptr;  // the two axes' tables
+      int* over = nullptr;
+      std::vector<double> tx, ty;
+      x64_trig(n, c->g.face[0], c->g.face[1], tx);
+      x64_trig(n, c->g.face[2], c->g.face[3], ty);
+      const size_t nx = tx.size();
+      tx.insert(tx.end(), ty.begin(), ty.end());
+      if (x64_configure() != HELM6_OK) return fail(HELM6_ERR_CUDA);
+      if ((rc = dalloc(c, &trig, tx.size())) || (rc = dalloc(c, &over, 1))) return fail(rc);
+      if (cudaMemcpy(trig, tx.data(), tx.size() * sizeof(double), cudaMemcpyHostToDevice) != cudaSuccess ||
+          cudaMemset(over, 0, sizeof(int)) != cudaSuccess)
+        return fail(HELM6_ERR_CUDA);
+      for (int a = 0; a < 4; ++a) {
+        if ((rc = dalloc(c, &X[a]->dev, X[a]->bytes))) return fail(rc);
+        launch_x64_digits(n, c->g.face[2 * (a / 2)], c->g.face[2 * (a / 2) + 1], a % 2, *X[a], a < 2 ? trig : trig + nx,
+                          over, 0);
+      }
+      int out_of_range = 0;
+      if (cudaMemcpy(&out_of_range, over, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess) return fail(HELM6_ERR_CUDA);
+      c->x64 = !out_of_range;
+    }
+    if (!c->x64) {  // an axis out of range: the context takes the other forms, and keeps nothing of this one
+      for (size_t i = held; i < c->allocs.size(); ++i) cudaFree(c->allocs[i]);
+      c->allocs.resize(held);
+      for (X64Basis* b : X) *b = X64Basis{};
+    }
   }
   // the dense matrices: what the tensor-core tiles of a MIXED context are made from, and device
   // copies in the working precision where a SIMT dense form may read them

@@ -139,6 +139,7 @@ struct X64Basis {
   int m = 0, fold = 0, nk = 0, nch = 0, gcols = 0, ngroups = 0, eb = 0, tail = 0;
 };
 X64Basis x64_plan(int n, int lo, int hi);
+bool x64_may_fit(const X64Basis& h);  // false: out of the kernel's range whatever the digits
 void x64_trig(int n, int lo, int hi, std::vector<double>& trig);
 void launch_x64_digits(int n, int lo, int hi, int inverse, X64Basis& h, const double* trig, int* over, cudaStream_t s);
 int x64_configure();

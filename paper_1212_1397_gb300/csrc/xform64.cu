@@ -832,6 +832,11 @@ X64Basis x64_plan(int n, int lo, int hi) {
   return h;
 }
 
+// Products of more points than this never pass the digits' check (which fails for single lengths from 250
+// points of a quarter-wave axis on, from 232 point pairs of a cosine and 275 of a sine axis; the last lengths to
+// pass have 279 points, 282 and 284 pairs).
+bool x64_may_fit(const X64Basis& h) { return (h.fold ? (h.m + 1) / 2 : h.m) <= 288; }
+
 // The trigonometric table of an axis: sin or cos of pi t / D, t < 2 D, from the first octant.
 void x64_trig(int n, int lo, int hi, std::vector<double>& trig) {
   const bool nlo = lo != HELM6_DIRICHLET, nhi = hi != HELM6_DIRICHLET;
