@@ -93,7 +93,7 @@ constexpr int kMaxPolls = 1 << 22;
 struct TcArgs {
   const float* in;
   float* out;
-  const uint8_t* W;   // per column group: [kt][half][term][kc][npad_g / 2 columns][16 B]
+  const uint8_t* W;   // per column group: [kt][term][kc][npad_g columns][16 B]
   const float* Bt;    // tail basis rows (FP32, tail x K) or null
   int M_total, K, P, nk, terms, transposed, R;
   int ldin;  // input row pitch (floats, >= K)
